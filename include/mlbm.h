@@ -334,7 +334,7 @@ mlbm_status mlbm_run_to_steady_mean(mlbm_ctx* ctx, double threshold, int64_t dn,
                                     int64_t max_steps, int64_t* steps_taken);
 
 /*
- * Bounded device waits.  The bulk-copy ring step variants (4..7) wait on
+ * Bounded device waits.  The bulk-copy step variants (4..7, 27..29) wait on
  * shared-memory barriers for their tile copies; each wait gives up after
  * `seconds` (default 2; accepted range [1e-4, 60]), records an error word,
  * waits (bounded again) for the copies it issued and returns, and the next
@@ -345,7 +345,7 @@ mlbm_status mlbm_run_to_steady_mean(mlbm_ctx* ctx, double threshold, int64_t dn,
 mlbm_status mlbm_set_wait_limit(mlbm_ctx* ctx, double seconds);
 /*
  * Test of the bounded waits: the next step launch (which must use a
- * bulk-copy ring variant, 4..7, else MLBM_E_INVALID) issues no copies for
+ * bulk-copy variant, 4..7 or 27..29, else MLBM_E_INVALID) issues no copies for
  * the first tile of its first block, so that block's consumers wait for a
  * tile that never arrives until the wait limit runs out.  One launch only;
  * it is launched directly, never from a captured graph.  No paper counterpart.
@@ -419,14 +419,15 @@ double mlbm_last_step_ms(const mlbm_ctx* ctx);
  *        on the SM slots it frees, and the next grid prefetches its first
  *        stencil rows into L2 before it waits for the previous grid's writes
  *        (BGK and tau = 1; RBF-FD stencils run the plain capped kernel)
- *   27-29 persistent CTAs of one lane per node (the node code of 11) whose
- *        matrix, index and meta rows come from a shared-memory ring that a
- *        producer warp fills with bulk async copies, as 4-7: 27 = 128-node
- *        tiles, 2 stages, 2 CTAs/SM; 28 = 64-node tiles, 2 stages, 3 CTAs/SM;
- *        29 = 64-node tiles, 3 stages, 2 CTAs/SM (BGK and tau = 1; RBF-FD
- *        stencils run the plain capped kernel)
+ *   27-29 persistent blocks of independent warps, one lane per node: each
+ *        warp copies the stencil rows of its own 32-node tiles into a
+ *        shared-memory slot of its own, one tile ahead, with bulk async
+ *        copies; a warp with interpolated bounce-back links evaluates them in
+ *        the same pass: 27 = 12 warps per SM (K = 24: 10, K = 32: 8), 28 = 8
+ *        (K = 32: 6), 29 = 14 (K = 24: 11, K = 32: 7) (BGK and tau = 1;
+ *        RBF-FD stencils run the plain capped kernel)
  * Variants 4 and up are available for K = 12, 16, 24 and 32.
- * The default is 25 when available, else 1.  mlbm_autotune times every
+ * The default is 27 when available, else 1.  mlbm_autotune times every
  * available variant for steps_per_variant steps on the context's stream
  * (state saved and restored, step count unchanged), keeps the fastest and
  * returns its per-step time in *best_ms (may be NULL).

@@ -33,8 +33,10 @@ struct mlbm_ctx {
     cudaStream_t stream = nullptr;
     cudaStream_t own_stream = nullptr;
     // stencil data on the device
-    int4* idx = nullptr;
-    float4* M = nullptr;
+    float4* rec = nullptr;    // tile records (see dev::TileRec; least-squares stencils)
+    uint8_t* need = nullptr;  // what each tile fetches of its record
+    int* range = nullptr;     // tile ranges of the step's blocks
+    int4* idx = nullptr;      // RBF-FD stencils
     uint8_t* meta = nullptr;
     float* lag_r = nullptr;
     int* link_slot = nullptr;
@@ -62,7 +64,7 @@ struct mlbm_ctx {
     bool timing = false;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     double last_ms = -1.0;
-    int variant = 25;
+    int variant = 27;
     std::vector<int> inv_perm;  // caller's node id -> device position
     int* err = nullptr;  // device error word of the bounded waits
     dev::Stencil S{};
@@ -203,9 +205,9 @@ mlbm_status launch_one_step(mlbm_ctx* c, int variant) {
         if (variant <= 7)
             MLBM_CUDA(launch_step_tma(variant, model, c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->ruv[a],
                                       c->ruv[b], c->C, c->err, W, c->stream));
-        else
-            MLBM_CUDA(launch_step_ring1(variant, model, c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->ruv[a],
-                                        c->ruv[b], c->C, c->err, W, c->stream));
+        else  // every other step walks the tiles backwards
+            MLBM_CUDA(launch_step_warp(variant, model, c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->ruv[a],
+                                       c->ruv[b], c->C, a, c->err, W, c->stream));
     }
     else if (model == 0)
         MLBM_CUDA(launch_bgk_step(c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->C, variant, c->stream));
@@ -235,8 +237,9 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
     const int K = H.K, Kq = K / 4;
     // ---- host-side device layout
     const bool rbf = H.interp != MLBM_INTERP_WLS;  // per-direction RBF-FD weights
-    std::vector<int32_t> hidx((size_t)Kq * np * 4, 0);
-    std::vector<float> hM((size_t)6 * Kq * np * 4, 0.f);
+    const int rows = 7 * Kq - 1, sp = dev::special_group(Kq);
+    std::vector<int32_t> hrec(rbf ? 0 : (size_t)(np / 32) * rows * 128, 0);
+    std::vector<int32_t> hidx(rbf ? (size_t)Kq * np * 4 : 0, 0);
     std::vector<float> hW(rbf ? (size_t)8 * Kq * np * 4 : 0, 0.f);
     std::vector<uint8_t> hmeta(np, 0), hmask(np, 0);
     std::vector<float> hlag(np, 0.f), harea(np, 0.f), has2(np, 0.f);
@@ -262,6 +265,11 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         harea[q] = (float)H.area[q];
         const double sq = H.s_node.empty() ? H.s : H.s_node[q];
         has2[q] = (float)(H.area[q] / (sq * sq));
+        // sample of a batch's node, and the node's lane in its tile record
+        const int sample =
+            parts ? (int)(std::upper_bound(H.part_off.begin(), H.part_off.end(), q) - H.part_off.begin()) - 1 : 0;
+        int32_t* lane = rbf ? nullptr : hrec.data() + ((size_t)(q / 32) * rows * 32 + q % 32) * 4;
+        if (!rbf) lane[sp * 128 + 3] = (int32_t)hmeta[q] | (sample << 8);
         if (kind == kKindWls) {
             // stencil slots in increasing node position: lanes of a warp that
             // gather slot j of consecutive (Hilbert-ordered) nodes then touch
@@ -275,40 +283,52 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
                 std::sort(order, order + K, [&](int a, int b) {
                     return H.slot_key[(size_t)q * K + a] < H.slot_key[(size_t)q * K + b];
                 });
-            // the node's matrix (and RBF-FD weight) rows: its own, or its sample's
-            const double* Mq;
+            // the node's matrix or RBF-FD weight rows: its own, or its sample's
+            const double* Mq = nullptr;
             const double* Wq = nullptr;
             if (parts) {
-                const size_t i =
-                    (size_t)(std::upper_bound(H.part_off.begin(), H.part_off.end(), q) - H.part_off.begin()) - 1;
-                const size_t l = (size_t)(q - H.part_off[i]);
-                Mq = H.part_M[i] + l * 6 * K;
-                if (rbf) Wq = H.part_Wr[i] + l * 8 * K;
+                const size_t l = (size_t)(q - H.part_off[sample]);
+                if (rbf) Wq = H.part_Wr[sample] + l * 8 * K;
+                else Mq = H.part_M[sample] + l * 6 * K;
+            } else if (rbf) {
+                Wq = H.Wr.data() + (size_t)q * 8 * K;
             } else {
                 Mq = H.M.data() + (size_t)q * 6 * K;
-                if (rbf) Wq = H.Wr.data() + (size_t)q * 8 * K;
             }
-            for (int jj = 0; jj < K; ++jj) {
+            if (rbf)
+                for (int jj = 0; jj < K; ++jj) {
+                    const int j = order[jj];
+                    hidx[(((size_t)(jj / 4)) * np + q) * 4 + (jj % 4)] = H.idx[(size_t)q * K + j];
+                    for (int k = 0; k < 8; ++k)
+                        hW[(((size_t)(k * Kq + jj / 4)) * np + q) * 4 + (jj % 4)] = (float)Wq[(size_t)k * K + j];
+                }
+            int slot = 0;
+            for (int jj = 0; !rbf && jj < K; ++jj) {
                 const int j = order[jj];
-                hidx[(((size_t)(jj / 4)) * np + q) * 4 + (jj % 4)] = H.idx[(size_t)q * K + j];
+                const int32_t id = H.idx[(size_t)q * K + j];
+                if (id == q) continue;  // its weight multiplies a zero difference
+                if (slot == 4 * sp + 3) ++slot;
                 double m[6];
                 for (int a = 0; a < 6; ++a) m[a] = Mq[(size_t)a * K + j];
                 // D2Q9 departure basis (see device_common.cuh), formed in FP64
                 const double t[6] = {m[0] + m[3], m[0] + m[5], m[0] + m[3] + m[4] + m[5], m[0] + m[3] - m[4] + m[5],
                                      m[1], m[2]};
-                for (int a = 0; a < 6; ++a)
-                    hM[(((size_t)(a * Kq + jj / 4)) * np + q) * 4 + (jj % 4)] = (float)t[a];
-                if (rbf)
-                    for (int k = 0; k < 8; ++k)
-                        hW[(((size_t)(k * Kq + jj / 4)) * np + q) * 4 + (jj % 4)] =
-                            (float)Wq[(size_t)k * K + j];
+                const int g = slot / 4, cc = slot % 4, mr = Kq + 6 * g - (g > sp ? 1 : 0);
+                lane[g * 128 + cc] = id;
+                for (int a = 0; a < 6; ++a) {
+                    const float v = (float)t[a];
+                    std::memcpy(g == sp && a == 5 ? &lane[(mr + cc) * 128 + 3] : &lane[(mr + a) * 128 + cc], &v, 4);
+                }
+                ++slot;
             }
         } else if (kind == kKindLagrange) {
             for (int b = 0; b < 9; ++b) {
                 const int j = H.lag_slot[(size_t)q * 9 + b];
-                hidx[(((size_t)(b / 4)) * np + q) * 4 + (b % 4)] = H.idx[(size_t)q * K + j];
+                (rbf ? hidx[(((size_t)(b / 4)) * np + q) * 4 + (b % 4)] : lane[(b / 4) * 128 + (b % 4)]) =
+                    H.idx[(size_t)q * K + j];
             }
             hlag[q] = (float)(sq / H.lag_h[q]);
+            if (!rbf) std::memcpy(&lane[2 * 128 + 1], &hlag[q], 4);
         } else {
             heqv[q] = make_float4((float)(H.eqv[q * 3] - 1.0), (float)H.eqv[q * 3 + 1], (float)H.eqv[q * 3 + 2], 0.f);
         }
@@ -319,6 +339,9 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
             hlinks[(size_t)hslot[q]] = r;
         }
     }
+    // lanes past the last node read as equilibrium nodes, which gather nothing
+    for (int64_t q = n; !rbf && q < np; ++q)
+        hrec[((size_t)(q / 32) * rows * 32 + q % 32) * 4 + (size_t)sp * 128 + 3] = kKindEq;
     c->n_link_nodes = (int)hlinknodes.size();
     c->inv_perm.assign((size_t)n, -1);
     for (int64_t q = 0; q < n; ++q) c->inv_perm[(size_t)hperm[q]] = (int)q;
@@ -332,21 +355,27 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         const int64_t T = dev::kStageTile, nt = (n + T - 1) / T;
         std::vector<std::vector<int>> lists((size_t)nt);
         hlidx.assign((size_t)Kq * np * 4, 0);
+        auto member = [&](int64_t q, int jj) {
+            return hrec.data() + ((size_t)(q / 32) * rows * 32 + q % 32) * 4 + (size_t)(jj / 4) * 128 + jj % 4;
+        };
 #pragma omp parallel for schedule(dynamic, 8)
         for (int64_t b = 0; b < nt; ++b) {
             std::vector<int>& L = lists[(size_t)b];
             const int64_t q0 = b * T, q1 = std::min<int64_t>(n, q0 + T);
             for (int64_t q = q0; q < q1; ++q)
                 if ((hmeta[q] & 7) == 0)
-                    for (int jj = 0; jj < K; ++jj) L.push_back(hidx[(((size_t)(jj / 4)) * np + q) * 4 + (jj % 4)]);
+                    for (int jj = 0; jj < K; ++jj)
+                        if (jj != 4 * sp + 3) L.push_back(*member(q, jj));
             std::sort(L.begin(), L.end());
             L.erase(std::unique(L.begin(), L.end()), L.end());
             if ((int64_t)L.size() > dev::kStageMax) continue;  // too wide: the whole structure is dropped below
             for (int64_t q = q0; q < q1; ++q)
                 if ((hmeta[q] & 7) == 0)
                     for (int jj = 0; jj < K; ++jj) {
-                        const size_t at = (((size_t)(jj / 4)) * np + q) * 4 + (jj % 4);
-                        hlidx[at] = (uint16_t)(std::lower_bound(L.begin(), L.end(), hidx[at]) - L.begin());
+                        // the freed slot, whose weight is zero, repeats the first member
+                        const int id = *member(q, jj == 4 * sp + 3 ? 0 : jj);
+                        hlidx[(((size_t)(jj / 4)) * np + q) * 4 + (jj % 4)] =
+                            (uint16_t)(std::lower_bound(L.begin(), L.end(), id) - L.begin());
                     }
         }
         hsoff.assign((size_t)nt + 1, 0);
@@ -365,10 +394,16 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         }
     }
     // ---- device buffers
-    MLBM_TRY(dalloc(c, &c->idx, (size_t)Kq * np));
-    MLBM_TRY(dalloc(c, &c->M, (size_t)6 * Kq * np));
     float4* dW = nullptr;
-    if (rbf) MLBM_TRY(dalloc(c, &dW, (size_t)8 * Kq * np));
+    c->S.n_ranges = warp_step_ranges((int)n);
+    if (rbf) {
+        MLBM_TRY(dalloc(c, &c->idx, (size_t)Kq * np));
+        MLBM_TRY(dalloc(c, &dW, (size_t)8 * Kq * np));
+    } else {
+        MLBM_TRY(dalloc(c, &c->rec, hrec.size() / 4));
+        MLBM_TRY(dalloc(c, &c->need, (size_t)np / 32));
+        MLBM_TRY(dalloc(c, &c->range, (size_t)c->S.n_ranges + 1));
+    }
     MLBM_TRY(dalloc(c, &c->meta, np));
     MLBM_TRY(dalloc(c, &c->mask, np));
     MLBM_TRY(dalloc(c, &c->lag_r, np));
@@ -405,9 +440,12 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
     MLBM_TRY(dalloc(c, &c->err, 1));
     MLBM_CUDA(cudaMemsetAsync(c->err, 0, sizeof(int), c->stream));
     if (!tma_supported(Kq)) c->variant = 1;  // variants >= 4 exist for K in {12, 16, 24, 32}
-    MLBM_TRY(upload(c, c->idx, hidx.data(), hidx.size() * 4));
-    MLBM_TRY(upload(c, c->M, hM.data(), hM.size() * 4));
-    if (rbf) MLBM_TRY(upload(c, dW, hW.data(), hW.size() * 4));
+    if (rbf) {
+        MLBM_TRY(upload(c, c->idx, hidx.data(), hidx.size() * 4));
+        MLBM_TRY(upload(c, dW, hW.data(), hW.size() * 4));
+    } else {
+        MLBM_TRY(upload(c, c->rec, hrec.data(), hrec.size() * 4));
+    }
     MLBM_TRY(upload(c, c->meta, hmeta.data(), np));
     MLBM_TRY(upload(c, c->mask, hmask.data(), np));
     MLBM_TRY(upload(c, c->lag_r, hlag.data(), np * 4));
@@ -433,7 +471,10 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
     c->S.Kq = Kq;
     c->S.bb_mode = H.bb_mode;
     c->S.idx = c->idx;
-    c->S.M = c->M;
+    c->S.rec = c->rec;
+    c->S.need = c->need;
+    c->S.range = c->range;
+    c->S.rows = rows;
     c->S.meta = c->meta;
     c->S.lag_r = c->lag_r;
     c->S.link_slot = c->link_slot;
@@ -461,6 +502,7 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         c->S.stage_ids = dids;
         c->S.stage_max = stage_max;
     }
+    MLBM_CUDA(launch_record_kinds(c->S, c->rec, c->need, c->range, c->stream));
     set_collide(c);
     // ---- initial state
     std::vector<double> ru((size_t)n * 3);
@@ -695,8 +737,10 @@ mlbm_status run_steady(mlbm_ctx* c, int mode, double tol, int64_t window, int64_
                     --remaining;
                     if (saved_meta && remaining > 0) {
                         const int64_t o = c->seg_off[i];
-                        MLBM_CUDA(launch_freeze_tau1((int)(c->seg_off[i + 1] - o), c->meta + o, c->eqv + o,
-                                                     c->ruv[c->cur] + o, c->stream));
+                        MLBM_CUDA(launch_freeze_tau1((int)o, (int)(c->seg_off[i + 1] - o), c->meta, c->eqv,
+                                                     c->ruv[c->cur], c->stream));
+                        MLBM_CUDA(launch_record_kinds(c->S, c->rec, c->need, c->range, c->stream));
+                        MLBM_TRY(sync(c));
                         frozen_any = true;
                     }
                 }
@@ -709,12 +753,13 @@ mlbm_status run_steady(mlbm_ctx* c, int mode, double tol, int64_t window, int64_
         const size_t np = (size_t)c->n_pad;
         cudaMemcpyAsync(c->meta, saved_meta, np, cudaMemcpyDeviceToDevice, c->stream);
         cudaMemcpyAsync(c->eqv, saved_eqv, np * sizeof(float4), cudaMemcpyDeviceToDevice, c->stream);
+        launch_record_kinds(c->S, c->rec, c->need, c->range, c->stream);
     }
     if (saved_meta) cudaFreeAsync(saved_meta, c->stream);
     if (saved_eqv) cudaFreeAsync(saved_eqv, c->stream);
     if (ring) cudaFreeAsync(ring, c->stream);
     if (means) cudaFreeAsync(means, c->stream);
-    if (ring || means || saved_meta) cudaStreamSynchronize(c->stream);
+    if (ring || means || saved_meta) cudaStreamSynchronize(c->stream);  // also before the next step reads the kinds
     if (at)
         for (int i = 0; i < ns; ++i) at[i] = done_at[i];
     return st;

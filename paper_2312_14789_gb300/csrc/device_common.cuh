@@ -3,11 +3,12 @@
 // Node data live in Hilbert order ("positions" p = 0..n-1), padded to n_pad
 // (a multiple of 128) so every row of the interleaved arrays starts on a
 // 512-byte boundary:
-//   idx  int4   [K/4][n_pad]     neighbour positions, 4 per int4 (Lagrange
-//                                nodes: slots 0..8 hold the 3x3 block, row b
-//                                outer, column a inner)
-//   M    float4 [6*(K/4)][n_pad] least-squares matrix in units of s: row a,
-//                                neighbour group g at (a*K/4 + g)*n_pad + p
+//   rec  tile records (least-squares stencils, see TileRec): neighbour
+//                                positions and the least-squares matrix in
+//                                units of s, 32 nodes to a contiguous block
+//   idx  int4   [K/4][n_pad]     RBF-FD stencils: neighbour positions, 4 per
+//                                int4 (Lagrange nodes: slots 0..8 hold the 3x3
+//                                block, row b outer, column a inner)
 //   meta uint8  [n_pad]          bits 0-1 kind (0 WLS, 1 Lagrange, 2 equilibrium),
 //                                bit 2 has bounce-back links, bits 4-7 block centre
 //   lag_r float [n_pad]          s / h of the Lagrange block
@@ -38,8 +39,15 @@ struct Collide {
 struct Stencil {
     int n, n_pad, K, Kq;
     int bb_mode;
-    const int4* idx;
-    const float4* M;
+    // least-squares stencils: tile records (see TileRec) of `rows` rows, what
+    // each 32-node tile has to fetch of its record (0 the kind words, 1 the
+    // Lagrange indices, 2 everything), and the tiles' ranges [range[b],
+    // range[b + 1]) of about equal cost for n_ranges blocks
+    const float4* rec;
+    const uint8_t* need;
+    const int* range;
+    int rows, n_ranges;
+    const int4* idx;  // RBF-FD stencils
     const uint8_t* meta;
     const float* lag_r;
     const int* link_slot;
@@ -67,6 +75,36 @@ struct Stencil {
     int stage_max;
 };
 
+// Tile records: the stencil rows of 32 consecutive nodes in one contiguous
+// block of rows of 32 x 16 bytes (lane l of a row belongs to node 32 t + l).
+//   rows 0 .. KQ-1   neighbour positions, 4 per int4, the node itself left out
+//                    (its weight multiplies a difference that is zero); the
+//                    slot it frees, number 4 kSp + 3, holds the node's kind
+//                    byte (as meta) and, above it, its sample
+//   then per group of four neighbours the six matrix rows U, V, W, W', m1, m2;
+//   the group with the freed slot holds three neighbours and keeps its m2
+//   entries in the fourth components of its first three rows (five rows)
+// Lagrange nodes: slots 0..8 the block, slot 9 the bits of s / h.
+// A tile is one bulk copy (or one prefetch), rows are at constant offsets, and
+// a least-squares node of K = 16 costs 432 bytes where separate arrays with
+// the node's own column, kind and sample took 451.
+__host__ __device__ constexpr int special_group(int KQ) { return KQ - 1 < 2 ? KQ - 1 : 2; }
+template <int KQ>
+struct TileRec {
+    static constexpr int kSp = special_group(KQ);
+    static constexpr int kRows = 7 * KQ - 1;
+    __host__ __device__ static constexpr int m_row(int q) { return KQ + 6 * q - (q > kSp ? 1 : 0); }
+};
+
+// row 0 of node p's lane in its tile record (row r: + 32 r)
+__device__ __forceinline__ const float4* rec_lane(const Stencil& S, int p) {
+    return S.rec + ((size_t)(p >> 5) * S.rows) * 32 + (p & 31);
+}
+template <int KQ>
+__device__ __forceinline__ const float4* rec_lane(const Stencil& S, int p) {
+    return S.rec + ((size_t)(p >> 5) * TileRec<KQ>::kRows) * 32 + (p & 31);
+}
+
 // bounded waits of the bulk-copy ring kernels: time budget of one wait, and a
 // test switch that makes block 0 withhold its first tile's copies
 struct Wait {
@@ -91,6 +129,49 @@ __device__ __forceinline__ float w_of(int k) { return k == 0 ? (4.0f / 9.0f) : (
 // out of L1 and mark them first for eviction in L2.
 __device__ __forceinline__ float4 ld_stream(const float4* p) { return __ldcs(p); }
 __device__ __forceinline__ int4 ld_stream(const int4* p) { return __ldcs(p); }
+
+// Neighbour positions of group q (the freed slot reads as the node itself,
+// which adds nothing) and its six matrix rows, from a node's lane of a tile
+// record.  LD loads one row.
+template <int KQ, class LD>
+__device__ __forceinline__ int4 rec_ids(const float4* b, int q, int p, LD ld) {
+    const float4 v = ld(b + q * 32);
+    int4 id = make_int4(__float_as_int(v.x), __float_as_int(v.y), __float_as_int(v.z), __float_as_int(v.w));
+    if (q == TileRec<KQ>::kSp) id.w = p;
+    return id;
+}
+template <int KQ, class LD>
+__device__ __forceinline__ void rec_group(const float4* b, int q, float4* m, LD ld) {
+    const float4* r = b + TileRec<KQ>::m_row(q) * 32;
+#pragma unroll
+    for (int a = 0; a < 5; ++a) m[a] = ld(r + a * 32);
+    if (q == TileRec<KQ>::kSp) {
+        m[5] = make_float4(m[0].w, m[1].w, m[2].w, 0.f);
+#pragma unroll
+        for (int a = 0; a < 5; ++a) m[a].w = 0.f;
+    } else {
+        m[5] = ld(r + 5 * 32);
+    }
+}
+struct LdStream {
+    __device__ __forceinline__ float4 operator()(const float4* p) const { return __ldcs(p); }
+};
+struct LdCached {
+    __device__ __forceinline__ float4 operator()(const float4* p) const { return __ldg(p); }
+};
+struct LdPlain {
+    __device__ __forceinline__ float4 operator()(const float4* p) const { return *p; }
+};
+
+// A node's eight moving populations (one aligned 32-byte sector) in one
+// 256-bit load.  Two 16-byte loads of 32-byte records walk the same sectors
+// twice, and the gathers' share of the L1 data pipe is what the BGK step
+// kernels feel first.
+__device__ __forceinline__ void ldg_pair(const float4* p, float4& a, float4& b) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "l"(p));
+}
 
 // 1D quadratic Lagrange basis on {-1, 0, 1} at t
 __device__ __forceinline__ void lag3(float t, float& l0, float& l1, float& l2) {
@@ -169,8 +250,8 @@ __device__ __forceinline__ void wls_acc_diff(float a1, float a2, float a3, float
 
 __device__ __forceinline__ void wls_acc(const float4* __restrict__ f8, int j, float U, float V, float W, float Wp,
                                         float m1, float m2, const float4& oa, const float4& ob, float* acc) {
-    const float4 ra = __ldg(f8 + 2 * (size_t)j);
-    const float4 rb = __ldg(f8 + 2 * (size_t)j + 1);
+    float4 ra, rb;
+    ldg_pair(f8 + 2 * (size_t)j, ra, rb);
     wls_acc_diff(ra.x - oa.x, ra.y - oa.y, ra.z - oa.z, ra.w - oa.w, rb.x - ob.x, rb.y - ob.y, rb.z - ob.z,
                  rb.w - ob.w, U, V, W, Wp, m1, m2, acc);
 }
@@ -199,13 +280,13 @@ template <int KQ>
 __device__ __forceinline__ float wls_general(const Stencil& S, const float4* __restrict__ f8, int p, int k_src,
                                              const float* pb) {
     const float own = pop(f8, p, k_src);
+    const float4* b = rec_lane<KQ>(S, p);
     float acc = 0.f;
 #pragma unroll
     for (int q = 0; q < KQ; ++q) {
-        const int4 id = __ldg(S.idx + (size_t)q * S.n_pad + p);
+        const int4 id = rec_ids<KQ>(b, q, p, LdCached{});
         float4 m[6];
-#pragma unroll
-        for (int a = 0; a < 6; ++a) m[a] = __ldg(S.M + (size_t)(a * KQ + q) * S.n_pad + p);
+        rec_group<KQ>(b, q, m, LdCached{});
         const int ids[4] = {id.x, id.y, id.z, id.w};
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -224,9 +305,11 @@ __device__ __forceinline__ float wls_general(const Stencil& S, const float4* __r
 }
 
 __device__ __forceinline__ void lag_block(const Stencil& S, int p, int* ids) {
-    const int4 i0 = __ldg(S.idx + p);
-    const int4 i1 = __ldg(S.idx + (size_t)S.n_pad + p);
-    const int4 i2 = __ldg(S.idx + 2 * (size_t)S.n_pad + p);
+    const int4* b = S.rec ? reinterpret_cast<const int4*>(rec_lane(S, p)) : S.idx + p;
+    const size_t step = S.rec ? 32 : S.n_pad;
+    const int4 i0 = __ldg(b);
+    const int4 i1 = __ldg(b + step);
+    const int4 i2 = __ldg(b + 2 * step);
     ids[0] = i0.x; ids[1] = i0.y; ids[2] = i0.z; ids[3] = i0.w;
     ids[4] = i1.x; ids[5] = i1.y; ids[6] = i1.z; ids[7] = i1.w;
     ids[8] = i2.x;

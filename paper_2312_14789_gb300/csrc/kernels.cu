@@ -1,6 +1,6 @@
 // State I/O, macroscopic fields, the momentum-exchange force and the FP64
 // reductions; the step kernels are in kernels_bgk.cu, kernels_tau1.cu,
-// kernels_rbf.cu, kernels_ring1.cu and kernels_tma.cu.
+// kernels_rbf.cu, kernels_warp.cu and kernels_tma.cu.
 //
 // All population values are stored minus their weight omega_k (and rho as
 // rho - 1) so that FP32 keeps the small deviations that carry the flow.
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(128) force_kernel(Stencil S, int model, int n_
             if (model == 0) {
                 if (S.bb_mode == 0) {
                     val = pop(st8, p, kp);
-                } else if (kind == 0 && S.Wr) {
+                } else if (kind == 0 && !S.rec) {
                     val = rbf_general<KQ>(S, st8, p, k - 1, kp);
                 } else if (kind == 0) {
                     float pb[6];
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(128) force_kernel(Stencil S, int model, int n_
                 if (S.bb_mode == 0) {
                     const float4 me = ruv[p];
                     d[0] = me.x; d[1] = me.y; d[2] = me.z;
-                } else if (kind == 0 && S.Wr) {
+                } else if (kind == 0 && !S.rec) {
                     d[0] = d[1] = d[2] = 0.f;
                     for (int q = 0; q < KQ; ++q) {
                         const int4 id = S.idx[(size_t)q * S.n_pad + p];
@@ -197,24 +197,32 @@ __global__ void __launch_bounds__(128) force_kernel(Stencil S, int model, int n_
                     float pb[6];
                     basis_at(k, L.t[k - 1], pb);
                     d[0] = d[1] = d[2] = 0.f;
+                    // centred on the node's own values, as its own column is not stored
+                    const float4* lane_rows = rec_lane<KQ>(S, p);
+                    const float4 me = ruv[p];
                     for (int q = 0; q < KQ; ++q) {
-                        const int4 id = S.idx[(size_t)q * S.n_pad + p];
+                        const int4 id = rec_ids<KQ>(lane_rows, q, p, LdCached{});
+                        float4 m[6];
+                        rec_group<KQ>(lane_rows, q, m, LdCached{});
                         const int ids[4] = {id.x, id.y, id.z, id.w};
+#pragma unroll
                         for (int c = 0; c < 4; ++c) {
                             float tcol[6], mm[6];
-                            for (int aa = 0; aa < 6; ++aa) {
-                                const float4 m = S.M[(size_t)(aa * KQ + q) * S.n_pad + p];
-                                tcol[aa] = c == 0 ? m.x : (c == 1 ? m.y : (c == 2 ? m.z : m.w));
-                            }
+#pragma unroll
+                            for (int aa = 0; aa < 6; ++aa) tcol[aa] = reinterpret_cast<const float*>(m)[4 * aa + c];
                             unbasis(tcol, mm);
                             float w = 0.f;
+#pragma unroll
                             for (int aa = 0; aa < 6; ++aa) w = fmaf(pb[aa], mm[aa], w);
                             const float4 v = ruv[ids[c]];
-                            d[0] = fmaf(w, v.x, d[0]);
-                            d[1] = fmaf(w, v.y, d[1]);
-                            d[2] = fmaf(w, v.z, d[2]);
+                            d[0] = fmaf(w, v.x - me.x, d[0]);
+                            d[1] = fmaf(w, v.y - me.y, d[1]);
+                            d[2] = fmaf(w, v.z - me.z, d[2]);
                         }
                     }
+                    d[0] += me.x;
+                    d[1] += me.y;
+                    d[2] += me.z;
                 } else {
                     int ids[9];
                     lag_block(S, p, ids);

@@ -40,7 +40,18 @@ cudaError_t launch_set_tau1(int n, const int* perm, const double* ru, float4* s,
 // tau = 1: holds the m nodes' states fixed in later steps by making them
 // equilibrium-kind nodes whose record is their current state (run to steady
 // state of a batch: samples that have converged)
-cudaError_t launch_freeze_tau1(int m, uint8_t* meta, float4* eqv, const float4* state, cudaStream_t st);
+cudaError_t launch_freeze_tau1(int first, int m, uint8_t* meta, float4* eqv, const float4* state, cudaStream_t st);
+// brings the tile records and what each tile fetches in line with the kind
+// bytes after they changed; no step may be launched before the stream has
+// been synchronised
+cudaError_t launch_record_kinds(const dev::Stencil& S, float4* rec, uint8_t* need, int* range, cudaStream_t st);
+// blocks (and tile ranges) of the per-warp-slot step for n nodes
+int warp_step_ranges(int n);
+// step kernels with a shared-memory slot per warp (kernels_warp.cu), variants
+// 27..29; backward walks the tiles from the last one where that is of use
+cudaError_t launch_step_warp(int variant, int model, const dev::Stencil& S, const float4* a8, const float* a0,
+                             float4* b8, float* b0, const float4* ra, float4* rb, const dev::Collide& C, int backward,
+                             int* err, const dev::Wait& W, cudaStream_t st);
 cudaError_t launch_get_tau1(int n, const int* perm, const float4* s, double* ru, cudaStream_t st);
 cudaError_t launch_macroscopics(int model, int n, const int* perm, const float4* f8, const float* f0,
                                 const float4* ruv, float ax, float ay, const uint16_t* node_sample,
@@ -51,11 +62,6 @@ bool tma_supported(int Kq);
 cudaError_t launch_step_tma(int variant, int model, const dev::Stencil& S, const float4* f8in, const float* f0in,
                             float4* f8out, float* f0out, const float4* rin, float4* rout, const dev::Collide& C,
                             int* err, const dev::Wait& W, cudaStream_t st);
-// persistent one-lane-per-node step with a bulk-copy ring of stencil rows
-// (kernels.cu), variants 27..29
-cudaError_t launch_step_ring1(int variant, int model, const dev::Stencil& S, const float4* f8in, const float* f0in,
-                              float4* f8out, float* f0out, const float4* rin, float4* rout, const dev::Collide& C,
-                              int* err, const dev::Wait& W, cudaStream_t st);
 int force_blocks(int n_link_nodes);
 cudaError_t launch_force(const dev::Stencil& S, int model, int n_link_nodes, const int* link_nodes,
                          const float* area_over_s2, const float4* f8, const float4* ruv, const dev::Collide& C,

@@ -67,20 +67,24 @@ __global__ void __launch_bounds__(128) bgk_link_nodes(Stencil S, const float4* _
     }
     const LinkRec L = S.links[S.link_slot[p]];
     const bool interp = S.bb_mode != 0;
-    const float4 oa = __ldg(f8in + 2 * (size_t)p);
-    const float4 ob = __ldg(f8in + 2 * (size_t)p + 1);
+    float4 oa, ob;
+    ldg_pair(f8in + 2 * (size_t)p, oa, ob);
     const float own[8] = {oa.x, oa.y, oa.z, oa.w, ob.x, ob.y, ob.z, ob.w};
     float acc[8], lk[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc[k] = lk[k] = 0.f;
+    const float4* lane_rows = rec_lane<KQ>(S, p);
     for (int j = r; j < 4 * KQ; j += 16) {
         const int q = j >> 2, c = j & 3;
-        const int id = reinterpret_cast<const int*>(S.idx + (size_t)q * S.n_pad + p)[c];
+        const bool sp = q == TileRec<KQ>::kSp;
+        if (sp && c == 3) continue;  // the kind word
+        const int id = reinterpret_cast<const int*>(lane_rows + q * 32)[c];
         float t[6];
 #pragma unroll
-        for (int a = 0; a < 6; ++a) t[a] = reinterpret_cast<const float*>(S.M + (size_t)(a * KQ + q) * S.n_pad + p)[c];
-        const float4 ra = __ldg(f8in + 2 * (size_t)id);
-        const float4 rb = __ldg(f8in + 2 * (size_t)id + 1);
+        for (int a = 0; a < 5; ++a) t[a] = reinterpret_cast<const float*>(lane_rows + (TileRec<KQ>::m_row(q) + a) * 32)[c];
+        t[5] = reinterpret_cast<const float*>(lane_rows + (TileRec<KQ>::m_row(q) + (sp ? c : 5)) * 32)[sp ? 3 : c];
+        float4 ra, rb;
+        ldg_pair(f8in + 2 * (size_t)id, ra, rb);
         const float d[8] = {ra.x - oa.x, ra.y - oa.y, ra.z - oa.z, ra.w - oa.w,
                             rb.x - ob.x, rb.y - ob.y, rb.z - ob.z, rb.w - ob.w};
         wls_acc_diff(d[0], d[1], d[2], d[3], d[4], d[5], d[6], d[7], t[0], t[1], t[2], t[3], t[4], t[5], acc);
@@ -147,18 +151,16 @@ __device__ __forceinline__ void prefetch_tile_staged(const Stencil& S, int tile,
     if (tile >= n_tiles) return;
     const int base = tile * kStageTile;
     const int nodes = min(kStageTile, S.n_pad - base);
-    for (int c = (int)lane; c < 7 * KQ + 2; c += 32) {
-        if (c < 6 * KQ)
-            prefetch_l2(S.M + (size_t)c * S.n_pad + base, (uint32_t)nodes * 16u);
-        else if (c < 7 * KQ)
-            prefetch_l2(S.lidx + (size_t)(c - 6 * KQ) * S.n_pad + base, (uint32_t)nodes * 8u);
-        else if (c == 7 * KQ)
-            prefetch_l2(S.meta + base, (uint32_t)((nodes + 15) / 16 * 16));
-        else {
-            // the member list, widened to 16-byte bounds (the list is padded)
-            const int a0 = __ldg(S.stage_off + tile) & ~3, a1 = (__ldg(S.stage_off + tile + 1) + 3) & ~3;
-            if (a1 > a0) prefetch_l2(S.stage_ids + a0, (uint32_t)(a1 - a0) * 4u);
-        }
+    const uint32_t bytes = (uint32_t)(nodes / 32) * (TileRec<KQ>::kRows * 512u), part = bytes / 32u;
+    prefetch_l2(reinterpret_cast<const uint8_t*>(rec_lane<KQ>(S, base)) + lane * part, part);
+    if ((int)lane < KQ) {
+        prefetch_l2(S.lidx + (size_t)lane * S.n_pad + base, (uint32_t)nodes * 8u);
+    } else if ((int)lane == KQ) {
+        prefetch_l2(S.meta + base, (uint32_t)((nodes + 15) / 16 * 16));
+    } else if ((int)lane == KQ + 1) {
+        // the member list, widened to 16-byte bounds (the list is padded)
+        const int a0 = __ldg(S.stage_off + tile) & ~3, a1 = (__ldg(S.stage_off + tile + 1) + 3) & ~3;
+        if (a1 > a0) prefetch_l2(S.stage_ids + a0, (uint32_t)(a1 - a0) * 4u);
     }
 }
 
@@ -185,8 +187,9 @@ __device__ __forceinline__ void staged_node(const Stencil& S, const float4* nb, 
         return;
     }
     const Collide C = collide_of(S, C0, p);
-    const float4 oa = __ldg(f8in + 2 * (size_t)p);
-    const float4 ob = __ldg(f8in + 2 * (size_t)p + 1);
+    float4 oa, ob;
+    ldg_pair(f8in + 2 * (size_t)p, oa, ob);
+    const float4* lane_rows = rec_lane<KQ>(S, p);
     ushort4 lv[KQ];
 #pragma unroll
     for (int q = 0; q < KQ; ++q) lv[q] = __ldcs(S.lidx + (size_t)q * S.n_pad + p);
@@ -196,8 +199,7 @@ __device__ __forceinline__ void staged_node(const Stencil& S, const float4* nb, 
 #pragma unroll
     for (int q = 0; q < KQ; ++q) {
         float4 m[6];
-#pragma unroll
-        for (int a = 0; a < 6; ++a) m[a] = ld_stream(S.M + (size_t)(a * KQ + q) * S.n_pad + p);
+        rec_group<KQ>(lane_rows, q, m, LdStream{});
         const float* mc = reinterpret_cast<const float*>(m);
         const int l[4] = {lv[q].x, lv[q].y, lv[q].z, lv[q].w};
 #pragma unroll

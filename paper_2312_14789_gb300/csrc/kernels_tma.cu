@@ -2,10 +2,9 @@
 //
 // The per-node stencil data (least-squares matrix M, neighbour indices, meta
 // byte) are read exactly once per step and make up ~90% of the bytes, so they
-// are streamed through shared memory: one producer warp per CTA issues
-// cp.async.bulk copies of whole node tiles (TN nodes: 6K/4 matrix rows, K/4
-// index rows and the meta bytes, each a contiguous TN x 16-byte chunk of the
-// interleaved layout) into a ring of STAGES buffers guarded by mbarriers;
+// are streamed through shared memory: one producer warp per CTA copies whole
+// node tiles (TN nodes: TN / 32 consecutive tile records, one cp.async.bulk)
+// into a ring of STAGES buffers guarded by mbarriers;
 // TN * 4 consumer threads (four lanes per node, one neighbour group of four
 // each) gather the neighbours' populations through L1/L2, combine their
 // partial sums with quad shuffles and split the collision.  The grid holds
@@ -25,6 +24,7 @@
 #include "device_common.cuh"
 #include "kernels.h"
 #include "ring.cuh"
+#include "step_node.cuh"
 
 namespace mlbm {
 namespace dev {
@@ -61,12 +61,11 @@ __global__ void __launch_bounds__(Tile<KQ, TN, STAGES>::kThreads, MINB)
             return;
         }
         const uint8_t* st = smem + s * L::kStage;
-        const float4* sM = reinterpret_cast<const float4*>(st);
-        const int4* sI = reinterpret_cast<const int4*>(st + L::kM);
         const int p = tile * TN + t;
+        const SmemRows<KQ> R(st, t, p);
         if (p < S.n) {
             const Collide C = collide_of(S, C0, p);
-            const uint8_t meta = st[L::kM + L::kI + t];
+            const uint8_t meta = R.meta();
             const int kind = meta & 3;
             float g[9];
             if (kind == 2) {
@@ -76,8 +75,8 @@ __global__ void __launch_bounds__(Tile<KQ, TN, STAGES>::kThreads, MINB)
                 float acc[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) acc[k] = 0.f;
-                const float4 oa = __ldg(f8in + 2 * (size_t)p);
-                const float4 ob = __ldg(f8in + 2 * (size_t)p + 1);
+                float4 oa, ob;
+                ldg_pair(f8in + 2 * (size_t)p, oa, ob);
                 const float r = (kind == 1) ? __ldg(S.lag_r + p) : 0.f;
                 const float cx = (kind == 1) ? (float)ex_of(meta >> 4) : 0.f;
                 const float cy = (kind == 1) ? (float)ey_of(meta >> 4) : 0.f;
@@ -86,10 +85,9 @@ __global__ void __launch_bounds__(Tile<KQ, TN, STAGES>::kThreads, MINB)
                     for (int i = 0; i < (KQ + 3) / 4; ++i) {
                         const int q = 4 * i + h;
                         if (q < KQ) {
-                            const int4 id = sI[q * TN + t];
+                            const int4 id = R.idx_row(q);
                             float4 m[6];
-#pragma unroll
-                            for (int a = 0; a < 6; ++a) m[a] = sM[(a * KQ + q) * TN + t];
+                            R.group(q, m);
                             wls_acc(f8in, id.x, m[0].x, m[1].x, m[2].x, m[3].x, m[4].x, m[5].x, oa, ob, acc);
                             wls_acc(f8in, id.y, m[0].y, m[1].y, m[2].y, m[3].y, m[4].y, m[5].y, oa, ob, acc);
                             wls_acc(f8in, id.z, m[0].z, m[1].z, m[2].z, m[3].z, m[4].z, m[5].z, oa, ob, acc);
@@ -97,8 +95,8 @@ __global__ void __launch_bounds__(Tile<KQ, TN, STAGES>::kThreads, MINB)
                         }
                     }
                 } else {
-                    const int4 i0 = sI[t], i1 = sI[TN + t], i2 = sI[2 * TN + t];
-                    const int ids[9] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w, i2.x};
+                    int ids[9];
+                    R.lag(ids);
                     float xp[3], x0[3], xm[3], yp[3], y0[3], ym[3];
                     lag3(-r - cx, xp[0], xp[1], xp[2]);
                     lag3(-cx, x0[0], x0[1], x0[2]);
@@ -111,8 +109,8 @@ __global__ void __launch_bounds__(Tile<KQ, TN, STAGES>::kThreads, MINB)
                         if ((bp & 3) != h) continue;
                         const int b = bp / 3, a = bp % 3;
                         const int j = ids[bp];
-                        const float4 ra = __ldg(f8in + 2 * (size_t)j);
-                        const float4 rb = __ldg(f8in + 2 * (size_t)j + 1);
+                        float4 ra, rb;
+                        ldg_pair(f8in + 2 * (size_t)j, ra, rb);
                         acc[0] = fmaf(xp[a] * y0[b], ra.x - oa.x, acc[0]);
                         acc[1] = fmaf(x0[a] * yp[b], ra.y - oa.y, acc[1]);
                         acc[2] = fmaf(xm[a] * y0[b], ra.z - oa.z, acc[2]);
@@ -218,12 +216,11 @@ __global__ void __launch_bounds__(Tile<KQ, TN, STAGES>::kThreads, MINB)
             return;
         }
         const uint8_t* st = smem + s * L::kStage;
-        const float4* sM = reinterpret_cast<const float4*>(st);
-        const int4* sI = reinterpret_cast<const int4*>(st + L::kM);
         const int p = tile * TN + t;
+        const SmemRows<KQ> R(st, t, p);
         if (p < S.n) {
             const Collide C = collide_of(S, C0, p);
-            const uint8_t meta = st[L::kM + L::kI + t];
+            const uint8_t meta = R.meta();
             const int kind = meta & 3;
             if (kind == 2) {
                 if (h == 0) out[p] = S.eqv[p];
@@ -241,10 +238,9 @@ __global__ void __launch_bounds__(Tile<KQ, TN, STAGES>::kThreads, MINB)
                     for (int i = 0; i < (KQ + 3) / 4; ++i) {
                         const int q = 4 * i + h;
                         if (q < KQ) {
-                            const int4 id = sI[q * TN + t];
+                            const int4 id = R.idx_row(q);
                             float4 m[6];
-#pragma unroll
-                            for (int a = 0; a < 6; ++a) m[a] = sM[(a * KQ + q) * TN + t];
+                            R.group(q, m);
                             const int ids[4] = {id.x, id.y, id.z, id.w};
 #pragma unroll
                             for (int cc = 0; cc < 4; ++cc) {
@@ -276,8 +272,8 @@ __global__ void __launch_bounds__(Tile<KQ, TN, STAGES>::kThreads, MINB)
                         unbasis(tc, c[f]);
                     }
                 } else {
-                    const int4 i0 = sI[t], i1 = sI[TN + t], i2 = sI[2 * TN + t];
-                    const int ids[9] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w, i2.x};
+                    int ids[9];
+                    R.lag(ids);
 #pragma unroll
                     for (int b = 0; b < 9; ++b) v9[b] = __ldg(in + ids[b]);
                     r = __ldg(S.lag_r + p);

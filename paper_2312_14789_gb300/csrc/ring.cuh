@@ -1,7 +1,6 @@
-// Bulk-copy ring shared by the pipelined step kernels (kernels_tma.cu: four
-// lanes per node; kernels.cu: one lane per node).  A producer warp streams
-// each tile's stencil rows (least-squares matrix, neighbour indices, meta
-// bytes: contiguous TN x 16-byte chunks of the interleaved layout) with
+// Bulk copies, mbarriers and the ring of the pipelined step kernels of four
+// lanes per node (kernels_tma.cu); kernels_warp.cu uses the copies and waits.  A producer warp streams
+// each tile's records (see TileRec; TN / 32 of them, contiguous) with one
 // cp.async.bulk into a ring of STAGES shared-memory buffers guarded by
 // mbarriers; consumer warps wait for a stage, read it, and release it.
 // Every wait is bounded by a time budget (Wait); see kernels_tma.cu.
@@ -58,10 +57,7 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 
 template <int KQ, int TN, int STAGES>
 struct Tile {
-    static constexpr int kM = 6 * KQ * TN * 16;
-    static constexpr int kI = KQ * TN * 16;
-    static constexpr int kMeta = (TN + 15) / 16 * 16;
-    static constexpr int kStage = kM + kI + kMeta;
+    static constexpr int kStage = TN / 32 * TileRec<KQ>::kRows * 512;
     static constexpr int kBar = STAGES * kStage;
     static constexpr int kBytes = kBar + 2 * STAGES * 8;
     static constexpr int kConsumers = TN * 4;
@@ -69,14 +65,12 @@ struct Tile {
 };
 
 // producer warp: fill the ring for this CTA's tiles.  Lane 0 waits for a
-// free stage and arms its barrier with the byte count; then the 32 lanes issue
-// the tile's 7K/4 + 1 bulk copies in parallel.
+// free stage, arms its barrier with the byte count and issues the copy.
 template <int KQ, int TN, int STAGES>
 __device__ __forceinline__ void produce(const Stencil& S, uint8_t* smem, uint64_t* full, uint64_t* empty,
                                        int n_tiles, int* err, const Wait W) {
     using L = Tile<KQ, TN, STAGES>;
     const unsigned lane = threadIdx.x & 31u;
-    constexpr int kCopies = 7 * KQ + 1;
     // test switch: block 0 issues nothing for its first tile (no arrival, no
     // copies), so the consumers' bounded wait for that tile runs out
     const bool withhold = W.withhold && blockIdx.x == 0;
@@ -96,17 +90,9 @@ __device__ __forceinline__ void produce(const Stencil& S, uint8_t* smem, uint64_
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) break;
         if (skip) continue;
-        uint8_t* st = smem + s * L::kStage;
-        const size_t base = (size_t)tile * TN;
-        for (int c = lane; c < kCopies; c += 32) {
-            if (c < 6 * KQ)
-                bulk_g2s(st + c * TN * 16, S.M + (size_t)c * S.n_pad + base, TN * 16, &full[s]);
-            else if (c < 7 * KQ)
-                bulk_g2s(st + L::kM + (c - 6 * KQ) * TN * 16, S.idx + (size_t)(c - 6 * KQ) * S.n_pad + base,
-                         TN * 16, &full[s]);
-            else
-                bulk_g2s(st + L::kM + L::kI, S.meta + base, L::kMeta, &full[s]);
-        }
+        if (lane == 0)
+            bulk_g2s(smem + s * L::kStage, reinterpret_cast<const uint8_t*>(S.rec) + (size_t)tile * L::kStage,
+                     L::kStage, &full[s]);
         __syncwarp();
     }
     // drain: do not leave while copies may still be landing in this CTA's

@@ -1,6 +1,6 @@
 // Per-node device code of the fused step kernels, shared by the translation
 // units that instantiate them (kernels_bgk.cu, kernels_tau1.cu,
-// kernels_rbf.cu, kernels_ring1.cu).
+// kernels_rbf.cu, kernels_tma.cu, kernels_warp.cu).
 //
 // BGK/TRT step (Sec. 2.2 streaming, Eq. (3)-(9) collision), per node x:
 //   gather the post-collision populations of the K stencil nodes, evaluate the
@@ -23,6 +23,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 
 #include "device_common.cuh"
 
@@ -33,17 +34,34 @@ namespace dev {
 // Where a node's streamed stencil rows (meta byte, neighbour index groups,
 // matrix rows) come from: global memory (streaming loads, each row read once
 // per step), or a tile that a producer warp has already copied into shared
-// memory (the one-lane-per-node bulk-copy ring, variants 27-29).
+// memory (the bulk-copy ring, variants 4-7).
+template <int KQ>
 struct GlobalRows {
+    const float4* b;
+    const uint8_t* mt;
+    int p;
+    __device__ __forceinline__ GlobalRows(const Stencil& S, int p_) : b(rec_lane<KQ>(S, p_)), mt(S.meta), p(p_) {}
+    __device__ __forceinline__ uint8_t meta() const { return mt[p]; }
+    __device__ __forceinline__ int4 idx_row(int q) const { return rec_ids<KQ>(b, q, p, LdStream{}); }
+    __device__ __forceinline__ void group(int q, float4* m) const { rec_group<KQ>(b, q, m, LdStream{}); }
+    __device__ __forceinline__ void lag(int* ids) const {
+        const int4* i = reinterpret_cast<const int4*>(b);
+        const int4 i0 = __ldg(i), i1 = __ldg(i + 32), i2 = __ldg(i + 64);
+        ids[0] = i0.x; ids[1] = i0.y; ids[2] = i0.z; ids[3] = i0.w;
+        ids[4] = i1.x; ids[5] = i1.y; ids[6] = i1.z; ids[7] = i1.w;
+        ids[8] = i2.x;
+    }
+};
+
+// RBF-FD stencils: separate index rows; the weight rows are read by the node code
+struct RbfRows {
     const int4* idx;
-    const float4* M;
     const uint8_t* mt;
     int n_pad, p;
-    __device__ __forceinline__ GlobalRows(const Stencil& S, int p_)
-        : idx(S.idx), M(S.M), mt(S.meta), n_pad(S.n_pad), p(p_) {}
+    __device__ __forceinline__ RbfRows(const Stencil& S, int p_) : idx(S.idx), mt(S.meta), n_pad(S.n_pad), p(p_) {}
     __device__ __forceinline__ uint8_t meta() const { return mt[p]; }
     __device__ __forceinline__ int4 idx_row(int q) const { return ld_stream(idx + (size_t)q * n_pad + p); }
-    __device__ __forceinline__ float4 m_row(int r) const { return ld_stream(M + (size_t)r * n_pad + p); }
+    __device__ __forceinline__ void group(int, float4*) const {}
     __device__ __forceinline__ void lag(int* ids) const {
         const int4 i0 = __ldg(idx + p), i1 = __ldg(idx + (size_t)n_pad + p), i2 = __ldg(idx + 2 * (size_t)n_pad + p);
         ids[0] = i0.x; ids[1] = i0.y; ids[2] = i0.z; ids[3] = i0.w;
@@ -52,24 +70,77 @@ struct GlobalRows {
     }
 };
 
+template <int KQ>
 struct SmemRows {
-    const float4* sM;     // [6 K/4][TN]
-    const int4* sI;       // [K/4][TN]
-    const uint8_t* sMeta; // [TN]
-    int t, tn;
-    __device__ __forceinline__ uint8_t meta() const { return sMeta[t]; }
-    __device__ __forceinline__ int4 idx_row(int q) const { return sI[q * tn + t]; }
-    __device__ __forceinline__ float4 m_row(int r) const { return sM[r * tn + t]; }
+    const float4* b;  // row 0 of the node's lane in the staged record
+    int p;
+    __device__ __forceinline__ SmemRows(const uint8_t* stage, int t, int p_)
+        : b(reinterpret_cast<const float4*>(stage) + ((t >> 5) * TileRec<KQ>::kRows) * 32 + (t & 31)), p(p_) {}
+    __device__ __forceinline__ uint8_t meta() const {
+        return (uint8_t)(__float_as_int(b[TileRec<KQ>::kSp * 32].w) & 0xff);
+    }
+    __device__ __forceinline__ int4 idx_row(int q) const { return rec_ids<KQ>(b, q, p, LdPlain{}); }
+    __device__ __forceinline__ void group(int q, float4* m) const { rec_group<KQ>(b, q, m, LdPlain{}); }
     __device__ __forceinline__ void lag(int* ids) const {
-        const int4 i0 = sI[t], i1 = sI[tn + t], i2 = sI[2 * tn + t];
+        const int4* i = reinterpret_cast<const int4*>(b);
+        const int4 i0 = i[0], i1 = i[32], i2 = i[64];
         ids[0] = i0.x; ids[1] = i0.y; ids[2] = i0.z; ids[3] = i0.w;
         ids[4] = i1.x; ids[5] = i1.y; ids[6] = i1.z; ids[7] = i1.w;
         ids[8] = i2.x;
     }
 };
 
-__device__ __forceinline__ GlobalRows rows_of(const Stencil& S, int p, const GlobalRows*) { return GlobalRows(S, p); }
-__device__ __forceinline__ SmemRows rows_of(const Stencil&, int, const SmemRows* r) { return *r; }
+template <class Rows>
+__device__ __forceinline__ Rows rows_of(const Stencil& S, int p, const Rows* given) {
+    if constexpr (std::is_constructible<Rows, const Stencil&, int>::value) return Rows(S, p);
+    else return *given;
+}
+
+// Increments of the eight streamed populations over the node's own (oa, ob)
+// from its 3x3 Lagrange block (LPN = 2: this lane's half of the nine points).
+template <int LPN>
+__device__ __forceinline__ void lagrange_increments(const float4* __restrict__ f8in, const int* ids, float r, float cx,
+                                                    float cy, const float4& oa, const float4& ob, int h, float* acc) {
+    // basis values for e_x, e_y in {+1, 0, -1}: t = -r e - c
+    float xp[3], x0[3], xm[3], yp[3], y0[3], ym[3];
+    lag3(-r - cx, xp[0], xp[1], xp[2]);
+    lag3(-cx, x0[0], x0[1], x0[2]);
+    lag3(r - cx, xm[0], xm[1], xm[2]);
+    lag3(-r - cy, yp[0], yp[1], yp[2]);
+    lag3(-cy, y0[0], y0[1], y0[2]);
+    lag3(r - cy, ym[0], ym[1], ym[2]);
+#pragma unroll
+    for (int bp = 0; bp < 9; ++bp) {
+        if (LPN == 2 && (bp & 1) != h) continue;
+        const int b = bp / 3, a = bp % 3;
+        const int j = ids[bp];
+        float4 ra, rb;
+        ldg_pair(f8in + 2 * (size_t)j, ra, rb);
+        const float4 fa = make_float4(ra.x - oa.x, ra.y - oa.y, ra.z - oa.z, ra.w - oa.w);
+        const float4 fb = make_float4(rb.x - ob.x, rb.y - ob.y, rb.z - ob.z, rb.w - ob.w);
+        acc[0] = fmaf(xp[a] * y0[b], fa.x, acc[0]);
+        acc[1] = fmaf(x0[a] * yp[b], fa.y, acc[1]);
+        acc[2] = fmaf(xm[a] * y0[b], fa.z, acc[2]);
+        acc[3] = fmaf(x0[a] * ym[b], fa.w, acc[3]);
+        acc[4] = fmaf(xp[a] * yp[b], fb.x, acc[4]);
+        acc[5] = fmaf(xm[a] * yp[b], fb.y, acc[5]);
+        acc[6] = fmaf(xm[a] * ym[b], fb.z, acc[6]);
+        acc[7] = fmaf(xp[a] * ym[b], fb.w, acc[7]);
+    }
+}
+
+// A Lagrange node's interpolated bounce-back link in direction k: population
+// k' (own value o) at the reflected point x + tt s e_k.
+__device__ __forceinline__ float lagrange_link(const float4* __restrict__ f8in, const int* ids, float r, float cx,
+                                               float cy, int k, float tt, float o) {
+    float lx[3], ly[3];
+    lag3(tt * r * ex_of(k) - cx, lx[0], lx[1], lx[2]);
+    lag3(tt * r * ey_of(k) - cy, ly[0], ly[1], ly[2]);
+    float v = 0.f;
+    for (int b = 0; b < 3; ++b)
+        for (int a = 0; a < 3; ++a) v = fmaf(lx[a] * ly[b], pop(f8in, ids[b * 3 + a], opp_of(k)) - o, v);
+    return o + v;
+}
 
 // ------------------------------------------------------------ BGK / TRT
 // LPN lanes (1 or 2) cooperate on one node: lane h takes the neighbour groups
@@ -80,7 +151,8 @@ __device__ __forceinline__ SmemRows rows_of(const Stencil&, int, const SmemRows*
 // loads the first three index rows and the rest population before the node
 // kind is known (they are read by every stencil kind), so they are in flight
 // together with the meta byte
-template <int KQ, int LPN, bool LINKS = true, bool RBF = false, bool SPEC = false, class Rows = GlobalRows>
+template <int KQ, int LPN, bool LINKS = true, bool RBF = false, bool SPEC = false,
+          class Rows = typename std::conditional<RBF, RbfRows, GlobalRows<KQ>>::type>
 __device__ __forceinline__ void bgk_node(const Stencil& S, const float4* __restrict__ f8in,
                                          const float* __restrict__ f0in, float4* __restrict__ f8out,
                                          float* __restrict__ f0out, const Collide& C0, int p, int h, unsigned grp,
@@ -110,8 +182,8 @@ __device__ __forceinline__ void bgk_node(const Stencil& S, const float4* __restr
         const float r = (kind == 1) ? __ldg(S.lag_r + p) : 0.f;
         const float cx = (kind == 1) ? (float)ex_of(meta >> 4) : 0.f;
         const float cy = (kind == 1) ? (float)ey_of(meta >> 4) : 0.f;
-        const float4 oa = __ldg(f8in + 2 * (size_t)p);
-        const float4 ob = __ldg(f8in + 2 * (size_t)p + 1);
+        float4 oa, ob;
+        ldg_pair(f8in + 2 * (size_t)p, oa, ob);
         if (kind == 0 && RBF) {
             // f_k(x) = own_k + sum_j w_kj (f_k(j) - own_k), weights per direction
 #pragma unroll
@@ -133,8 +205,8 @@ __device__ __forceinline__ void bgk_node(const Stencil& S, const float4* __restr
                     const int ids[4] = {id.x, id.y, id.z, id.w};
 #pragma unroll
                     for (int c = 0; c < 4; ++c) {
-                        const float4 ra = __ldg(f8in + 2 * (size_t)ids[c]);
-                        const float4 rb = __ldg(f8in + 2 * (size_t)ids[c] + 1);
+                        float4 ra, rb;
+                        ldg_pair(f8in + 2 * (size_t)ids[c], ra, rb);
                         acc[0] = fmaf(wt[0][c], ra.x - oa.x, acc[0]);
                         acc[1] = fmaf(wt[1][c], ra.y - oa.y, acc[1]);
                         acc[2] = fmaf(wt[2][c], ra.z - oa.z, acc[2]);
@@ -160,8 +232,7 @@ __device__ __forceinline__ void bgk_node(const Stencil& S, const float4* __restr
                 if (q < KQ) {
                     const int4 id = idv[i];
                     float4 m[6];
-#pragma unroll
-                    for (int a = 0; a < 6; ++a) m[a] = R.m_row(a * KQ + q);
+                    R.group(q, m);
                     wls_acc(f8in, id.x, m[0].x, m[1].x, m[2].x, m[3].x, m[4].x, m[5].x, oa, ob, acc);
                     wls_acc(f8in, id.y, m[0].y, m[1].y, m[2].y, m[3].y, m[4].y, m[5].y, oa, ob, acc);
                     wls_acc(f8in, id.z, m[0].z, m[1].z, m[2].z, m[3].z, m[4].z, m[5].z, oa, ob, acc);
@@ -171,32 +242,7 @@ __device__ __forceinline__ void bgk_node(const Stencil& S, const float4* __restr
         } else {
             int ids[9];
             R.lag(ids);
-            // basis values for e_x, e_y in {+1, 0, -1}: t = -r e - c
-            float xp[3], x0[3], xm[3], yp[3], y0[3], ym[3];
-            lag3(-r - cx, xp[0], xp[1], xp[2]);
-            lag3(-cx, x0[0], x0[1], x0[2]);
-            lag3(r - cx, xm[0], xm[1], xm[2]);
-            lag3(-r - cy, yp[0], yp[1], yp[2]);
-            lag3(-cy, y0[0], y0[1], y0[2]);
-            lag3(r - cy, ym[0], ym[1], ym[2]);
-#pragma unroll
-            for (int bp = 0; bp < 9; ++bp) {
-                if (LPN == 2 && (bp & 1) != h) continue;
-                const int b = bp / 3, a = bp % 3;
-                const int j = ids[bp];
-                const float4 ra = __ldg(f8in + 2 * (size_t)j);
-                const float4 rb = __ldg(f8in + 2 * (size_t)j + 1);
-                const float4 fa = make_float4(ra.x - oa.x, ra.y - oa.y, ra.z - oa.z, ra.w - oa.w);
-                const float4 fb = make_float4(rb.x - ob.x, rb.y - ob.y, rb.z - ob.z, rb.w - ob.w);
-                acc[0] = fmaf(xp[a] * y0[b], fa.x, acc[0]);
-                acc[1] = fmaf(x0[a] * yp[b], fa.y, acc[1]);
-                acc[2] = fmaf(xm[a] * y0[b], fa.z, acc[2]);
-                acc[3] = fmaf(x0[a] * ym[b], fa.w, acc[3]);
-                acc[4] = fmaf(xp[a] * yp[b], fb.x, acc[4]);
-                acc[5] = fmaf(xm[a] * yp[b], fb.y, acc[5]);
-                acc[6] = fmaf(xm[a] * ym[b], fb.z, acc[6]);
-                acc[7] = fmaf(xp[a] * ym[b], fb.w, acc[7]);
-            }
+            lagrange_increments<LPN>(f8in, ids, r, cx, cy, oa, ob, h, acc);
         }
         if (LPN == 2) {
 #pragma unroll
@@ -223,15 +269,7 @@ __device__ __forceinline__ void bgk_node(const Stencil& S, const float4* __restr
                 } else {
                     int ids[9];
                     lag_block(S, p, ids);
-                    const float tt = L.t[k - 1];
-                    float lx[3], ly[3];
-                    lag3(tt * r * ex_of(k) - cx, lx[0], lx[1], lx[2]);
-                    lag3(tt * r * ey_of(k) - cy, ly[0], ly[1], ly[2]);
-                    const float o = own[kp - 1];
-                    float v = 0.f;
-                    for (int b = 0; b < 3; ++b)
-                        for (int a = 0; a < 3; ++a) v = fmaf(lx[a] * ly[b], pop(f8in, ids[b * 3 + a], kp) - o, v);
-                    acc[k - 1] = o + v;
+                    acc[k - 1] = lagrange_link(f8in, ids, r, cx, cy, k, L.t[k - 1], own[kp - 1]);
                 }
             }
         }
@@ -273,14 +311,26 @@ __device__ __forceinline__ void bgk_node_split(const Stencil& S, const float4* _
         const float cy = (kind == 1) ? (float)ey_of(meta >> 4) : 0.f;
         if (kind == 0) {
             const int ra = h ? 2 : 0, rb = h ? 3 : 1;
+            const float4* lane_rows = rec_lane<KQ>(S, p);
             // UQ neighbour groups in flight at a time (register budget)
 #pragma unroll UQ
             for (int q = 0; q < KQ; ++q) {
-                const int4 id = ld_stream(S.idx + (size_t)q * S.n_pad + p);
-                const float4 mA = ld_stream(S.M + (size_t)(ra * KQ + q) * S.n_pad + p);
-                const float4 mB = ld_stream(S.M + (size_t)(rb * KQ + q) * S.n_pad + p);
-                const float4 m1 = ld_stream(S.M + (size_t)(4 * KQ + q) * S.n_pad + p);
-                const float4 m2 = ld_stream(S.M + (size_t)(5 * KQ + q) * S.n_pad + p);
+                const int4 id = rec_ids<KQ>(lane_rows, q, p, LdStream{});
+                const float4* grp_rows = lane_rows + TileRec<KQ>::m_row(q) * 32;
+                float4 mA, mB, m1, m2;
+                if (q == TileRec<KQ>::kSp) {
+                    float4 m[6];
+                    rec_group<KQ>(lane_rows, q, m, LdStream{});
+                    mA = h ? m[2] : m[0];
+                    mB = h ? m[3] : m[1];
+                    m1 = m[4];
+                    m2 = m[5];
+                } else {
+                    mA = ld_stream(grp_rows + ra * 32);
+                    mB = ld_stream(grp_rows + rb * 32);
+                    m1 = ld_stream(grp_rows + 4 * 32);
+                    m2 = ld_stream(grp_rows + 5 * 32);
+                }
                 const int ids[4] = {id.x, id.y, id.z, id.w};
                 const float A4[4] = {mA.x, mA.y, mA.z, mA.w}, B4[4] = {mB.x, mB.y, mB.z, mB.w};
                 const float P4[4] = {m1.x, m1.y, m1.z, m1.w}, Q4[4] = {m2.x, m2.y, m2.z, m2.w};
@@ -387,15 +437,11 @@ __device__ __forceinline__ void prefetch_l2(const void* ptr, uint32_t bytes) {
 template <int KQ>
 __device__ __forceinline__ void prefetch_tile(const Stencil& S, int base, int tn, unsigned lane) {
     if (base >= S.n) return;
+    // base is a multiple of 32: the tile's records are contiguous
     const int nodes = min(tn, S.n_pad - base);
-    for (int c = (int)lane; c < 7 * KQ + 1; c += 32) {
-        if (c < 6 * KQ)
-            prefetch_l2(S.M + (size_t)c * S.n_pad + base, (uint32_t)nodes * 16u);
-        else if (c < 7 * KQ)
-            prefetch_l2(S.idx + (size_t)(c - 6 * KQ) * S.n_pad + base, (uint32_t)nodes * 16u);
-        else
-            prefetch_l2(S.meta + base, (uint32_t)((nodes + 15) / 16 * 16));
-    }
+    const uint32_t bytes = (uint32_t)(nodes / 32) * (TileRec<KQ>::kRows * 512u), part = bytes / 32u;
+    prefetch_l2(reinterpret_cast<const uint8_t*>(rec_lane<KQ>(S, base)) + lane * part, part);
+    if (lane == 0) prefetch_l2(S.meta + base, (uint32_t)((nodes + 15) / 16 * 16));
 }
 
 // Programmatic dependent launch (variants 25, 26): a step grid lets the next
@@ -433,10 +479,58 @@ __device__ __forceinline__ void eval_coeffs(const float (*c)[6], const float* pb
     }
 }
 
+// A node's new state from its fitted coefficients (kind 0, monomial basis) or
+// its block's values (kind 1), one lane per node.
+__device__ __forceinline__ float4 tau1_finish(const Stencil& S, const Collide& C, const float4& me, int kind,
+                                              const float (*c)[6], const float4* v9, float r, float cx, float cy,
+                                              bool has_links, int p) {
+    LinkRec L;
+    L.mask = 0;
+    if (has_links) L = S.links[S.link_slot[p]];
+    const float rhox = 1.0f + me.x;
+    float mx = 0.f, my = 0.f;
+    float dm = w_of(0) * rhox * (-1.5f * (me.y * me.y + me.z * me.z)) + 0.5f * src(0, rhox, me.y, me.z, C.ax, C.ay);
+#pragma unroll
+    for (int k = 1; k < 9; ++k) {
+        const bool is_link = (L.mask >> k) & 1u;
+        const int sk = is_link ? opp_of(k) : k;
+        float d[3] = {0.f, 0.f, 0.f};  // increments over the node's own (dr, u, v)
+        if (!(is_link && S.bb_mode == 0)) {
+            const float tt = is_link ? L.t[k - 1] : -1.0f;
+            if (kind == 0) {
+                float pb[6];
+                basis_at(k, tt, pb);
+                eval_coeffs(c, pb, d);
+            } else {
+                float lx[3], ly[3];
+                lag3(tt * r * ex_of(k) - cx, lx[0], lx[1], lx[2]);
+                lag3(tt * r * ey_of(k) - cy, ly[0], ly[1], ly[2]);
+#pragma unroll
+                for (int b = 0; b < 3; ++b)
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        const float w = lx[a] * ly[b];
+                        const float4 v = v9[b * 3 + a];
+                        d[0] = fmaf(w, v.x - me.x, d[0]);
+                        d[1] = fmaf(w, v.y - me.y, d[1]);
+                        d[2] = fmaf(w, v.z - me.z, d[2]);
+                    }
+            }
+        }
+        tau1_accumulate(k, sk, is_link, d[0], d[1], d[2], rhox, me.y, me.z, C, dm, mx, my);
+    }
+    const float rho = rhox + dm;
+    const float inv = 1.0f / rho;
+    const float nux = me.y + (mx + 0.5f * rho * C.ax - dm * me.y) * inv;
+    const float nuy = me.z + (my + 0.5f * rho * C.ay - dm * me.z) * inv;
+    return make_float4(me.x + dm, nux, nuy, 0.f);
+}
+
 // LPN lanes per node: neighbour groups split as in the BGK kernel, the 18
 // fitted coefficients combined by a pair shuffle, the 8 directions split
 // (lane 0: k = 0..4, lane 1: k = 5..8) and the moment sums combined again.
-template <int KQ, int LPN, bool RBF = false, class Rows = GlobalRows>
+template <int KQ, int LPN, bool RBF = false,
+          class Rows = typename std::conditional<RBF, RbfRows, GlobalRows<KQ>>::type>
 __device__ __forceinline__ void tau1_node(const Stencil& S, const float4* __restrict__ in, float4* __restrict__ out,
                                           const Collide& C0, int p, int h, unsigned grp, const Rows* rows = nullptr) {
     const Rows R = rows_of(S, p, rows);
@@ -497,8 +591,7 @@ __device__ __forceinline__ void tau1_node(const Stencil& S, const float4* __rest
             if (q < KQ) {
                 const int4 id = idv[i];
                 float4 m[6];
-#pragma unroll
-                for (int a = 0; a < 6; ++a) m[a] = R.m_row(a * KQ + q);
+                R.group(q, m);
                 const int ids[4] = {id.x, id.y, id.z, id.w};
 #pragma unroll
                 for (int cc = 0; cc < 4; ++cc) {

@@ -49,10 +49,12 @@ __global__ void __launch_bounds__(128) wall_traction(Stencil S, int model, const
     double dr, ux, uy;
     node_state(model, f8, f0, ruv, ax, ay, p, dr, ux, uy);
     double uxx = 0, uxy = 0, uyx = 0, uyy = 0;
+    const float4* lane_rows = rec_lane<KQ>(S, p);
     for (int q = 0; q < KQ; ++q) {
-        const int4 id = S.idx[(size_t)q * S.n_pad + p];
-        const float4 gx = S.M[(size_t)(4 * KQ + q) * S.n_pad + p];
-        const float4 gy = S.M[(size_t)(5 * KQ + q) * S.n_pad + p];
+        const int4 id = rec_ids<KQ>(lane_rows, q, p, LdCached{});
+        float4 m[6];
+        rec_group<KQ>(lane_rows, q, m, LdCached{});
+        const float4 gx = m[4], gy = m[5];
         const int ids[4] = {id.x, id.y, id.z, id.w};
         const float wx[4] = {gx.x, gx.y, gx.z, gx.w};
         const float wy[4] = {gy.x, gy.y, gy.z, gy.w};
