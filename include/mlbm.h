@@ -536,17 +536,17 @@ mlbm_status mlbm_partition_nodes(const mlbm_stencils* st, int n_parts, const int
 /*
  * The partitioned step on the current device: one context per partition (its
  * owned stencils and a state with halo slots), all on one stream.  Every
- * mlbm_part_step advances each partition once, then for every pair (owner o,
- * receiver q) packs o's new states of q's halo nodes into a buffer of o and
- * copies it into q's own halo slots (cudaMemcpyAsync), so that no step reads
- * another partition's memory; after n steps the stream is synchronised.
+ * mlbm_part_step advances each partition once and puts every new state that
+ * another partition q references into q's own halo slots, so that no step
+ * reads another partition's memory; after n steps the stream is synchronised.
  * A node's arithmetic is the unpartitioned context's, in the same order, so
  * with the same kernel variant the results are bitwise equal to mlbm_init's.
  * Fields and populations are in the caller's order for all nodes (as
  * mlbm_set_fields / mlbm_get_populations); mlbm_part_permeability adds the
  * partitions' FP64 sums in partition order.  mlbm_part_info gives a
  * partition's first position, owned and halo counts and the bytes its halo
- * receives per step.  Starts at rest.  No CUDA graphs.
+ * receives per step.  Starts at rest.  Steps are replayed from captured graphs
+ * of 16.
  * Errors: as mlbm_init, MLBM_E_INVALID for bad bounds.
  */
 typedef struct mlbm_part mlbm_part;

@@ -112,18 +112,6 @@ __global__ void l2_flush_read(const float4* __restrict__ buf, size_t n, float* s
     if (acc != 0.f) *sink = acc;  // never taken on the zeroed buffer; keeps the loads
 }
 
-// Sending side of a halo copy: the states of the listed positions into one
-// contiguous block, w float4 per node (out[i*w + c] = in[list[i]*w + c]).
-__global__ void gather_states(const float4* __restrict__ in, const int* __restrict__ list, int64_t m, int w,
-                              float4* __restrict__ out) {
-    const int64_t total = m * w;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t node = i / w;
-        const int c = (int)(i - node * w);
-        out[i] = in[(size_t)list[node] * w + c];
-    }
-}
-
 namespace {
 
 #define MLBM_CUDA(call)                                                                                      \
@@ -1580,38 +1568,55 @@ mlbm_status mlbm_reduce_fields_device(const float* rho, const float* ux, const f
 
 // ------------------------------------------------------ partitioned step
 // P logical partitions of one node set, each a context over a contiguous
-// range of the device positions with halo slots after its own nodes.  After
-// every step each partition's new states of the nodes that another
-// partition references are packed (on the owner) and copied into that
-// partition's own halo slots, so every step reads local memory only.  All
-// partitions live on the current device and run on one stream, in order.
+// range of the device positions with halo slots after its own nodes.  In a
+// step every partition reads its own buffers only, and the new states of the
+// nodes that another partition references go into that partition's halo slots
+// of the buffer being written.  With kernel variants 27..29 all partitions
+// step in one launch whose threads store those states themselves; with any
+// other variant each partition is launched in turn and one kernel then copies
+// the states.  Steps are replayed from captured graphs of kGraphSteps.  (Four
+// partitions of 96k nodes, tau = 1: 110 us a step with a launch per partition
+// and a packing kernel and a copy per pair of partitions, 9.5 us now.)
 }  // extern "C"
 
 struct mlbm_part {
     int P = 0;
     int model = 0;
+    int64_t n = 0;
     double box_area = 1.0;
     std::vector<mlbm_ctx*> ctx;
-    std::vector<std::vector<int64_t>> caller_ids;  // [P][n_owned]: the caller's node id of each local position
     std::vector<int64_t> first, n_owned, n_halo;
-    struct Block {
-        int q, o;           // receiver, owner
-        int64_t count;      // nodes
-        int64_t halo_off;   // first halo slot of the block in q
-        int* list;          // device: positions local to o
-        float4* buf;        // device: packed states
-    };
-    std::vector<Block> blocks;
+    // device: the partitions, the step's blocks as (partition, range), the
+    // halo entries (owner, position, receiver, slot), the FP64 I/O array of
+    // all nodes in the caller's order, and the partitions' error words
+    dev::PartDev* parts = nullptr;
+    int2* work = nullptr;
+    int blocks = 0;
+    int4* halo = nullptr;
+    int64_t n_copies = 0;
+    double* io = nullptr;
+    int* err = nullptr;
     cudaStream_t stream = nullptr;
+    cudaGraphExec_t graph[2] = {nullptr, nullptr};  // kGraphSteps steps from buffer 0 / 1
+    int graph_variant = -1;
     std::vector<void*> allocations;
     int64_t steps = 0;
 };
 
 namespace {
 
+void drop_part_graphs(mlbm_part* P) {
+    for (cudaGraphExec_t& g : P->graph) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+    }
+    P->graph_variant = -1;
+}
+
 void free_part(mlbm_part* P) {
     if (!P) return;
     if (P->stream) cudaStreamSynchronize(P->stream);
+    drop_part_graphs(P);
     for (mlbm_ctx* c : P->ctx) free_ctx(c);
     for (void* q : P->allocations) cudaFree(q);
     if (P->stream) cudaStreamDestroy(P->stream);
@@ -1620,18 +1625,66 @@ void free_part(mlbm_part* P) {
 
 int state_width(const mlbm_part* P) { return P->model == MLBM_MODEL_BGK ? 2 : 1; }
 
-float4* state_of(mlbm_ctx* c) { return c->f8[c->cur] ? c->f8[c->cur] : c->ruv[c->cur]; }
+template <class T>
+mlbm_status part_upload(mlbm_part* P, T** dst, const std::vector<T>& src) {
+    void* d = nullptr;
+    if (cudaMalloc(&d, std::max<size_t>(src.size(), 1) * sizeof(T)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return set_error(MLBM_E_OOM, "part_init: cudaMalloc");
+    }
+    P->allocations.push_back(d);
+    *dst = static_cast<T*>(d);
+    MLBM_CUDA(cudaMemcpyAsync(d, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, P->stream));
+    MLBM_CUDA(cudaStreamSynchronize(P->stream));
+    return MLBM_OK;
+}
 
 // fill every partition's halo slots from the owners' current states
 mlbm_status exchange(mlbm_part* P) {
-    const int w = state_width(P);
-    for (const mlbm_part::Block& b : P->blocks) {
-        const int grid = (int)std::min<int64_t>(4 * 152, (b.count * w + 255) / 256);
-        gather_states<<<std::max(grid, 1), 256, 0, P->stream>>>(state_of(P->ctx[b.o]), b.list, b.count, w, b.buf);
-        MLBM_CUDA(cudaGetLastError());
-        float4* dst = state_of(P->ctx[b.q]) + (size_t)(P->n_owned[b.q] + b.halo_off) * w;
-        MLBM_CUDA(cudaMemcpyAsync(dst, b.buf, (size_t)b.count * w * sizeof(float4), cudaMemcpyDeviceToDevice,
-                                  P->stream));
+    MLBM_CUDA(launch_exchange(P->parts, P->halo, P->n_copies, state_width(P), P->ctx[0]->cur, P->stream));
+    return MLBM_OK;
+}
+
+mlbm_status part_sync(mlbm_part* P) {
+    std::vector<int> e(P->P, 0);
+    MLBM_CUDA(cudaMemcpyAsync(e.data(), P->err, e.size() * sizeof(int), cudaMemcpyDeviceToHost, P->stream));
+    MLBM_CUDA(cudaStreamSynchronize(P->stream));
+    for (mlbm_ctx* c : P->ctx)
+        if (e[(size_t)(c->err - P->err)] != 0) return sync(c);  // clears the word and reports it
+    return MLBM_OK;
+}
+
+// one step of every partition on the stream
+mlbm_status part_launch_step(mlbm_part* P) {
+    mlbm_ctx* c0 = P->ctx[0];
+    if (c0->variant >= 27 && c0->variant <= 29 && c0->S.rec) {
+        const dev::Wait W{c0->wait_ns, 0};
+        MLBM_CUDA(launch_step_parts(P->model == MLBM_MODEL_BGK ? 0 : 1, c0->S.Kq, P->n, P->parts, P->work, P->blocks,
+                                    c0->cur, P->err, W, P->stream));
+        for (mlbm_ctx* c : P->ctx) c->cur ^= 1;
+        return MLBM_OK;
+    }
+    for (mlbm_ctx* c : P->ctx) MLBM_TRY(launch_one_step(c, c->variant));
+    return exchange(P);
+}
+
+// instantiate the graph of kGraphSteps steps from buffer `parity`
+mlbm_status part_graph(mlbm_part* P, int parity) {
+    if (P->graph[parity]) return MLBM_OK;
+    cudaGraph_t g = nullptr;
+    const int cur = P->ctx[0]->cur;
+    MLBM_CUDA(cudaStreamBeginCapture(P->stream, cudaStreamCaptureModeThreadLocal));
+    for (mlbm_ctx* c : P->ctx) c->cur = parity;
+    mlbm_status s = MLBM_OK;
+    for (int i = 0; i < kGraphSteps && s == MLBM_OK; ++i) s = part_launch_step(P);
+    cudaError_t e = cudaStreamEndCapture(P->stream, &g);
+    for (mlbm_ctx* c : P->ctx) c->cur = cur;
+    if (s == MLBM_OK && e == cudaSuccess) e = cudaGraphInstantiate(&P->graph[parity], g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (s != MLBM_OK) return s;
+    if (e != cudaSuccess) {
+        P->graph[parity] = nullptr;
+        return set_error(MLBM_E_CUDA, std::string("part_step: graph: ") + cudaGetErrorString(e));
     }
     return MLBM_OK;
 }
@@ -1658,6 +1711,7 @@ mlbm_status mlbm_part_init(mlbm_part** out, const mlbm_stencils* st, const mlbm_
     if (!P) return set_error(MLBM_E_OOM, "part_init: out of host memory");
     P->P = n_parts;
     P->model = p->model;
+    P->n = st->h.n;
     P->box_area = st->h.box_area;
     auto fail = [&](mlbm_status s) {
         std::string msg = g_last_error;
@@ -1685,34 +1739,75 @@ mlbm_status mlbm_part_init(mlbm_part** out, const mlbm_stencils* st, const mlbm_
         P->first.push_back(a);
         P->n_owned.push_back(e - a);
         P->n_halo.push_back((int64_t)plan.halo[q].size());
-        P->caller_ids.emplace_back(st->h.perm.begin() + a, st->h.perm.begin() + e);
+        // I/O goes through one array of all nodes in the caller's order
+        std::vector<int> ids((size_t)c->n_pad, 0);
+        for (int64_t i = a; i < e; ++i) ids[(size_t)(i - a)] = (int)st->h.perm[i];
+        if (cudaMemcpyAsync(c->perm, ids.data(), ids.size() * sizeof(int), cudaMemcpyHostToDevice, P->stream) !=
+                cudaSuccess ||
+            cudaStreamSynchronize(P->stream) != cudaSuccess)
+            return fail(set_error(MLBM_E_CUDA, "part_init: upload"));
     }
-    const int w = p->model == MLBM_MODEL_BGK ? 2 : 1;
+    // halo copies, and per owner the slots each of its nodes is sent to
+    std::vector<int4> halo;
+    std::vector<std::vector<std::pair<int, int2>>> sends(n_parts);
     for (int q = 0; q < n_parts; ++q)
-        for (int o = 0; o < n_parts; ++o) {
-            const int64_t h0 = plan.halo_off[q][o], h1 = plan.halo_off[q][o + 1];
-            if (h1 == h0) continue;
-            std::vector<int> list((size_t)(h1 - h0));
-            for (int64_t i = h0; i < h1; ++i) list[(size_t)(i - h0)] = (int)(plan.halo[q][(size_t)i] - plan.bounds[o]);
-            mlbm_part::Block b{q, o, h1 - h0, h0, nullptr, nullptr};
-            void* d = nullptr;
-            if (cudaMalloc(&d, list.size() * sizeof(int)) != cudaSuccess)
-                return fail(set_error(MLBM_E_OOM, "part_init: cudaMalloc"));
-            P->allocations.push_back(d);
-            b.list = static_cast<int*>(d);
-            if (cudaMalloc(&d, (size_t)b.count * w * sizeof(float4)) != cudaSuccess)
-                return fail(set_error(MLBM_E_OOM, "part_init: cudaMalloc"));
-            P->allocations.push_back(d);
-            b.buf = static_cast<float4*>(d);
-            if (cudaMemcpyAsync(b.list, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice, P->stream) !=
-                cudaSuccess)
-                return fail(set_error(MLBM_E_CUDA, "part_init: upload"));
-            if (cudaStreamSynchronize(P->stream) != cudaSuccess)
-                return fail(set_error(MLBM_E_CUDA, "part_init: upload"));
-            P->blocks.push_back(b);
+        for (int o = 0; o < n_parts; ++o)
+            for (int64_t i = plan.halo_off[q][o]; i < plan.halo_off[q][o + 1]; ++i) {
+                const int pos = (int)(plan.halo[q][(size_t)i] - plan.bounds[o]), slot = (int)(P->n_owned[q] + i);
+                halo.push_back(make_int4(o, pos, q, slot));
+                sends[o].push_back({pos, make_int2(q, slot)});
+            }
+    P->n_copies = (int64_t)halo.size();
+    mlbm_status us = part_upload(P, &P->halo, halo);
+    if (us == MLBM_OK) us = part_upload(P, &P->io, std::vector<double>(9 * (size_t)P->n));
+    if (us == MLBM_OK) us = part_upload(P, &P->err, std::vector<int>(n_parts, 0));
+    if (us != MLBM_OK) return fail(us);
+    // the step's blocks, shared out by node count
+    const int sms = warp_step_ranges(1 << 30);
+    std::vector<dev::PartDev> dev_parts(n_parts);
+    std::vector<int2> work;
+    for (int q = 0; q < n_parts; ++q) {
+        mlbm_ctx* c = P->ctx[q];
+        c->err = P->err + q;
+        std::stable_sort(sends[q].begin(), sends[q].end(),
+                         [](const auto& x, const auto& y) { return x.first < y.first; });
+        std::vector<int> send_first((size_t)c->n + 1, 0);
+        std::vector<int2> to;
+        for (const auto& e : sends[q]) {
+            ++send_first[(size_t)e.first + 1];
+            to.push_back(e.second);
         }
+        for (int64_t i = 0; i < c->n; ++i) send_first[(size_t)i + 1] += send_first[(size_t)i];
+        dev::PartDev& D = dev_parts[q];
+        int* d_first = nullptr;
+        int2* d_to = nullptr;
+        us = part_upload(P, &d_first, send_first);
+        if (us == MLBM_OK) us = part_upload(P, &d_to, to);
+        if (us != MLBM_OK) return fail(us);
+        const int64_t lo = sms * P->first[q] / P->n, hi = sms * (P->first[q] + P->n_owned[q]) / P->n;
+        c->S.n_ranges = (int)std::max<int64_t>(1, std::min<int64_t>({hi - lo, (c->n + 31) / 32, c->S.n_ranges}));
+        for (int r = 0; r < c->S.n_ranges; ++r) work.push_back(make_int2(q, r));
+        cudaError_t e = launch_mark_sends((int)c->n, d_first, c->meta, P->stream);
+        if (e == cudaSuccess) e = launch_record_kinds(c->S, c->rec, c->need, c->range, P->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(P->stream);
+        if (e != cudaSuccess) return fail(set_error(MLBM_E_CUDA, "part_init: kinds"));
+        D.S = c->S;
+        D.C = c->C;
+        for (int b = 0; b < 2; ++b) {
+            D.state[b] = c->f8[b] ? c->f8[b] : c->ruv[b];
+            D.f0[b] = c->f0[b];
+        }
+        D.send_first = d_first;
+        D.sends = d_to;
+    }
+    P->blocks = (int)work.size();
+    us = part_upload(P, &P->parts, dev_parts);
+    if (us == MLBM_OK) us = part_upload(P, &P->work, work);
+    if (us != MLBM_OK) return fail(us);
     mlbm_status s = exchange(P);
-    if (s == MLBM_OK) s = sync(P->ctx[0]);
+    if (s == MLBM_OK) s = part_sync(P);
+    P->graph_variant = P->ctx[0]->variant;
+    for (int parity = 0; parity < 2 && s == MLBM_OK; ++parity) s = part_graph(P, parity);
     if (s != MLBM_OK) return fail(s);
     *out = P;
     return MLBM_OK;
@@ -1739,43 +1834,46 @@ mlbm_status mlbm_part_set_kernel_variant(mlbm_part* P, int variant) {
 mlbm_status mlbm_part_step(mlbm_part* P, int64_t n_steps) {
     if (!P) return set_error(MLBM_E_INVALID, "part_step: NULL");
     if (n_steps < 0) return set_error(MLBM_E_INVALID, "part_step: negative step count");
-    for (int64_t t = 0; t < n_steps; ++t) {
-        for (mlbm_ctx* c : P->ctx) {
-            MLBM_TRY(launch_one_step(c, c->variant));
-            ++c->steps;
+    int64_t left = n_steps;
+    if (n_steps >= kGraphSteps) {
+        if (P->graph_variant != P->ctx[0]->variant) {
+            drop_part_graphs(P);
+            P->graph_variant = P->ctx[0]->variant;
         }
-        MLBM_TRY(exchange(P));
-        ++P->steps;
+        for (; left >= kGraphSteps; left -= kGraphSteps) {
+            MLBM_TRY(part_graph(P, P->ctx[0]->cur));
+            MLBM_CUDA(cudaGraphLaunch(P->graph[P->ctx[0]->cur], P->stream));
+        }
     }
-    for (mlbm_ctx* c : P->ctx) MLBM_TRY(sync(c));  // also reports a bounded wait that ran out
-    return MLBM_OK;
+    for (; left > 0; --left) MLBM_TRY(part_launch_step(P));
+    for (mlbm_ctx* c : P->ctx) c->steps += n_steps;
+    P->steps += n_steps;
+    return part_sync(P);  // also reports a bounded wait that ran out
 }
 
 // fields or populations in the caller's order for all nodes; `width` values per node
 static mlbm_status part_set(mlbm_part* P, const double* v, int width, bool fields) {
-    std::vector<double> loc;
-    for (int q = 0; q < P->P; ++q) {
-        const std::vector<int64_t>& ids = P->caller_ids[q];
-        loc.assign(ids.size() * width, 0.0);
-        for (size_t p = 0; p < ids.size(); ++p)
-            for (int k = 0; k < width; ++k) loc[p * width + k] = v[(size_t)ids[p] * width + k];
-        MLBM_TRY(fields ? mlbm_set_fields(P->ctx[q], loc.data()) : mlbm_set_populations(P->ctx[q], loc.data()));
+    MLBM_CUDA(cudaMemcpyAsync(P->io, v, (size_t)P->n * width * 8, cudaMemcpyHostToDevice, P->stream));
+    for (mlbm_ctx* c : P->ctx) {
+        const int n = (int)c->n, b = c->cur;
+        if (!fields) MLBM_CUDA(launch_set_bgk(n, c->perm, P->io, c->f8[b], c->f0[b], P->stream));
+        else if (P->model == MLBM_MODEL_BGK)
+            MLBM_CUDA(launch_set_bgk_equilibrium(n, c->perm, P->io, c->f8[b], c->f0[b], P->stream));
+        else MLBM_CUDA(launch_set_tau1(n, c->perm, P->io, c->ruv[b], P->stream));
+        c->steps = 0;
     }
     MLBM_TRY(exchange(P));
     P->steps = 0;
-    return sync(P->ctx[0]);
+    return part_sync(P);
 }
 
 static mlbm_status part_get(mlbm_part* P, double* v, int width, bool fields) {
-    std::vector<double> loc;
-    for (int q = 0; q < P->P; ++q) {
-        const std::vector<int64_t>& ids = P->caller_ids[q];
-        loc.assign(ids.size() * width, 0.0);
-        MLBM_TRY(fields ? mlbm_get_fields(P->ctx[q], loc.data()) : mlbm_get_populations(P->ctx[q], loc.data()));
-        for (size_t p = 0; p < ids.size(); ++p)
-            for (int k = 0; k < width; ++k) v[(size_t)ids[p] * width + k] = loc[p * width + k];
+    for (mlbm_ctx* c : P->ctx) {
+        if (fields) MLBM_TRY(fields_to_work(c, P->io));
+        else MLBM_CUDA(launch_get_bgk((int)c->n, c->perm, c->f8[c->cur], c->f0[c->cur], P->io, P->stream));
     }
-    return MLBM_OK;
+    MLBM_CUDA(cudaMemcpyAsync(v, P->io, (size_t)P->n * width * 8, cudaMemcpyDeviceToHost, P->stream));
+    return part_sync(P);
 }
 
 mlbm_status mlbm_part_set_fields(mlbm_part* P, const double* ru) {

@@ -10,7 +10,8 @@
 //                                int4 (Lagrange nodes: slots 0..8 hold the 3x3
 //                                block, row b outer, column a inner)
 //   meta uint8  [n_pad]          bits 0-1 kind (0 WLS, 1 Lagrange, 2 equilibrium),
-//                                bit 2 has bounce-back links, bits 4-7 block centre
+//                                bit 2 has bounce-back links, bit 3 the node's state
+//                                is sent to another partition, bits 4-7 block centre
 //   lag_r float [n_pad]          s / h of the Lagrange block
 //   link_slot int [n_pad], links LinkRec[]  bounce-back links of a node
 //   eqv  float4 [n_pad]          (rho_b - 1, ux_b, uy_b, 0) of equilibrium nodes
@@ -110,6 +111,19 @@ __device__ __forceinline__ const float4* rec_lane(const Stencil& S, int p) {
 struct Wait {
     unsigned long long budget_ns;
     int withhold;
+};
+
+// One partition of a partitioned node set on the device: its stencils, its two
+// state buffers (halo slots after its own nodes), and for its nodes that other
+// partitions reference (bit 3 of the kind byte) where their new states go:
+// sends[send_first[p] .. send_first[p + 1]) = (partition, slot).
+struct PartDev {
+    Stencil S;
+    Collide C;
+    float4* state[2];
+    float* f0[2];
+    const int* send_first;
+    const int2* sends;
 };
 
 constexpr int kStageTile = 256;   // nodes per staged tile (one block)

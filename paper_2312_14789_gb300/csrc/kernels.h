@@ -47,6 +47,14 @@ cudaError_t launch_freeze_tau1(int first, int m, uint8_t* meta, float4* eqv, con
 cudaError_t launch_record_kinds(const dev::Stencil& S, float4* rec, uint8_t* need, int* range, cudaStream_t st);
 // blocks (and tile ranges) of the per-warp-slot step for n nodes
 int warp_step_ranges(int n);
+// one step of every partition (variants 27..29): the partitions' ranges in one
+// launch, new halo states stored straight into the receivers' slots
+cudaError_t launch_step_parts(int model, int Kq, int64_t n, const dev::PartDev* parts, const int2* work, int blocks,
+                              int from, int* err, const dev::Wait& W, cudaStream_t st);
+cudaError_t launch_mark_sends(int n, const int* send_first, uint8_t* meta, cudaStream_t st);
+// halo slots of all partitions from their owners' states in buffer `cur`, w
+// float4 a state
+cudaError_t launch_exchange(const dev::PartDev* parts, const int4* list, int64_t m, int w, int cur, cudaStream_t st);
 // step kernels with a shared-memory slot per warp (kernels_warp.cu), variants
 // 27..29; backward walks the tiles from the last one where that is of use
 cudaError_t launch_step_warp(int variant, int model, const dev::Stencil& S, const float4* a8, const float* a0,

@@ -124,10 +124,31 @@ __device__ __forceinline__ void wls_increments(const float4* __restrict__ f8in, 
     }
 }
 
-template <int KQ, int MODEL, int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, 1)
-    step_warp(Stencil S, const float4* __restrict__ in, const float* __restrict__ f0in, float4* __restrict__ out,
-              float* __restrict__ f0out, Collide C0, int backward, int* __restrict__ err, const Wait W) {
+// the new state of a node that other partitions reference, into their halo slots
+__device__ __forceinline__ void send_state(const PartDev* parts, const PartDev& own, int parity, int p, const float4& a,
+                                           const float4* b) {
+    const int e1 = own.send_first[p + 1];
+    for (int e = own.send_first[p]; e < e1; ++e) {
+        const int2 to = own.sends[e];
+        float4* dst = parts[to.x].state[parity];
+        if (b) {
+            dst[2 * (size_t)to.y] = a;
+            dst[2 * (size_t)to.y + 1] = *b;
+        } else {
+            dst[to.y] = a;
+        }
+    }
+}
+
+// One block's walk over range `rb` of the tiles.  PART: a partition of a
+// partitioned set (own, one of parts), whose new states go to buffer `parity`
+// of the partitions that hold them as halo.
+template <int KQ, int MODEL, int WARPS, bool PART>
+__device__ __forceinline__ void walk_tiles(const Stencil& S, const float4* __restrict__ in,
+                                           const float* __restrict__ f0in, float4* __restrict__ out,
+                                           float* __restrict__ f0out, const Collide& C0, int rb, int backward,
+                                           int* __restrict__ err, const Wait& W, const PartDev* parts,
+                                           const PartDev* own, int parity) {
     using L = WarpTile<KQ, WARPS>;
     using R = TileRec<KQ>;
     extern __shared__ __align__(128) uint8_t smem[];
@@ -136,7 +157,7 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
     uint8_t* slot = smem + warp * L::kBytes;
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::kWarps * L::kBytes) + 2 * warp;
     const float4* base = reinterpret_cast<const float4*>(slot) + lane;
-    const int t0 = S.range[blockIdx.x], t1 = S.range[blockIdx.x + 1];
+    const int t0 = S.range[rb], t1 = S.range[rb + 1];
     if (warp >= t1 - t0) return;
     int t = backward ? t1 - 1 - warp : t0 + warp;
     const int hop = backward ? -L::kWarps : L::kWarps;
@@ -287,6 +308,10 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
                 out[2 * (size_t)p] = make_float4(g[1], g[2], g[3], g[4]);
                 out[2 * (size_t)p + 1] = make_float4(g[5], g[6], g[7], g[8]);
                 f0out[p] = g[0];
+                if (PART && (meta & 8)) {
+                    const float4 hi = make_float4(g[5], g[6], g[7], g[8]);
+                    send_state(parts, *own, parity, p, make_float4(g[1], g[2], g[3], g[4]), &hi);
+                }
             }
         } else {
             float4 me = make_float4(0, 0, 0, 0);
@@ -333,7 +358,10 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
                 return;
             }
             if (kind == 2) {
-                if (p < S.n) out[p] = S.eqv[p];
+                if (p < S.n) {
+                    out[p] = S.eqv[p];
+                    if (PART && (meta & 8)) send_state(parts, *own, parity, p, S.eqv[p], nullptr);
+                }
             } else {
                 float r = 0.f, cx = 0.f, cy = 0.f;
                 if (kind == 0) {
@@ -354,9 +382,52 @@ __global__ void __launch_bounds__(WARPS * 32, 1)
                     cy = (float)ey_of(meta >> 4);
                 }
                 const float4 o = tau1_finish(S, C, me, kind, c, v9, r, cx, cy, (meta & 4) != 0, p);
-                if (p < S.n) out[p] = o;
+                if (p < S.n) {
+                    out[p] = o;
+                    if (PART && (meta & 8)) send_state(parts, *own, parity, p, o, nullptr);
+                }
             }
         }
+    }
+}
+
+template <int KQ, int MODEL, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 1)
+    step_warp(Stencil S, const float4* __restrict__ in, const float* __restrict__ f0in, float4* __restrict__ out,
+              float* __restrict__ f0out, Collide C0, int backward, int* __restrict__ err, const Wait W) {
+    walk_tiles<KQ, MODEL, WARPS, false>(S, in, f0in, out, f0out, C0, blockIdx.x, backward, err, W, nullptr, nullptr,
+                                        0);
+}
+
+// All partitions of a partitioned set in one launch: block b walks range
+// work[b].y of partition work[b].x, from buffer `from` into the other one.
+template <int KQ, int MODEL, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, 1)
+    step_parts(const PartDev* __restrict__ parts, const int2* __restrict__ work, int from, int backward,
+               int* __restrict__ err, const Wait W) {
+    const int2 job = work[blockIdx.x];
+    const PartDev* own = parts + job.x;
+    const Stencil S = own->S;
+    const Collide C0 = own->C;
+    walk_tiles<KQ, MODEL, WARPS, true>(S, own->state[from], own->f0[from], own->state[from ^ 1], own->f0[from ^ 1], C0,
+                                       job.y, backward, err, W, parts, own, from ^ 1);
+}
+
+// bit 3 of the kind bytes (and the records' copies) of nodes whose states are sent
+__global__ void mark_sends(int n, const int* __restrict__ send_first, uint8_t* __restrict__ meta) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < n && send_first[p + 1] > send_first[p]) meta[p] |= 8;
+}
+
+// Halo copies of all partitions, w float4 a state: entry (owner, its position,
+// receiver, its slot).
+__global__ void exchange_states(const PartDev* __restrict__ parts, const int4* __restrict__ list, int64_t m, int w,
+                                int cur) {
+    const int64_t total = m * w;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int4 e = list[i / w];
+        const size_t c = (size_t)(i % w);
+        parts[e.z].state[cur][(size_t)e.w * w + c] = parts[e.x].state[cur][(size_t)e.y * w + c];
     }
 }
 
@@ -412,6 +483,13 @@ __global__ void __launch_bounds__(1024) tile_ranges(int n_tiles, const uint8_t* 
 
 namespace {
 
+// Bytes of records above which steps walk back over what the last one left in
+// L2.  Below ~100 MB everything stays there and the order is worth nothing
+// (192k nodes, 83 MB: 14.3 us forwards, 14.6 in turn); above it every step
+// saves what L2 holds (260k nodes, 112 MB: 22.9 -> 20.4 us; 420k tau = 1: 33.0
+// -> 30.1 us; 1.73M: 122.9 -> 120.1 us).
+constexpr size_t kResident = size_t(100) << 20;
+
 template <int KQ, int MODEL, int WARPS>
 cudaError_t run_warp(const dev::Stencil& S, const float4* in, const float* f0in, float4* out, float* f0out,
                      const dev::Collide& C, int backward, int* err, const dev::Wait& W, cudaStream_t st) {
@@ -420,12 +498,6 @@ cudaError_t run_warp(const dev::Stencil& S, const float4* in, const float* f0in,
     auto fn = dev::step_warp<KQ, MODEL, WARPS>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kSmem);
     if (e != cudaSuccess) return e;
-    // walk back only over what the last step left in L2: below ~100 MB of
-    // records everything stays there and the order is worth nothing (192k
-    // nodes, 83 MB: 14.3 us forwards, 14.6 in turn); above it every step saves
-    // what L2 holds (260k nodes, 112 MB: 22.9 -> 20.4 us; 420k tau = 1: 33.0
-    // -> 30.1 us; 1.73M: 122.9 -> 120.1 us)
-    constexpr size_t kResident = size_t(100) << 20;
     const int back = (size_t)((S.n + 31) / 32) * L::kBytes > kResident ? backward : 0;
     return launch_pdl_smem(fn, S.n_ranges, WARPS * 32, L::kSmem, st, S, in, f0in, out, f0out, C, back, err, W);
 }
@@ -465,6 +537,41 @@ cudaError_t launch_step_warp(int variant, int model, const dev::Stencil& S, cons
         case 8: return run_warp_variant<8, 8, 6, 7>(variant, model, S, a8, a0, b8, b0, ra, rb, C, backward, err, W, st);
         default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_step_parts(int model, int Kq, int64_t n, const dev::PartDev* parts, const int2* work, int blocks,
+                              int from, int* err, const dev::Wait& W, cudaStream_t st) {
+    const int back = (size_t)(n / 32) * (7 * Kq - 1) * 512 > kResident ? from : 0;
+    auto run = [&](auto fn, int warps, size_t smem) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        return launch_pdl_smem(fn, blocks, warps * 32, smem, st, parts, work, from, back, err, W);
+    };
+#define MLBM_PARTS(KQ, WARPS)                                                                              \
+    case KQ:                                                                                               \
+        return model == 0 ? run(dev::step_parts<KQ, 0, WARPS>, WARPS, dev::WarpTile<KQ, WARPS>::kSmem)     \
+                          : run(dev::step_parts<KQ, 1, WARPS>, WARPS, dev::WarpTile<KQ, WARPS>::kSmem);
+    switch (Kq) {
+        MLBM_PARTS(3, 12)
+        MLBM_PARTS(4, 12)
+        MLBM_PARTS(6, 10)
+        MLBM_PARTS(8, 8)
+        default: return cudaErrorInvalidValue;
+    }
+#undef MLBM_PARTS
+}
+
+cudaError_t launch_mark_sends(int n, const int* send_first, uint8_t* meta, cudaStream_t st) {
+    if (n == 0) return cudaSuccess;
+    dev::mark_sends<<<(n + 255) / 256, 256, 0, st>>>(n, send_first, meta);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_exchange(const dev::PartDev* parts, const int4* list, int64_t m, int w, int cur, cudaStream_t st) {
+    if (m == 0) return cudaSuccess;
+    const int grid = (int)std::min<int64_t>(8 * 152, (m * w + 255) / 256);
+    dev::exchange_states<<<grid, 256, 0, st>>>(parts, list, m, w, cur);
+    return cudaGetLastError();
 }
 
 int warp_step_ranges(int n) {

@@ -111,3 +111,24 @@ def test_mixed_kinds_over_the_ranges(M):
         M.step(ctx, 6)
         out[v] = M.get_populations(ctx)
     assert np.abs(out[27] - out[0]).max() < 6 * 3e-7
+
+
+@pytest.mark.parametrize("n_parts", [1, 7, 40])
+@pytest.mark.parametrize("model", ["bgk", "tau1"])
+def test_partitions_in_one_launch(M, n_parts, model):
+    """All ranges in one launch that stores the halo states itself: bitwise the
+    unpartitioned step over graph replays and single steps, for more ranges
+    than a small set has tiles per range, and after changing the variant."""
+    w = I.porous(seed=8, n_target=3000)
+    st = M.build_stencils_for(w, K=16, s=1.0)
+    p = M.Params(M.MODEL_BGK, 0.8, 0.0, 1e-6, 0.0) if model == "bgk" else M.Params(M.MODEL_TAU1, 1.0, 0.0, 1e-6, 0.0)
+    ref, part = M.init(st, p), M.Partitioned(st, p, n_parts)
+    for n, v in ((1, 27), (35, 27), (17, 11), (16, 29)):
+        M.set_kernel_variant(ref, v)
+        part.set_kernel_variant(v)
+        if v == 27:
+            M.set_fields(ref, _start(w))
+            part.set_fields(_start(w))
+        M.step(ref, n)
+        part.step(n)
+        assert np.array_equal(part.get_fields(), M.get_fields(ref)), (n, v)
