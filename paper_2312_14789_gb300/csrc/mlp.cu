@@ -3,21 +3,34 @@
 // kernels and Adam.
 //
 // Parameters are kept in FP32 ("master") in the packed order W1[16][64], b1,
-// W2[64][64], b2, W3[64][64], b3, W4[64][n_out], b4 (y = x W + b per layer); the
-// kernels convert the weights to BF16 in shared memory.  Rounding points:
-// the features and every hidden activation (after bias and ReLU) are rounded
-// to BF16 where they become an MMA operand; the output error and every hidden
-// error likewise.  Accumulation and biases are FP32.
+// W2[64][64], b2, W3[64][64], b3, W4[64][n_out], b4 (y = x W + b per layer).
+// Whoever writes a parameter also writes its BF16 copy in the network's weight
+// image ([out][in] rows, padded), so a block fetches all its weights with one
+// bulk copy; the transposed operands of the backward pass come from the same
+// rows through transposing fragment loads.  Rounding points: the features and
+// every hidden activation (after bias and ReLU) are rounded to BF16 where they
+// become an MMA operand; the output error and every hidden error likewise.
+// Accumulation and biases are FP32.
 //
 // Forward: one warp per 16-row tile; a layer's FP32 accumulator fragments are
 // re-packed in registers as the next layer's A fragments.
-// Gradients: blocks of 4 warps take 64-row chunks: each warp runs its 16 rows
-// forward and back through the layers (dX = dZ W^T), staging activations and
-// errors transposed ([feature][row], BF16) in shared memory; then the block
-// computes dW = H^T dZ for the chunk with MMAs whose K dimension is the 64
-// rows, each output tile owned by one warp (no atomics), and adds the bias
-// sums.  Each block writes its FP32 partial gradient; a second kernel adds
-// the partials in block order, so the result is reproducible run to run.
+// Gradients: blocks of 8 warps take up to 128 rows a round: each warp runs 16
+// rows forward and back through the layers (dX = dZ W^T), leaving activations
+// and errors in shared memory as [row][feature] BF16 pairs; then every warp
+// owns some output tiles of dW = H^T dZ and adds the round's rows to them in
+// registers (64 rows to an MMA chain, the chains added in FP32; no atomics),
+// while the bias columns are summed by the threads.  Each block writes its FP32
+// partial gradient once; the second kernel adds the partials in a fixed order
+// and, in training, takes the Adam step and refreshes the weight image, so the
+// result is reproducible run to run.
+//
+// What bounds a training step of 65,536 rows (3.7 GFLOP): the layer chain of a
+// 16-row tile is a few hundred dependent instructions, so the rate follows the
+// warps an SM runs side by side and what they do besides MMAs.  Four warps an
+// SM (143 KB of shared memory a block for two weight copies and gradient
+// accumulators), 2-byte transposed staging stores, dW accumulated in shared
+// memory, uncoalesced weight conversion in every block and 304 partials summed
+// one after the other took 133 us a step; this form takes 36 us.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -26,7 +39,10 @@
 #include <vector>
 
 #include "kernels.h"
+#include "launch_util.cuh"
 #include "mlbm_internal.h"
+#include "ring.cuh"
+#include "step_node.cuh"
 
 namespace mlbm {
 namespace mlp {
@@ -40,7 +56,7 @@ __host__ __device__ constexpr int off_b4(int no) { return oW4 + kH * no; }
 __host__ __device__ constexpr int param_count(int no) { return off_b4(no) + no; }
 static_assert(param_count(2) == 9538, "packing");
 
-// padded shared-memory strides (BF16 elements) that keep fragment loads free of bank conflicts
+// padded row strides (BF16 elements) that keep fragment loads free of bank conflicts
 constexpr int kS16 = 24, kS64 = 72;
 
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
@@ -57,35 +73,62 @@ __device__ __forceinline__ void mma(float* d, const uint32_t* a, uint32_t b0, ui
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Forward weights, transposed [out][in] BF16, padded strides; biases FP32.
-struct FwdSmem {
+// four 8x8 BF16 matrices (TRANS: transposed); lane i gives the address of row
+// i % 8 of matrix i / 8
+template <bool TRANS>
+__device__ __forceinline__ void ldsm4(uint32_t* r, const __nv_bfloat16* p) {
+    const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+
+// Weight image: [out][in] BF16 rows with padded strides (outputs padded to 8),
+// FP32 biases; padding is zero.
+struct __align__(16) Image {
     __nv_bfloat16 wt1[kH * kS16];
     __nv_bfloat16 wt2[kH * kS64];
     __nv_bfloat16 wt3[kH * kS64];
-    __nv_bfloat16 wt4[8 * kS64];  // outputs padded to 8
+    __nv_bfloat16 wt4[8 * kS64];
     float b1[kH], b2[kH], b3[kH], b4[8];
 };
+static_assert(sizeof(Image) % 16 == 0, "copied in bulk");
 
-__device__ void load_fwd(const float* __restrict__ P, int no, FwdSmem& s) {
-    for (int i = threadIdx.x; i < kH * kS16; i += blockDim.x) {
-        const int n = i / kS16, k = i % kS16;
-        s.wt1[i] = __float2bfloat16_rn(k < kIn ? P[oW1 + k * kH + n] : 0.f);
+// parameter i (packed order) into the image
+__device__ __forceinline__ void image_put(Image* I, int no, int i, float v) {
+    const __nv_bfloat16 w = __float2bfloat16_rn(v);
+    if (i < oB1) I->wt1[(i % kH) * kS16 + i / kH] = w;
+    else if (i < oW2) I->b1[i - oB1] = v;
+    else if (i < oB2) I->wt2[((i - oW2) % kH) * kS64 + (i - oW2) / kH] = w;
+    else if (i < oW3) I->b2[i - oB2] = v;
+    else if (i < oB3) I->wt3[((i - oW3) % kH) * kS64 + (i - oW3) / kH] = w;
+    else if (i < oW4) I->b3[i - oB3] = v;
+    else if (i < off_b4(no)) I->wt4[((i - oW4) % no) * kS64 + (i - oW4) / no] = w;
+    else I->b4[i - off_b4(no)] = v;
+}
+
+__global__ void refresh_image(int kp, int no, const float* __restrict__ P, Image* __restrict__ I) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < kp) image_put(I, no, i, P[i]);
+}
+
+// the image into the block's shared memory: started by one thread, awaited by
+// all.  The wait polls a copy this block issued itself; it gives up after two
+// seconds, as a lost copy would otherwise hold the GPU (the results are then
+// of whatever the memory held).
+__device__ __forceinline__ void fetch_image(Image* s, const Image* I, uint64_t* bar) {
+    if (threadIdx.x == 0) {
+        dev::mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async;" ::: "memory");  // the image was written by ordinary stores
+        dev::mbar_expect_tx(bar, sizeof(Image));
+        dev::bulk_g2s(s, I, sizeof(Image), bar);
     }
-    for (int i = threadIdx.x; i < kH * kS64; i += blockDim.x) {
-        const int n = i / kS64, k = i % kS64;
-        s.wt2[i] = __float2bfloat16_rn(k < kH ? P[oW2 + k * kH + n] : 0.f);
-        s.wt3[i] = __float2bfloat16_rn(k < kH ? P[oW3 + k * kH + n] : 0.f);
-    }
-    for (int i = threadIdx.x; i < 8 * kS64; i += blockDim.x) {
-        const int n = i / kS64, k = i % kS64;
-        s.wt4[i] = __float2bfloat16_rn((k < kH && n < no) ? P[oW4 + k * no + n] : 0.f);
-    }
-    for (int i = threadIdx.x; i < kH; i += blockDim.x) {
-        s.b1[i] = P[oB1 + i];
-        s.b2[i] = P[oB2 + i];
-        s.b3[i] = P[oB3 + i];
-    }
-    if (threadIdx.x < 8) s.b4[threadIdx.x] = (int)threadIdx.x < no ? P[off_b4(no) + threadIdx.x] : 0.f;
+    __syncthreads();
+    dev::mbar_wait(bar, 0, 2000000000ULL);
 }
 
 // Row of the data set that minibatch row r reads: r itself (seed 0), else a
@@ -125,48 +168,79 @@ __device__ __forceinline__ void load_x(const float* __restrict__ X, int64_t src0
 // next A fragments
 template <int KT>
 __device__ __forceinline__ void hidden_layer(const uint32_t (*a)[4], const __nv_bfloat16* wt, int stride,
-                                             const float* bias, int g, int t, uint32_t (*out)[4]) {
+                                             const float* bias, int lane, uint32_t (*out)[4]) {
+    const int t = lane & 3;
+    // row of an 8x8 matrix, and which half (KT = 1: which n-tile and half) of the k-tiles it belongs to
+    const __nv_bfloat16* row = wt + (lane & 7) * stride;
+    const int sel = lane >> 3;
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const float bl = bias[8 * nt + 2 * t], bh = bias[8 * nt + 2 * t + 1];
-        float d[4] = {bl, bh, bl, bh};
+    for (int np = 0; np < 4; ++np) {  // pairs of n-tiles
+        float d[2][4];
 #pragma unroll
-        for (int kt = 0; kt < KT; ++kt) {
-            const __nv_bfloat16* w = wt + (8 * nt + g) * stride + 16 * kt + 2 * t;
-            mma(d, a[kt], ld32(w), ld32(w + 8));
+        for (int j = 0; j < 2; ++j) {
+            const float2 bb = *reinterpret_cast<const float2*>(bias + 16 * np + 8 * j + 2 * t);
+            d[j][0] = bb.x; d[j][1] = bb.y; d[j][2] = bb.x; d[j][3] = bb.y;
         }
-        const float r0 = fmaxf(d[0], 0.f), r1 = fmaxf(d[1], 0.f), r2 = fmaxf(d[2], 0.f), r3 = fmaxf(d[3], 0.f);
-        out[nt >> 1][(nt & 1) * 2 + 0] = pack2(r0, r1);
-        out[nt >> 1][(nt & 1) * 2 + 1] = pack2(r2, r3);
-    }
-}
-
-__device__ __forceinline__ void output_layer(const uint32_t (*a)[4], const FwdSmem& s, int g, int t, float* d) {
-    const float bl = s.b4[2 * t], bh = s.b4[2 * t + 1];
-    d[0] = bl; d[1] = bh; d[2] = bl; d[3] = bh;
+        if (KT == 1) {
+            uint32_t b[4];  // n-tile 0 halves, n-tile 1 halves
+            ldsm4<false>(b, row + (16 * np + 8 * (sel >> 1)) * stride + 8 * (sel & 1));
+            mma(d[0], a[0], b[0], b[1]);
+            mma(d[1], a[0], b[2], b[3]);
+        } else {
 #pragma unroll
-    for (int kt = 0; kt < 4; ++kt) {
-        const __nv_bfloat16* w = s.wt4 + g * kS64 + 16 * kt + 2 * t;
-        mma(d, a[kt], ld32(w), ld32(w + 8));
+            for (int kp = 0; kp < KT / 2; ++kp) {
+                uint32_t b0[4], b1[4];  // k-tile 2 kp halves, k-tile 2 kp + 1 halves
+                ldsm4<false>(b0, row + 16 * np * stride + 32 * kp + 8 * sel);
+                ldsm4<false>(b1, row + (16 * np + 8) * stride + 32 * kp + 8 * sel);
+                mma(d[0], a[2 * kp], b0[0], b0[1]);
+                mma(d[1], a[2 * kp], b1[0], b1[1]);
+                mma(d[0], a[2 * kp + 1], b0[2], b0[3]);
+                mma(d[1], a[2 * kp + 1], b1[2], b1[3]);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            out[np][2 * j] = pack2(fmaxf(d[j][0], 0.f), fmaxf(d[j][1], 0.f));
+            out[np][2 * j + 1] = pack2(fmaxf(d[j][2], 0.f), fmaxf(d[j][3], 0.f));
+        }
     }
 }
 
-__global__ void __launch_bounds__(128) forward_kernel(const float* __restrict__ P, const float* __restrict__ X,
-                                                      int64_t n, int no, float* __restrict__ Y) {
-    __shared__ FwdSmem s;
-    load_fwd(P, no, s);
-    __syncthreads();
+__device__ __forceinline__ void output_layer(const uint32_t (*a)[4], const Image& s, int lane, float* d) {
+    const int t = lane & 3;
+    const float2 bb = *reinterpret_cast<const float2*>(s.b4 + 2 * t);
+    d[0] = bb.x; d[1] = bb.y; d[2] = bb.x; d[3] = bb.y;
+#pragma unroll
+    for (int kp = 0; kp < 2; ++kp) {
+        uint32_t b[4];
+        ldsm4<false>(b, s.wt4 + (lane & 7) * kS64 + 32 * kp + 8 * (lane >> 3));
+        mma(d, a[2 * kp], b[0], b[1]);
+        mma(d, a[2 * kp + 1], b[2], b[3]);
+    }
+}
+
+// Inference is bound by the layer chain as well (a 16-row tile is 76 MMAs in
+// four dependent layers; the rows are 2 MB of traffic in 192k): 16 warps an SM
+// with the weights fetched once per block.
+constexpr int kFwdWarps = 8;
+__global__ void __launch_bounds__(32 * kFwdWarps) forward_kernel(const Image* __restrict__ I,
+                                                                 const float* __restrict__ X, int64_t n, int no,
+                                                                 float* __restrict__ Y) {
+    __shared__ Image s;
+    __shared__ uint64_t bar;
+    dev::pdl_wait();
+    fetch_image(&s, I, &bar);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int64_t tiles = (n + 15) / 16;
-    for (int64_t tile = (int64_t)blockIdx.x * 4 + warp; tile < tiles; tile += (int64_t)gridDim.x * 4) {
+    for (int64_t tile = (int64_t)blockIdx.x * kFwdWarps + warp; tile < tiles; tile += (int64_t)gridDim.x * kFwdWarps) {
         const int64_t row0 = tile * 16;
         uint32_t a1[1][4], a2[4][4], a3[4][4], a4[4][4];
         load_x(X, row0 + g < n ? row0 + g : -1, row0 + g + 8 < n ? row0 + g + 8 : -1, t, a1[0]);
-        hidden_layer<1>(a1, s.wt1, kS16, s.b1, g, t, a2);
-        hidden_layer<4>(a2, s.wt2, kS64, s.b2, g, t, a3);
-        hidden_layer<4>(a3, s.wt3, kS64, s.b3, g, t, a4);
+        hidden_layer<1>(a1, s.wt1, kS16, s.b1, lane, a2);
+        hidden_layer<4>(a2, s.wt2, kS64, s.b2, lane, a3);
+        hidden_layer<4>(a3, s.wt3, kS64, s.b3, lane, a4);
         float d[4];
-        output_layer(a4, s, g, t, d);
+        output_layer(a4, s, lane, d);
         // this lane holds output columns 2t, 2t + 1 of rows g, g + 8
         const int c0 = 2 * t, c1 = 2 * t + 1;
         if (row0 + g < n) {
@@ -181,222 +255,208 @@ __global__ void __launch_bounds__(128) forward_kernel(const float* __restrict__ 
 }
 
 // ------------------------------------------------------------ gradients
-constexpr int kChunk = 64;  // rows per block iteration (4 warps x 16)
+constexpr int kGradWarps = 8;
+constexpr int kRound = 16 * kGradWarps;  // rows of a block's round
 
-struct BwdSmem {
-    FwdSmem f;
-    // row-major [in][out] BF16 weights for dX = dZ W^T
-    __nv_bfloat16 w2[kH * kS64];
-    __nv_bfloat16 w3[kH * kS64];
-    __nv_bfloat16 w4[kH * kS16];  // outputs padded to 16
-    // staging, transposed [feature][row] BF16
-    __nv_bfloat16 h0[kIn * kS64];
-    __nv_bfloat16 h1[kH * kS64], h2[kH * kS64], h3[kH * kS64];
-    __nv_bfloat16 dz1[kH * kS64], dz2[kH * kS64], dz3[kH * kS64];
-    __nv_bfloat16 dy[8 * kS64];
-    // FP32 gradient accumulators of the block
-    float gw1[kIn * kH], gw2[kH * kH], gw3[kH * kH], gw4[kH * 8];
-    float gb1[kH], gb2[kH], gb3[kH], gb4[8];
-    double loss[4];
+struct GradSmem {
+    Image w;
+    // the round's layer inputs and errors, [row][feature]
+    __nv_bfloat16 h0[kRound * kS16];
+    __nv_bfloat16 h[3][kRound * kS64];
+    __nv_bfloat16 dz[3][kRound * kS64];
+    __nv_bfloat16 dy[kRound * 8];
+    double loss[kGradWarps];
+    float bias[kGradWarps * 32];
+    uint64_t bar;
 };
 
-// write a warp's 16-row fragment of a [rows x 64] matrix (FP32 accumulator
-// layout, 8 n-tiles) into transposed staging [col][row], BF16
-__device__ __forceinline__ void stage_t(__nv_bfloat16* dst, const float (*v)[4], int rbase, int g, int t) {
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        const int c = 8 * nt + 2 * t;
-        dst[c * kS64 + rbase + g] = __float2bfloat16_rn(v[nt][0]);
-        dst[(c + 1) * kS64 + rbase + g] = __float2bfloat16_rn(v[nt][1]);
-        dst[c * kS64 + rbase + g + 8] = __float2bfloat16_rn(v[nt][2]);
-        dst[(c + 1) * kS64 + rbase + g + 8] = __float2bfloat16_rn(v[nt][3]);
-    }
-}
-
-// unpack A fragments (4 k-tiles, BF16 pairs) of a [rows x 64] activation to FP32 accumulator layout
-__device__ __forceinline__ void unpack_a(const uint32_t (*a)[4], float (*v)[4]) {
+// store a warp's [16 rows x 64] A fragments row-major
+__device__ __forceinline__ void stage(__nv_bfloat16* dst, const uint32_t (*a)[4], int rbase, int lane) {
+    const int g = lane >> 2, t = lane & 3;
 #pragma unroll
     for (int kt = 0; kt < 4; ++kt)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int nt = 2 * kt + h;
-            __nv_bfloat162 lo = *reinterpret_cast<const __nv_bfloat162*>(&a[kt][2 * h]);
-            __nv_bfloat162 hi = *reinterpret_cast<const __nv_bfloat162*>(&a[kt][2 * h + 1]);
-            v[nt][0] = __low2float(lo); v[nt][1] = __high2float(lo);
-            v[nt][2] = __low2float(hi); v[nt][3] = __high2float(hi);
-        }
+        for (int q = 0; q < 4; ++q)
+            *reinterpret_cast<uint32_t*>(dst + (rbase + g + 8 * (q & 1)) * kS64 + 16 * kt + 8 * (q >> 1) + 2 * t) =
+                a[kt][q];
 }
 
-// dA = dZ W^T for a layer with 64 inputs: dz (A fragments over the layer's
-// outputs, KT k-tiles), w row-major [in][out] with the given stride
+// dZ of the layer below: (dz W^T) where the activation h is positive, rounded
+// and packed; KT k-tiles over the layer's outputs (KT = 0: the output layer,
+// whose 8 padded outputs fill half a k-tile).  W^T comes from the forward rows
+// [out][in] by transposing loads.
 template <int KT>
-__device__ __forceinline__ void back_layer(const uint32_t (*dz)[4], const __nv_bfloat16* w, int stride, int g, int t,
-                                           float (*da)[4]) {
+__device__ __forceinline__ void back_layer(const uint32_t (*dz)[4], const __nv_bfloat16* wt, const uint32_t (*h)[4],
+                                           int lane, uint32_t (*out)[4]) {
+    const __nv_bfloat16* row = wt + (lane & 7) * kS64;
+    const int sel = lane >> 3;
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-        float d[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int np = 0; np < 4; ++np) {
+        float d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        if (KT == 0) {
+            uint32_t b[4];  // rows 0..7 of n-tiles 2 np, 2 np + 1 (the upper two matrices are not used)
+            ldsm4<true>(b, row + 16 * np + 8 * (sel & 1));
+            mma(d[0], dz[0], b[0], 0u);
+            mma(d[1], dz[0], b[1], 0u);
+        } else {
 #pragma unroll
-        for (int kt = 0; kt < KT; ++kt) {
-            const __nv_bfloat16* p = w + (8 * nt + g) * stride + 16 * kt + 2 * t;
-            mma(d, dz[kt], ld32(p), ld32(p + 8));
+            for (int kt = 0; kt < KT; ++kt) {
+                uint32_t b[4];  // n-tile 2 np rows 0..7, 8..15 of the k-tile; n-tile 2 np + 1 likewise
+                ldsm4<true>(b, row + (16 * kt + 8 * (sel & 1)) * kS64 + 16 * np + 8 * (sel >> 1));
+                mma(d[0], dz[kt], b[0], b[1]);
+                mma(d[1], dz[kt], b[2], b[3]);
+            }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) da[nt][i] = d[i];
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {  // rows g, g + 8
+                const __nv_bfloat162 hv = *reinterpret_cast<const __nv_bfloat162*>(&h[np][2 * j + r]);
+                out[np][2 * j + r] = pack2(__low2float(hv) > 0.f ? d[j][2 * r] : 0.f,
+                                           __high2float(hv) > 0.f ? d[j][2 * r + 1] : 0.f);
+            }
     }
 }
 
-// dZ = dA * [H > 0], rounded to BF16 and packed as A fragments
-__device__ __forceinline__ void mask_pack(float (*da)[4], const float (*h)[4], uint32_t (*out)[4]) {
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) da[nt][i] = h[nt][i] > 0.f ? da[nt][i] : 0.f;
-        out[nt >> 1][(nt & 1) * 2 + 0] = pack2(da[nt][0], da[nt][1]);
-        out[nt >> 1][(nt & 1) * 2 + 1] = pack2(da[nt][2], da[nt][3]);
-    }
+// A fragment (16 features from f0 x 16 rows from r0) of H^T, H [row][feature]
+__device__ __forceinline__ void frag_ht(uint32_t* a, const __nv_bfloat16* h, int stride, int r0, int f0, int lane) {
+    ldsm4<true>(a, h + (r0 + (lane & 7) + 8 * (lane >> 4)) * stride + f0 + 8 * ((lane >> 3) & 1));
+}
+// B fragments (16 rows from r0 x outputs c0 .. c0 + 15) of dZ [row][out]: b[0..1] and b[2..3]
+__device__ __forceinline__ void frag_dz(uint32_t* b, const __nv_bfloat16* z, int r0, int c0, int lane) {
+    ldsm4<true>(b, z + (r0 + (lane & 7) + 8 * ((lane >> 3) & 1)) * kS64 + c0 + 8 * (lane >> 4));
 }
 
-// dW tile (16 x 8) += H^T dZ over the chunk's 64 rows; h: [feat][row], dz: [out][row]
-__device__ __forceinline__ void dw_tile(const __nv_bfloat16* h, const __nv_bfloat16* dz, int mt, int nt, int g, int t,
-                                        float* d) {
-#pragma unroll
-    for (int kt = 0; kt < kChunk / 16; ++kt) {
-        const __nv_bfloat16* ap = h + (16 * mt + g) * kS64 + 16 * kt + 2 * t;
-        const uint32_t a[4] = {ld32(ap), ld32(ap + 8 * kS64), ld32(ap + 8), ld32(ap + 8 * kS64 + 8)};
-        const __nv_bfloat16* bp = dz + (8 * nt + g) * kS64 + 16 * kt + 2 * t;
-        mma(d, a, ld32(bp), ld32(bp + 8));
-    }
-}
-
-// n rows of the minibatch, drawn from n_data rows of (X, T) by data_row
-__global__ void __launch_bounds__(128) grad_kernel(const float* __restrict__ P, const float* __restrict__ X,
-                                                   const float* __restrict__ T, int no, int64_t n, int64_t n_data,
-                                                   uint64_t seed, uint64_t step, float inv_n2,
-                                                   float* __restrict__ partial, double* __restrict__ loss_partial) {
-    extern __shared__ __align__(16) uint8_t smem_raw[];
-    BwdSmem& s = *reinterpret_cast<BwdSmem*>(smem_raw);
-    load_fwd(P, no, s.f);
-    for (int i = threadIdx.x; i < kH * kS64; i += blockDim.x) {
-        const int r = i / kS64, c = i % kS64;
-        s.w2[i] = __float2bfloat16_rn(c < kH ? P[oW2 + r * kH + c] : 0.f);
-        s.w3[i] = __float2bfloat16_rn(c < kH ? P[oW3 + r * kH + c] : 0.f);
-    }
-    for (int i = threadIdx.x; i < kH * kS16; i += blockDim.x) {
-        const int r = i / kS16, c = i % kS16;
-        s.w4[i] = __float2bfloat16_rn(c < no ? P[oW4 + r * no + c] : 0.f);
-    }
-    for (int i = threadIdx.x; i < kIn * kH; i += blockDim.x) s.gw1[i] = 0.f;
-    for (int i = threadIdx.x; i < kH * kH; i += blockDim.x) { s.gw2[i] = 0.f; s.gw3[i] = 0.f; }
-    for (int i = threadIdx.x; i < kH * 8; i += blockDim.x) s.gw4[i] = 0.f;
-    for (int i = threadIdx.x; i < kH; i += blockDim.x) { s.gb1[i] = 0.f; s.gb2[i] = 0.f; s.gb3[i] = 0.f; }
-    if (threadIdx.x < 8) s.gb4[threadIdx.x] = 0.f;
-    if (threadIdx.x < 4) s.loss[threadIdx.x] = 0.0;
-    __syncthreads();
+// n rows of the minibatch, drawn from n_data rows of (X, T) by data_row.  Warp
+// w owns of dW2 and dW3 feature rows 16 (w % 4) .. + 15, outputs 32 (w / 4) ..
+// + 31; of dW1 outputs 8 w .. + 7; warps 0..3 of dW4 feature rows 16 w .. + 15.
+__global__ void __launch_bounds__(32 * kGradWarps, 1)
+    grad_kernel(const Image* __restrict__ I, const float* __restrict__ X, const float* __restrict__ T, int no, int64_t n,
+                int64_t n_data, uint64_t seed, uint64_t step, float inv_n2, float* __restrict__ partial,
+                double* __restrict__ loss_partial) {
+    extern __shared__ __align__(128) uint8_t smem_raw[];
+    GradSmem& s = *reinterpret_cast<GradSmem*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    dev::pdl_trigger();
+    dev::pdl_wait();  // the image is written by the kernel before
+    fetch_image(&s.w, I, &s.bar);
+    float m1[4] = {}, m2[4][4] = {}, m3[4][4] = {}, m4[4] = {};
+    float mb0 = 0.f, mb1 = 0.f;
     double my_loss = 0.0;
-    const int64_t chunks = (n + kChunk - 1) / kChunk;
-    for (int64_t ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
-        const int64_t row0 = ch * kChunk + warp * 16;
+    // contiguous 16-row tiles per block
+    const int64_t tiles = (n + 15) / 16;
+    const int64_t tile0 = tiles * blockIdx.x / gridDim.x, tile1 = tiles * (blockIdx.x + 1) / gridDim.x;
+    for (int64_t tb = tile0; tb < tile1; tb += kGradWarps) {
+        const int act = (int)(tile1 - tb < kGradWarps ? tile1 - tb : kGradWarps);  // tiles of this round
         const int rb = warp * 16;
-        // ---- forward for the warp's 16 rows, keeping every activation
-        uint32_t a1[1][4], a2[4][4], a3[4][4], a4[4][4];
-        const int64_t r0 = row0 + g, r1 = row0 + g + 8;
-        const int64_t src0 = r0 < n ? data_row(r0, n_data, seed, step) : -1;
-        const int64_t src1 = r1 < n ? data_row(r1, n_data, seed, step) : -1;
-        load_x(X, src0, src1, t, a1[0]);
-        hidden_layer<1>(a1, s.f.wt1, kS16, s.f.b1, g, t, a2);
-        hidden_layer<4>(a2, s.f.wt2, kS64, s.f.b2, g, t, a3);
-        hidden_layer<4>(a3, s.f.wt3, kS64, s.f.b3, g, t, a4);
-        float y[4];
-        output_layer(a4, s.f, g, t, y);
-        // ---- output error dY = 2 (Y - T) / n (zero on padding rows and
-        // columns); this lane holds columns 2t, 2t + 1 of rows g, g + 8
-        float dy[4] = {0.f, 0.f, 0.f, 0.f};
+        if (warp < act) {
+            // ---- forward for the warp's 16 rows, keeping every activation
+            const int64_t row0 = (tb + warp) * 16;
+            int64_t mine = -1;
+            if (lane < 16 && row0 + lane < n) mine = data_row(row0 + lane, n_data, seed, step);
+            const int64_t src0 = __shfl_sync(0xffffffffu, mine, g), src1 = __shfl_sync(0xffffffffu, mine, g + 8);
+            uint32_t a1[1][4], a2[4][4], a3[4][4], a4[4][4];
+            load_x(X, src0, src1, t, a1[0]);
+            float tv[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = 2 * t + (q & 1);
-            const int64_t src = q < 2 ? src0 : src1;
-            if (c < no && src >= 0) {
-                const float e = y[q] - T[src * no + c];
-                my_loss += (double)e * e;
-                dy[q] = inv_n2 * e;
+            for (int q = 0; q < 4; ++q) {
+                const int c = 2 * t + (q & 1);
+                const int64_t src = q < 2 ? src0 : src1;
+                if (c < no && src >= 0) tv[q] = T[src * no + c];
             }
+            hidden_layer<1>(a1, s.w.wt1, kS16, s.w.b1, lane, a2);
+            hidden_layer<4>(a2, s.w.wt2, kS64, s.w.b2, lane, a3);
+            hidden_layer<4>(a3, s.w.wt3, kS64, s.w.b3, lane, a4);
+            float y[4];
+            output_layer(a4, s.w, lane, y);
+            // ---- output error dY = 2 (Y - T) / n (zero on padding rows and
+            // columns); this lane holds columns 2t, 2t + 1 of rows g, g + 8
+            float dy[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int c = 2 * t + (q & 1);
+                const int64_t src = q < 2 ? src0 : src1;
+                if (c < no && src >= 0) {
+                    const float e = y[q] - tv[q];
+                    my_loss += (double)e * e;
+                    dy[q] = inv_n2 * e;
+                }
+            }
+            uint32_t ady[1][4] = {{pack2(dy[0], dy[1]), pack2(dy[2], dy[3]), 0u, 0u}};
+            // ---- the inputs of every layer and dY
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<uint32_t*>(s.h0 + (rb + g + 8 * (q & 1)) * kS16 + 8 * (q >> 1) + 2 * t) = a1[0][q];
+            stage(s.h[0], a2, rb, lane);
+            stage(s.h[1], a3, rb, lane);
+            stage(s.h[2], a4, rb, lane);
+            *reinterpret_cast<uint32_t*>(s.dy + (rb + g) * 8 + 2 * t) = ady[0][0];
+            *reinterpret_cast<uint32_t*>(s.dy + (rb + g + 8) * 8 + 2 * t) = ady[0][1];
+            // ---- back through the layers: dZ3 = (dY W4^T) * [H3 > 0], ...
+            uint32_t dz[4][4], dn[4][4];
+            back_layer<0>(ady, s.w.wt4, a4, lane, dz);
+            stage(s.dz[2], dz, rb, lane);
+            back_layer<4>(dz, s.w.wt3, a3, lane, dn);
+            stage(s.dz[1], dn, rb, lane);
+            back_layer<4>(dn, s.w.wt2, a2, lane, dz);
+            stage(s.dz[0], dz, rb, lane);
         }
-        // staging of the inputs of every layer and of dY
-        {
-            float v[8][4];
-            unpack_a(a2, v);
-            stage_t(s.h1, v, rb, g, t);
-            unpack_a(a3, v);
-            stage_t(s.h2, v, rb, g, t);
-            unpack_a(a4, v);
-            stage_t(s.h3, v, rb, g, t);
-            // features: rows g, g+8; cols 2t, 2t+1, 2t+8, 2t+9
-            const __nv_bfloat162* xa = reinterpret_cast<const __nv_bfloat162*>(a1[0]);
-            s.h0[(2 * t) * kS64 + rb + g] = xa[0].x; s.h0[(2 * t + 1) * kS64 + rb + g] = xa[0].y;
-            s.h0[(2 * t) * kS64 + rb + g + 8] = xa[1].x; s.h0[(2 * t + 1) * kS64 + rb + g + 8] = xa[1].y;
-            s.h0[(2 * t + 8) * kS64 + rb + g] = xa[2].x; s.h0[(2 * t + 9) * kS64 + rb + g] = xa[2].y;
-            s.h0[(2 * t + 8) * kS64 + rb + g + 8] = xa[3].x; s.h0[(2 * t + 9) * kS64 + rb + g + 8] = xa[3].y;
-            // dY (cols 0..7, only 0 and 1 non-zero)
-            s.dy[(2 * t) * kS64 + rb + g] = __float2bfloat16_rn(dy[0]);
-            s.dy[(2 * t + 1) * kS64 + rb + g] = __float2bfloat16_rn(dy[1]);
-            s.dy[(2 * t) * kS64 + rb + g + 8] = __float2bfloat16_rn(dy[2]);
-            s.dy[(2 * t + 1) * kS64 + rb + g + 8] = __float2bfloat16_rn(dy[3]);
-        }
-        // ---- back through the layers: dZ3 = (dY W4^T) * [H3 > 0], ...
-        uint32_t ady[1][4] = {{pack2(dy[0], dy[1]), pack2(dy[2], dy[3]), 0u, 0u}};
-        float da[8][4], hv[8][4];
-        uint32_t dz3[4][4], dz2[4][4], dz1[4][4];
-        back_layer<1>(ady, s.w4, kS16, g, t, da);
-        unpack_a(a4, hv);
-        mask_pack(da, hv, dz3);
-        stage_t(s.dz3, da, rb, g, t);
-        back_layer<4>(dz3, s.w3, kS64, g, t, da);
-        unpack_a(a3, hv);
-        mask_pack(da, hv, dz2);
-        stage_t(s.dz2, da, rb, g, t);
-        back_layer<4>(dz2, s.w2, kS64, g, t, da);
-        unpack_a(a2, hv);
-        mask_pack(da, hv, dz1);
-        stage_t(s.dz1, da, rb, g, t);
         __syncthreads();
-        // ---- weight gradients of the chunk: 76 output tiles, warp w takes w, w+4, ...
-        for (int tile = warp; tile < 76; tile += 4) {
-            float d[4] = {0.f, 0.f, 0.f, 0.f};
-            float* gw;
-            int ld, mt, nt, ncols;
-            if (tile < 8) {  // dW1 [16][64]
-                mt = 0; nt = tile; gw = s.gw1; ld = kH; ncols = kH;
-                dw_tile(s.h0, s.dz1, mt, nt, g, t, d);
-            } else if (tile < 40) {  // dW2 [64][64]
-                mt = (tile - 8) >> 3; nt = (tile - 8) & 7; gw = s.gw2; ld = kH; ncols = kH;
-                dw_tile(s.h1, s.dz2, mt, nt, g, t, d);
-            } else if (tile < 72) {  // dW3
-                mt = (tile - 40) >> 3; nt = (tile - 40) & 7; gw = s.gw3; ld = kH; ncols = kH;
-                dw_tile(s.h2, s.dz3, mt, nt, g, t, d);
-            } else {  // dW4 [64][8]
-                mt = tile - 72; nt = 0; gw = s.gw4; ld = 8; ncols = 8;
-                dw_tile(s.h3, s.dy, mt, nt, g, t, d);
+        // ---- weight gradients: chains of up to 64 rows, added in FP32
+        const int mt = warp & 3, c0 = 32 * (warp >> 2);
+        for (int half = 0; 4 * half < act; ++half) {
+            float d1[4] = {}, d2[4][4] = {}, d3[4][4] = {}, d4[4] = {};
+            const int kend = act < 4 * half + 4 ? act : 4 * half + 4;
+            for (int kt = 4 * half; kt < kend; ++kt) {
+                const int r0 = 16 * kt;
+                uint32_t a[4], b[8];
+                frag_ht(a, s.h[0], kS64, r0, 16 * mt, lane);
+                frag_dz(b, s.dz[1], r0, c0, lane);
+                frag_dz(b + 4, s.dz[1], r0, c0 + 16, lane);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) mma(d2[j], a, b[2 * j], b[2 * j + 1]);
+                frag_ht(a, s.h[1], kS64, r0, 16 * mt, lane);
+                frag_dz(b, s.dz[2], r0, c0, lane);
+                frag_dz(b + 4, s.dz[2], r0, c0 + 16, lane);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) mma(d3[j], a, b[2 * j], b[2 * j + 1]);
+                frag_ht(a, s.h0, kS16, r0, 0, lane);
+                frag_dz(b, s.dz[0], r0, 16 * (warp >> 1), lane);
+                mma(d1, a, warp & 1 ? b[2] : b[0], warp & 1 ? b[3] : b[1]);
+                if (warp < 4) {
+                    frag_ht(a, s.h[2], kS64, r0, 16 * warp, lane);
+                    // rows 0..7 and 8..15 of dY (lanes above 15 repeat them)
+                    ldsm4<true>(b, s.dy + (r0 + (lane & 7) + 8 * ((lane >> 3) & 1)) * 8);
+                    mma(d4, a, b[0], b[1]);
+                }
             }
-            const int r = 16 * mt + g, c = 8 * nt + 2 * t;
-            if (c < ncols) {
-                gw[r * ld + c] += d[0];
-                gw[r * ld + c + 1] += d[1];
-                gw[(r + 8) * ld + c] += d[2];
-                gw[(r + 8) * ld + c + 1] += d[3];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                m1[i] += d1[i];
+                m4[i] += d4[i];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    m2[j][i] += d2[j][i];
+                    m3[j][i] += d3[j][i];
+                }
             }
         }
-        // ---- bias gradients: column sums of the BF16 errors over the chunk
-        for (int c = threadIdx.x; c < 3 * kH + no; c += blockDim.x) {
-            const __nv_bfloat16* src;
-            float* dst;
-            if (c < kH) { src = s.dz1 + c * kS64; dst = &s.gb1[c]; }
-            else if (c < 2 * kH) { src = s.dz2 + (c - kH) * kS64; dst = &s.gb2[c - kH]; }
-            else if (c < 3 * kH) { src = s.dz3 + (c - 2 * kH) * kS64; dst = &s.gb3[c - 2 * kH]; }
-            else { src = s.dy + (c - 3 * kH) * kS64; dst = &s.gb4[c - 3 * kH]; }
-            float acc = 0.f;
-            for (int r = 0; r < kChunk; ++r) acc += __bfloat162float(src[r]);
-            *dst += acc;
+        // ---- bias gradients: sums of the BF16 errors over the round's rows;
+        // threads 0..191 take column pairs (even and odd rows apart), 192.. dY
+        if (threadIdx.x < 192) {
+            const int pr = threadIdx.x >> 1, layer = pr >> 5, c = 2 * (pr & 31);
+            float u = 0.f, v = 0.f;
+            for (int r = threadIdx.x & 1; r < 16 * act; r += 2) {
+                const __nv_bfloat162 z = *reinterpret_cast<const __nv_bfloat162*>(s.dz[layer] + r * kS64 + c);
+                u += __low2float(z);
+                v += __high2float(z);
+            }
+            mb0 += u;
+            mb1 += v;
+        } else if (threadIdx.x < 192 + 8) {
+            float u = 0.f;
+            for (int r = 0; r < 16 * act; ++r) u += __bfloat162float(s.dy[r * 8 + threadIdx.x - 192]);
+            mb0 += u;
         }
         __syncthreads();
     }
@@ -404,49 +464,88 @@ __global__ void __launch_bounds__(128) grad_kernel(const float* __restrict__ P, 
     for (int o = 16; o > 0; o >>= 1) my_loss += __shfl_xor_sync(0xffffffffu, my_loss, o);
     if (lane == 0) s.loss[warp] = my_loss;
     __syncthreads();
-    float* out = partial + (size_t)blockIdx.x * param_count(no);
-    for (int i = threadIdx.x; i < kIn * kH; i += blockDim.x) out[oW1 + i] = s.gw1[i];
-    for (int i = threadIdx.x; i < kH * kH; i += blockDim.x) {
-        out[oW2 + i] = s.gw2[i];
-        out[oW3 + i] = s.gw3[i];
-    }
-    for (int i = threadIdx.x; i < kH; i += blockDim.x) {
-        out[oB1 + i] = s.gb1[i];
-        out[oB2 + i] = s.gb2[i];
-        out[oB3 + i] = s.gb3[i];
-        for (int j = 0; j < no; ++j) out[oW4 + i * no + j] = s.gw4[i * 8 + j];
-    }
-    if ((int)threadIdx.x < no) out[off_b4(no) + threadIdx.x] = s.gb4[threadIdx.x];
-    if (threadIdx.x == 0) loss_partial[blockIdx.x] = (s.loss[0] + s.loss[1]) + (s.loss[2] + s.loss[3]);
-}
-
-__global__ void sum_partials(int nb, int kp, const float* __restrict__ partial, const double* __restrict__ loss_partial,
-                             float* __restrict__ grad, double* __restrict__ loss) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < kp) {
-        float acc = 0.f;
-        for (int b = 0; b < nb; ++b) acc += partial[(size_t)b * kp + i];
-        grad[i] = acc;
-    }
-    if (i == 0) {
+    if (threadIdx.x == 0) {
         double l = 0.0;
-        for (int b = 0; b < nb; ++b) l += loss_partial[b];
-        *loss = l;
+        for (int w = 0; w < kGradWarps; ++w) l += s.loss[w];
+        loss_partial[blockIdx.x] = l;
+    }
+    float* out = partial + (size_t)blockIdx.x * param_count(no);
+    auto put = [&](int o, int ld, int r, int c, const float* v) {  // C fragment at row r, column c
+        out[o + r * ld + c] = v[0];
+        out[o + r * ld + c + 1] = v[1];
+        out[o + (r + 8) * ld + c] = v[2];
+        out[o + (r + 8) * ld + c + 1] = v[3];
+    };
+    const int mt = warp & 3, c0 = 32 * (warp >> 2);
+    put(oW1, kH, g, 8 * warp + 2 * t, m1);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        put(oW2, kH, 16 * mt + g, c0 + 8 * j + 2 * t, m2[j]);
+        put(oW3, kH, 16 * mt + g, c0 + 8 * j + 2 * t, m3[j]);
+    }
+    if (warp < 4)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (2 * t + (i & 1) < no) out[oW4 + (16 * warp + g + 8 * (i >> 1)) * no + 2 * t + (i & 1)] = m4[i];
+    // even and odd rows of a bias column together
+    mb0 += __shfl_down_sync(0xffffffffu, threadIdx.x < 192 ? mb0 : 0.f, 1);
+    mb1 += __shfl_down_sync(0xffffffffu, mb1, 1);
+    if (threadIdx.x < 192) {
+        if (!(threadIdx.x & 1)) {
+            const int pr = threadIdx.x >> 1, layer = pr >> 5, c = 2 * (pr & 31);
+            const int o = layer == 0 ? oB1 : (layer == 1 ? oB2 : oB3);
+            out[o + c] = mb0;
+            out[o + c + 1] = mb1;
+        }
+    } else if ((int)threadIdx.x < 192 + no) {
+        out[off_b4(no) + threadIdx.x - 192] = mb0;
     }
 }
 
-// Adam (Kingma & Ba), bias-corrected, on the FP32 master parameters
-__global__ void adam_kernel(int kp, float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ grad, float lr, float b1, float b2, float eps, float c1,
-                            float c2) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= kp) return;
-    const float gi = grad[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+// Adds the blocks' partial gradients and losses in a fixed order (eight slices
+// of the blocks per parameter side by side, then the slices), and with ADAM
+// takes the bias-corrected Adam step (Kingma & Ba) on the FP32 master
+// parameters and writes the changed weights into the image.  It is bound by
+// reading the partials (38 KB a block) from L2, so it spreads each parameter
+// over eight threads.
+constexpr int kSumParams = 32, kSumSlices = 8;
+template <bool ADAM>
+__global__ void __launch_bounds__(kSumParams * kSumSlices)
+    sum_partials(int nb, int kp, int no, const float* __restrict__ partial, const double* __restrict__ loss_partial,
+                 float* __restrict__ grad, double* __restrict__ loss, float* __restrict__ p, float* __restrict__ m,
+                 float* __restrict__ v, Image* __restrict__ I, float lr, float b1, float b2, float eps, float c1,
+                 float c2) {
+    __shared__ float slice[kSumSlices][kSumParams];
+    const int lane = threadIdx.x % kSumParams, sl = threadIdx.x / kSumParams;
+    const int i = blockIdx.x * kSumParams + lane;
+    dev::pdl_trigger();
+    dev::pdl_wait();
+    float acc = 0.f;
+    if (i < kp)
+        for (int b = sl; b < nb; b += kSumSlices) acc += partial[(size_t)b * kp + i];
+    slice[sl][lane] = acc;
+    __syncthreads();
+    if (sl == 0 && i < kp) {
+        float gi = slice[0][lane];
+#pragma unroll
+        for (int q = 1; q < kSumSlices; ++q) gi += slice[q][lane];
+        grad[i] = gi;
+        if (ADAM) {
+            const float mi = b1 * m[i] + (1.f - b1) * gi;
+            const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+            m[i] = mi;
+            v[i] = vi;
+            const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+            p[i] = pi;
+            image_put(I, no, i, pi);
+        }
+    }
+    if (blockIdx.x == 0 && sl == 1) {  // one warp: 32 strided sums, then across the lanes
+        double l = 0.0;
+        for (int b = lane; b < nb; b += 32) l += loss_partial[b];
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) *loss = l;
+    }
 }
 
 }  // namespace mlp
@@ -455,6 +554,7 @@ __global__ void adam_kernel(int kp, float* __restrict__ p, float* __restrict__ m
 using namespace mlbm;
 
 struct mlbm_mlp {
+    mlp::Image* img = nullptr;  // BF16 weights and biases, kept in line with p
     float* p = nullptr;
     float* m = nullptr;
     float* v = nullptr;
@@ -486,10 +586,10 @@ double gauss(uint64_t& s) {
     const double u2 = ((splitmix(s) >> 11) + 0.5) * (1.0 / 9007199254740992.0);
     return std::sqrt(-2.0 * std::log(u1)) * std::cos(6.283185307179586 * u2);
 }
-constexpr int kMaxGradBlocks = 2 * 152;
+constexpr int kMaxGradBlocks = 152;  // one per SM
 int grad_blocks(int64_t n) {
-    const int64_t chunks = (n + mlp::kChunk - 1) / mlp::kChunk;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(chunks, kMaxGradBlocks));
+    const int64_t rounds = (n + mlp::kRound - 1) / mlp::kRound;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(rounds, kMaxGradBlocks));
 }
 }  // namespace
 
@@ -511,6 +611,8 @@ mlbm_status mlbm_mlp_create(mlbm_mlp** out, int n_out, uint64_t seed) {
     m->n_out = n_out;
     m->kp = mlp::param_count(n_out);
     cudaError_t e = cudaSuccess;
+    e = e == cudaSuccess ? cudaMalloc(&m->img, sizeof(mlp::Image)) : e;
+    e = e == cudaSuccess ? cudaMemset(m->img, 0, sizeof(mlp::Image)) : e;
     e = e == cudaSuccess ? cudaMalloc(&m->p, m->kp * 4) : e;
     e = e == cudaSuccess ? cudaMalloc(&m->m, m->kp * 4) : e;
     e = e == cudaSuccess ? cudaMalloc(&m->v, m->kp * 4) : e;
@@ -545,7 +647,7 @@ mlbm_status mlbm_mlp_create(mlbm_mlp** out, int n_out, uint64_t seed) {
 
 void mlbm_mlp_destroy(mlbm_mlp* m) {
     if (!m) return;
-    cudaFree(m->p); cudaFree(m->m); cudaFree(m->v); cudaFree(m->grad); cudaFree(m->partial);
+    cudaFree(m->img); cudaFree(m->p); cudaFree(m->m); cudaFree(m->v); cudaFree(m->grad); cudaFree(m->partial);
     cudaFree(m->loss_partial); cudaFree(m->loss);
     delete m;
 }
@@ -555,6 +657,9 @@ mlbm_status mlbm_mlp_set_params(mlbm_mlp* m, const float* params) {
     MLP_CUDA(cudaMemcpy(m->p, params, m->kp * 4, cudaMemcpyHostToDevice));
     MLP_CUDA(cudaMemset(m->m, 0, m->kp * 4));
     MLP_CUDA(cudaMemset(m->v, 0, m->kp * 4));
+    mlp::refresh_image<<<(m->kp + 255) / 256, 256>>>(m->kp, m->n_out, m->p, m->img);
+    MLP_CUDA(cudaGetLastError());
+    MLP_CUDA(cudaStreamSynchronize(nullptr));
     m->t = 0;
     return MLBM_OK;
 }
@@ -569,8 +674,10 @@ mlbm_status mlbm_mlp_forward_device(mlbm_mlp* m, const float* X, int64_t n, floa
     if (!m || (n > 0 && (!X || !Y)) || n < 0) return set_error(MLBM_E_INVALID, "mlp_forward: bad arguments");
     if (n == 0) return MLBM_OK;
     const int64_t tiles = (n + 15) / 16;
-    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((tiles + 3) / 4, 152 * 8));
-    mlp::forward_kernel<<<blocks, 128, 0, static_cast<cudaStream_t>(stream)>>>(m->p, X, n, m->n_out, Y);
+    const int blocks =
+        (int)std::max<int64_t>(1, std::min<int64_t>((tiles + mlp::kFwdWarps - 1) / mlp::kFwdWarps, 152 * 2));
+    mlp::forward_kernel<<<blocks, 32 * mlp::kFwdWarps, 0, static_cast<cudaStream_t>(stream)>>>(m->img, X, n, m->n_out,
+                                                                                               Y);
     MLP_CUDA(cudaGetLastError());
     return MLBM_OK;
 }
@@ -578,18 +685,20 @@ mlbm_status mlbm_mlp_forward_device(mlbm_mlp* m, const float* X, int64_t n, floa
 }  // extern "C"
 
 namespace {
-// one gradient evaluation over n minibatch rows into m->grad and the
-// device loss sum m->loss
+// one gradient evaluation over n minibatch rows into m->grad and the device
+// loss sum m->loss, and with lr > 0 the Adam step number m->t on it
 mlbm_status grad_pass(mlbm_mlp* m, const float* X, const float* T, int64_t n, int64_t n_data, uint64_t seed,
-                      uint64_t step, cudaStream_t st) {
+                      uint64_t step, float lr, cudaStream_t st) {
     const int nb = grad_blocks(n);
-    const size_t smem = sizeof(mlp::BwdSmem);
+    const size_t smem = sizeof(mlp::GradSmem);
     MLP_CUDA(cudaFuncSetAttribute(mlp::grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    mlp::grad_kernel<<<nb, 128, smem, st>>>(m->p, X, T, m->n_out, n, n_data, seed, step, (float)(2.0 / (double)n),
-                                            m->partial, m->loss_partial);
-    MLP_CUDA(cudaGetLastError());
-    mlp::sum_partials<<<(m->kp + 255) / 256, 256, 0, st>>>(nb, m->kp, m->partial, m->loss_partial, m->grad, m->loss);
-    MLP_CUDA(cudaGetLastError());
+    MLP_CUDA(launch_pdl_smem(mlp::grad_kernel, nb, 32 * mlp::kGradWarps, smem, st, m->img, X, T, m->n_out, n, n_data,
+                             seed, step, (float)(2.0 / (double)n), m->partial, m->loss_partial));
+    const int blocks = (m->kp + mlp::kSumParams - 1) / mlp::kSumParams, threads = mlp::kSumParams * mlp::kSumSlices;
+    const double c1 = 1.0 - std::pow(0.9, (double)m->t), c2 = 1.0 - std::pow(0.999, (double)m->t);
+    auto fn = lr > 0 ? mlp::sum_partials<true> : mlp::sum_partials<false>;
+    MLP_CUDA(launch_pdl_smem(fn, blocks, threads, 0, st, nb, m->kp, m->n_out, m->partial, m->loss_partial, m->grad,
+                             m->loss, m->p, m->m, m->v, m->img, lr, 0.9f, 0.999f, 1e-8f, (float)c1, (float)c2));
     return MLBM_OK;
 }
 
@@ -608,7 +717,7 @@ mlbm_status mlbm_mlp_gradients_device(mlbm_mlp* m, const float* X, const float* 
                                       double* loss, void* stream) {
     if (!m || !X || !T || n <= 0) return set_error(MLBM_E_INVALID, "mlp_gradients: bad arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    mlbm_status s = grad_pass(m, X, T, n, n, 0, 0, st);
+    mlbm_status s = grad_pass(m, X, T, n, n, 0, 0, 0.f, st);
     if (s != MLBM_OK) return s;
     if (grads) MLP_CUDA(cudaMemcpyAsync(grads, m->grad, m->kp * 4, cudaMemcpyDeviceToDevice, st));
     if (loss) return read_loss(m, n, loss, st);
@@ -621,13 +730,13 @@ mlbm_status mlbm_mlp_train_device(mlbm_mlp* m, const float* X, const float* T, i
         return set_error(MLBM_E_INVALID, "mlp_train: bad arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     for (int64_t k = 0; k < steps; ++k) {
-        mlbm_status s = grad_pass(m, X, T, batch, n, seed, (uint64_t)m->t, st);
-        if (s != MLBM_OK) return s;
+        const uint64_t draw = (uint64_t)m->t;
         m->t += 1;
-        const double c1 = 1.0 - std::pow(0.9, (double)m->t), c2 = 1.0 - std::pow(0.999, (double)m->t);
-        mlp::adam_kernel<<<(m->kp + 255) / 256, 256, 0, st>>>(m->kp, m->p, m->m, m->v, m->grad, lr, 0.9f, 0.999f, 1e-8f,
-                                                                (float)c1, (float)c2);
-        MLP_CUDA(cudaGetLastError());
+        mlbm_status s = grad_pass(m, X, T, batch, n, seed, draw, lr, st);
+        if (s != MLBM_OK) {
+            m->t -= 1;
+            return s;
+        }
     }
     if (loss) {
         if (steps == 0) return set_error(MLBM_E_INVALID, "mlp_train: no step taken, no loss to report");
