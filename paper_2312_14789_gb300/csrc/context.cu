@@ -54,11 +54,10 @@ struct mlbm_ctx {
     float4* ruv[2] = {nullptr, nullptr};
     int cur = 0;
     // work
-    float *rho = nullptr, *ux = nullptr, *uy = nullptr, *px = nullptr, *py = nullptr;
+    float *rho = nullptr, *px = nullptr, *py = nullptr;
     double* io = nullptr;
     double* scratch = nullptr;
     int64_t scratch_len = 0;
-    double* small = nullptr;
     int64_t steps = 0;
     int64_t steps_in_last_run = 0;  // steps taken by the last run to steady state
     bool timing = false;
@@ -75,7 +74,13 @@ struct mlbm_ctx {
     std::vector<mlbm_params> seg_params;
     std::vector<double> seg_box_area;
     std::vector<double> seg_s;  // streaming distance of each sample
-    double* seg_out = nullptr;  // device, 6 doubles per sample
+    // device: the error word of the bounded waits (err, 8 bytes) and behind it
+    // the results of an observable, up to 9 doubles per sample, so that one
+    // copy brings both back
+    double* seg_out = nullptr;
+    int64_t* seg_dev = nullptr;  // seg_off on the device
+    int max_blocks = 1;          // reduction blocks of the largest sample
+    std::vector<int> link_off;   // first link node of each sample, plus the total
     // captured step graphs: chunk of kGraphSteps steps starting from buffer 0 / 1
     bool use_graphs = true;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -167,20 +172,37 @@ mlbm_status check_params(const mlbm_params* p) {
     return MLBM_OK;
 }
 
-mlbm_status sync(mlbm_ctx* c) {
+// a set error word: cleared in stream order, before any later launch can set
+// it again, and reported
+mlbm_status wait_failed(mlbm_ctx* c, int code) {
+    MLBM_CUDA(cudaMemsetAsync(c->err, 0, sizeof(int), c->stream));
     MLBM_CUDA(cudaStreamSynchronize(c->stream));
-    if (c->err) {
-        int e = 0;
-        MLBM_CUDA(cudaMemcpyAsync(&e, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    return set_error(MLBM_E_TIMEOUT, "a bounded device wait gave up (code " + std::to_string(code) +
+                                         "); the step result is invalid");
+}
+
+mlbm_status sync(mlbm_ctx* c) {
+    int e = 0;
+    if (c->err) MLBM_CUDA(cudaMemcpyAsync(&e, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    MLBM_CUDA(cudaStreamSynchronize(c->stream));
+    return e != 0 ? wait_failed(c, e) : MLBM_OK;
+}
+
+// the first `count` results and the error word, in one copy
+mlbm_status read_results(mlbm_ctx* c, double* h, size_t count) {
+    std::vector<double> buf(count + 1);
+    const bool together = reinterpret_cast<double*>(c->err) + 1 == c->seg_out;
+    if (together) {
+        MLBM_CUDA(cudaMemcpyAsync(buf.data(), c->err, (count + 1) * 8, cudaMemcpyDeviceToHost, c->stream));
         MLBM_CUDA(cudaStreamSynchronize(c->stream));
-        if (e != 0) {
-            // cleared in stream order, before any later launch can set it again
-            MLBM_CUDA(cudaMemsetAsync(c->err, 0, sizeof(int), c->stream));
-            MLBM_CUDA(cudaStreamSynchronize(c->stream));
-            return set_error(MLBM_E_TIMEOUT, "a bounded device wait gave up (code " + std::to_string(e) +
-                                                 "); the step result is invalid");
-        }
+        int e = 0;
+        std::memcpy(&e, buf.data(), sizeof(int));
+        if (e != 0) return wait_failed(c, e);
+    } else {  // a partition, whose error word lies elsewhere
+        MLBM_CUDA(cudaMemcpyAsync(buf.data() + 1, c->seg_out, count * 8, cudaMemcpyDeviceToHost, c->stream));
+        MLBM_TRY(sync(c));
     }
+    std::copy(buf.begin() + 1, buf.end(), h);
     return MLBM_OK;
 }
 
@@ -411,22 +433,31 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         }
     }
     MLBM_TRY(dalloc(c, &c->rho, np));
-    MLBM_TRY(dalloc(c, &c->ux, np));
-    MLBM_TRY(dalloc(c, &c->uy, np));
     MLBM_TRY(dalloc(c, &c->px, np));
     MLBM_TRY(dalloc(c, &c->py, np));
     MLBM_TRY(dalloc(c, &c->io, (size_t)9 * np));
-    c->scratch_len = std::max<int64_t>(6 * reduce_blocks(np), 2 * force_blocks(c->n_link_nodes));
-    MLBM_TRY(dalloc(c, &c->scratch, c->scratch_len));
-    MLBM_TRY(dalloc(c, &c->small, 16));
     if (c->seg_off.empty()) {
         c->seg_off = {0, n};
         c->seg_params = {*p};
         c->seg_box_area = {H.box_area};
     }
-    MLBM_TRY(dalloc(c, &c->seg_out, 6 * (c->seg_off.size() - 1)));
-    MLBM_TRY(dalloc(c, &c->err, 1));
-    MLBM_CUDA(cudaMemsetAsync(c->err, 0, sizeof(int), c->stream));
+    const size_t ns = c->seg_off.size() - 1;
+    for (size_t i = 0; i < ns; ++i)
+        c->max_blocks = std::max(c->max_blocks, reduce_blocks(c->seg_off[i + 1] - c->seg_off[i]));
+    c->link_off.resize(ns + 1);
+    for (size_t i = 0; i <= ns; ++i)
+        c->link_off[i] = (int)(std::lower_bound(hlinknodes.begin(), hlinknodes.end(), (int)c->seg_off[i]) -
+                               hlinknodes.begin());
+    c->scratch_len = std::max<int64_t>((int64_t)kObserveBoth * (int64_t)ns * c->max_blocks,
+                                       2 * force_blocks(c->n_link_nodes));
+    MLBM_TRY(dalloc(c, &c->scratch, c->scratch_len));
+    double* results = nullptr;
+    MLBM_TRY(dalloc(c, &results, 1 + kObserveBoth * ns));
+    c->err = reinterpret_cast<int*>(results);
+    c->seg_out = results + 1;
+    MLBM_TRY(dalloc(c, &c->seg_dev, ns + 1));
+    MLBM_TRY(upload(c, c->seg_dev, c->seg_off.data(), (ns + 1) * sizeof(int64_t)));
+    MLBM_CUDA(cudaMemsetAsync(c->err, 0, sizeof(double), c->stream));
     if (!tma_supported(Kq)) c->variant = 1;  // variants >= 4 exist for K in {12, 16, 24, 32}
     if (rbf) {
         MLBM_TRY(upload(c, c->idx, hidx.data(), hidx.size() * 4));
@@ -576,11 +607,39 @@ void free_ctx(mlbm_ctx* c) {
     delete c;
 }
 
-mlbm_status fields_to_work(mlbm_ctx* c, double* ru_dev_or_null) {
-    const int n = (int)c->n;
-    MLBM_CUDA(launch_macroscopics(c->params.model, n, c->perm, c->f8[c->cur], c->f0[c->cur], c->ruv[c->cur],
-                                  (float)c->params.gx, (float)c->params.gy, c->S.node_sample, c->S.coll, c->rho,
-                                  c->ux, c->uy, ru_dev_or_null, c->stream));
+// (rho, u) of every node in the caller's order into FP64 device memory: rows
+// [n][3], or (split) rho[n] followed by u[n][2]
+mlbm_status fields_to(mlbm_ctx* c, double* out, int split) {
+    MLBM_CUDA(launch_macroscopics(c->params.model, (int)c->n, c->perm, c->f8[c->cur], c->f0[c->cur], c->ruv[c->cur],
+                                  (float)c->params.gx, (float)c->params.gy, c->S.node_sample, c->S.coll, split, out,
+                                  c->stream));
+    return MLBM_OK;
+}
+
+// observables of every sample into seg_out (see launch_observe)
+mlbm_status observe(mlbm_ctx* c, int what, float* px, float* py) {
+    dev::Collide C{};  // body force of a single sample as the fields use it
+    C.ax = (float)c->params.gx;
+    C.ay = (float)c->params.gy;
+    MLBM_CUDA(launch_observe(c->params.model, what, (int)c->seg_off.size() - 1, c->max_blocks, c->seg_dev,
+                             c->f8[c->cur], c->f0[c->cur], c->ruv[c->cur], C, c->S.coll, c->area, c->mask, px, py,
+                             c->scratch, c->seg_out, c->stream));
+    return MLBM_OK;
+}
+
+// the six field sums over all nodes of a context, as one sample
+mlbm_status sums_of_all(mlbm_ctx* c, double* h) {
+    if (c->seg_off.size() == 2) {
+        MLBM_TRY(observe(c, kObserveFields, nullptr, nullptr));
+        return read_results(c, h, 6);
+    }
+    const size_t ns = c->seg_off.size() - 1;
+    std::vector<double> v(6 * ns);
+    MLBM_TRY(observe(c, kObserveFields, nullptr, nullptr));
+    MLBM_TRY(read_results(c, v.data(), v.size()));
+    std::fill(h, h + 6, 0.0);
+    for (size_t i = 0; i < ns; ++i)
+        for (int q = 0; q < 6; ++q) h[q] += v[6 * i + q];
     return MLBM_OK;
 }
 
@@ -626,19 +685,10 @@ mlbm_status run_steady(mlbm_ctx* c, int mode, double tol, int64_t window, int64_
     std::vector<int64_t> done_at(ns, -1);
     c->steps_in_last_run = 0;
     float* ring = nullptr;
-    double* means = nullptr;
     if (R > 1) {
         if ((double)R * 2.0 * (double)n * 4.0 > 64e9)
             return set_error(MLBM_E_INVALID, nm + ": snapshot ring over 64 GB (use a larger check interval)");
         MLBM_CUDA(cudaMallocAsync(&ring, (size_t)R * 2 * (size_t)n * sizeof(float), c->stream));
-    }
-    if (mode == kMeanVelocity) {
-        cudaError_t e = cudaMallocAsync(&means, 48 * (size_t)ns, c->stream);
-        if (e != cudaSuccess) {
-            if (ring) cudaFreeAsync(ring, c->stream);
-            cudaStreamSynchronize(c->stream);
-            return set_error(MLBM_E_OOM, nm + ": " + cudaGetErrorString(e));
-        }
     }
     // converged samples of a tau = 1 batch are held (see above)
     uint8_t* saved_meta = nullptr;
@@ -664,7 +714,8 @@ mlbm_status run_steady(mlbm_ctx* c, int mode, double tol, int64_t window, int64_
     }
     auto slot_u = [&](int64_t k) { return R > 1 ? ring + (size_t)k * 2 * n : c->px; };
     auto slot_v = [&](int64_t k) { return R > 1 ? ring + ((size_t)k * 2 + 1) * n : c->py; };
-    std::vector<double> h(3 * (size_t)ns), hm(6 * (size_t)ns);
+    const int what = mode == kMeanVelocity ? kObserveBoth : kObserveChange;
+    std::vector<double> h((size_t)what * ns);  // per sample: change sums, then (mean velocity) the field sums
     std::vector<std::vector<double>> hist(ns);  // <u> every `check` steps (mean-velocity criterion)
     // physical time step of each sample: the caller's, else the paper's
     // units (side length 1, kinematic viscosity 1): dt = nu_lb (s / L)^2 with
@@ -676,24 +727,15 @@ mlbm_status run_steady(mlbm_ctx* c, int mode, double tol, int64_t window, int64_
         dts[i] = dt ? dt[i] : (c->seg_params[i].tau - 0.5) / 3.0 * (si / L) * (si / L);
     }
     auto snapshot = [&](int64_t k) -> mlbm_status {
-        MLBM_TRY(fields_to_work(c, nullptr));
+        MLBM_TRY(observe(c, what, slot_u(k), slot_v(k)));
+        MLBM_TRY(read_results(c, h.data(), h.size()));
         for (int i = 0; i < ns; ++i) {
-            const int64_t o = c->seg_off[i], m = c->seg_off[i + 1] - o;
-            MLBM_CUDA(launch_change(c->rho + o, c->ux + o, c->uy + o, slot_u(k) + o, slot_v(k) + o, c->mask + o, m,
-                                    c->scratch, c->seg_out + 3 * i, c->stream));
-            if (means)
-                MLBM_CUDA(launch_reduce_fields(c->rho + o, c->ux + o, c->uy + o, c->area + o, c->mask + o, m,
-                                               c->scratch, means + 6 * i, c->stream));
-        }
-        MLBM_CUDA(cudaMemcpyAsync(h.data(), c->seg_out, 24 * (size_t)ns, cudaMemcpyDeviceToHost, c->stream));
-        if (means) MLBM_CUDA(cudaMemcpyAsync(hm.data(), means, 48 * (size_t)ns, cudaMemcpyDeviceToHost, c->stream));
-        MLBM_TRY(sync(c));
-        for (int i = 0; i < ns; ++i) {
-            if (h[3 * i + 2] != 0.0 || !std::isfinite(h[3 * i]) || !std::isfinite(h[3 * i + 1]))
+            const double* v = &h[(size_t)what * i];
+            if (v[2] != 0.0 || !std::isfinite(v[0]) || !std::isfinite(v[1]))
                 return set_error(MLBM_E_DIVERGED, nm + ": non-positive density or non-finite field in sample " +
                                                       std::to_string(i) + " (" +
-                                                      std::to_string((int64_t)h[3 * i + 2]) + " nodes)");
-            if (means) hist[i].push_back(hm[6 * i + 2] / c->seg_box_area[i]);
+                                                      std::to_string((int64_t)v[2]) + " nodes)");
+            if (mode == kMeanVelocity) hist[i].push_back(v[5] / c->seg_box_area[i]);
         }
         return MLBM_OK;
     };
@@ -713,7 +755,8 @@ mlbm_status run_steady(mlbm_ctx* c, int mode, double tol, int64_t window, int64_
                 if (done_at[i] >= 0) continue;
                 bool steady;
                 if (mode == kFieldNorm) {
-                    const double delta = h[3 * i + 1] > 0 ? std::sqrt(h[3 * i] / h[3 * i + 1]) / (double)window : 0.0;
+                    const double* v = &h[(size_t)what * i];
+                    const double delta = v[1] > 0 ? std::sqrt(v[0] / v[1]) / (double)window : 0.0;
                     steady = delta < tol;
                 } else {
                     const size_t j = hist[i].size() - 1, lag = (size_t)(window / check);
@@ -746,8 +789,7 @@ mlbm_status run_steady(mlbm_ctx* c, int mode, double tol, int64_t window, int64_
     if (saved_meta) cudaFreeAsync(saved_meta, c->stream);
     if (saved_eqv) cudaFreeAsync(saved_eqv, c->stream);
     if (ring) cudaFreeAsync(ring, c->stream);
-    if (means) cudaFreeAsync(means, c->stream);
-    if (ring || means || saved_meta) cudaStreamSynchronize(c->stream);  // also before the next step reads the kinds
+    if (ring || saved_meta) cudaStreamSynchronize(c->stream);  // also before the next step reads the kinds
     if (at)
         for (int i = 0; i < ns; ++i) at[i] = done_at[i];
     return st;
@@ -825,7 +867,7 @@ mlbm_status mlbm_get_populations(mlbm_ctx* c, double* f) {
 
 mlbm_status mlbm_get_fields(mlbm_ctx* c, double* ru) {
     if (!c || !ru) return set_error(MLBM_E_INVALID, "get_fields: NULL argument");
-    MLBM_TRY(fields_to_work(c, c->io));
+    MLBM_TRY(fields_to(c, c->io, 0));
     MLBM_CUDA(cudaMemcpyAsync(ru, c->io, (size_t)c->n * 3 * 8, cudaMemcpyDeviceToHost, c->stream));
     return sync(c);
 }
@@ -896,18 +938,12 @@ double mlbm_last_step_ms(const mlbm_ctx* c) { return c ? c->last_ms : -1.0; }
 
 mlbm_status mlbm_macroscopics(mlbm_ctx* c, double* rho, double* u) {
     if (!c) return set_error(MLBM_E_INVALID, "macroscopics: NULL context");
-    MLBM_TRY(fields_to_work(c, c->io));
-    std::vector<double> ru((size_t)c->n * 3);
-    MLBM_CUDA(cudaMemcpyAsync(ru.data(), c->io, ru.size() * 8, cudaMemcpyDeviceToHost, c->stream));
-    MLBM_TRY(sync(c));
-    for (int64_t i = 0; i < c->n; ++i) {
-        if (rho) rho[i] = ru[i * 3];
-        if (u) {
-            u[2 * i] = ru[i * 3 + 1];
-            u[2 * i + 1] = ru[i * 3 + 2];
-        }
-    }
-    return MLBM_OK;
+    if (!rho && !u) return sync(c);
+    MLBM_TRY(fields_to(c, c->io, 1));
+    const size_t n = (size_t)c->n;
+    if (rho) MLBM_CUDA(cudaMemcpyAsync(rho, c->io, n * 8, cudaMemcpyDeviceToHost, c->stream));
+    if (u) MLBM_CUDA(cudaMemcpyAsync(u, c->io + n, n * 16, cudaMemcpyDeviceToHost, c->stream));
+    return sync(c);
 }
 
 mlbm_status mlbm_wall_stress_force(mlbm_ctx* c, const int64_t* nodes, const double* normals, const double* ds,
@@ -980,9 +1016,8 @@ mlbm_status mlbm_drag_lift(mlbm_ctx* c, double ref_length, double u_ref, double*
     double h[2] = {0, 0};
     if (c->n_link_nodes > 0) {
         MLBM_CUDA(launch_force(c->S, c->params.model, c->n_link_nodes, c->link_nodes, c->area_over_s2,
-                               c->f8[c->cur], c->ruv[c->cur], c->C, c->scratch, c->small, c->stream));
-        MLBM_CUDA(cudaMemcpyAsync(h, c->small, 16, cudaMemcpyDeviceToHost, c->stream));
-        MLBM_TRY(sync(c));
+                               c->f8[c->cur], c->ruv[c->cur], c->C, c->scratch, c->seg_out, c->stream));
+        MLBM_TRY(read_results(c, h, 2));
     }
     if (fx) *fx = h[0];
     if (fy) *fy = h[1];
@@ -995,11 +1030,8 @@ mlbm_status mlbm_drag_lift(mlbm_ctx* c, double ref_length, double u_ref, double*
 
 mlbm_status mlbm_permeability(mlbm_ctx* c, double* k, double* us, double* ui, double* tort) {
     if (!c) return set_error(MLBM_E_INVALID, "permeability: NULL context");
-    MLBM_TRY(fields_to_work(c, nullptr));
-    MLBM_CUDA(launch_reduce_fields(c->rho, c->ux, c->uy, c->area, c->mask, c->n, c->scratch, c->small, c->stream));
     double h[6];
-    MLBM_CUDA(cudaMemcpyAsync(h, c->small, 48, cudaMemcpyDeviceToHost, c->stream));
-    MLBM_TRY(sync(c));
+    MLBM_TRY(sums_of_all(c, h));
     const double sup = h[2] / c->box_area;
     const double gmag = std::sqrt(c->params.gx * c->params.gx + c->params.gy * c->params.gy);
     const double nu = (c->params.tau - 0.5) / 3.0;
@@ -1357,15 +1389,9 @@ mlbm_status mlbm_batch_range(const mlbm_ctx* c, int sample, int64_t* first, int6
 mlbm_status mlbm_batch_permeability(mlbm_ctx* c, double* k, double* us, double* ui, double* tort) {
     if (!c) return set_error(MLBM_E_INVALID, "batch_permeability: NULL context");
     const int ns = (int)c->seg_off.size() - 1;
-    MLBM_TRY(fields_to_work(c, nullptr));
-    for (int i = 0; i < ns; ++i) {
-        const int64_t o = c->seg_off[i], m = c->seg_off[i + 1] - o;
-        MLBM_CUDA(launch_reduce_fields(c->rho + o, c->ux + o, c->uy + o, c->area + o, c->mask + o, m, c->scratch,
-                                       c->seg_out + 6 * i, c->stream));
-    }
     std::vector<double> h(6 * (size_t)ns);
-    MLBM_CUDA(cudaMemcpyAsync(h.data(), c->seg_out, h.size() * 8, cudaMemcpyDeviceToHost, c->stream));
-    MLBM_TRY(sync(c));
+    MLBM_TRY(observe(c, kObserveFields, nullptr, nullptr));
+    MLBM_TRY(read_results(c, h.data(), h.size()));
     for (int i = 0; i < ns; ++i) {
         const double* v = &h[6 * (size_t)i];
         const mlbm_params& p = c->seg_params[i];
@@ -1402,16 +1428,7 @@ mlbm_status mlbm_batch_drag_lift(mlbm_ctx* c, const double* ref_length, const do
     const int ns = (int)c->seg_off.size() - 1;
     // link nodes are listed in position order and samples own contiguous
     // position ranges, so each sample's links are a contiguous slice
-    std::vector<int> lo(ns + 1, 0);
-    {
-        std::vector<int> hl(c->n_link_nodes);
-        if (c->n_link_nodes)
-            MLBM_CUDA(cudaMemcpyAsync(hl.data(), c->link_nodes, hl.size() * 4, cudaMemcpyDeviceToHost, c->stream));
-        MLBM_TRY(sync(c));
-        for (int i = 0; i <= ns; ++i)
-            lo[i] = (int)(std::lower_bound(hl.begin(), hl.end(), (int)c->seg_off[i]) - hl.begin());
-    }
-    std::vector<double> h(2 * (size_t)ns, 0.0);
+    const std::vector<int>& lo = c->link_off;
     for (int i = 0; i < ns; ++i) {
         const int m = lo[i + 1] - lo[i];
         if (m == 0) continue;
@@ -1419,8 +1436,7 @@ mlbm_status mlbm_batch_drag_lift(mlbm_ctx* c, const double* ref_length, const do
                                c->ruv[c->cur], c->C, c->scratch, c->seg_out + 2 * i, c->stream));
     }
     std::vector<double> dv(2 * (size_t)ns);
-    MLBM_CUDA(cudaMemcpyAsync(dv.data(), c->seg_out, dv.size() * 8, cudaMemcpyDeviceToHost, c->stream));
-    MLBM_TRY(sync(c));
+    MLBM_TRY(read_results(c, dv.data(), dv.size()));
     for (int i = 0; i < ns; ++i) {
         const bool any = lo[i + 1] > lo[i];
         const double Fx = any ? dv[2 * i] : 0.0, Fy = any ? dv[2 * i + 1] : 0.0;
@@ -1475,22 +1491,12 @@ mlbm_status mlbm_warm_start(mlbm_ctx* c, mlbm_mlp* m, const float* X, const doub
     if (st != MLBM_OK) return release(st);
     e = launch_warm_check(n, c->perm, c->S.node_sample, c->meta, Y, no, dscale_u, dscale_r, 0.3f, 0.1f, flag,
                           c->stream);
-    std::vector<double> hmean(ns, 0.0);
     if (e == cudaSuccess && no == 3) {
         // area-weighted mean of the predicted density deviation per sample
         e = launch_warm_drho(n, c->perm, c->S.node_sample, c->meta, Y, no, dscale_r, c->rho, c->stream);
-        std::vector<double> sums(6 * (size_t)ns);
-        for (int i = 0; i < ns && e == cudaSuccess; ++i) {
-            const int64_t o = c->seg_off[i], cnt = c->seg_off[i + 1] - o;
-            e = launch_reduce_fields(c->rho + o, c->ux + o, c->uy + o, c->area + o, c->mask + o, cnt, c->scratch,
-                                     c->seg_out + 6 * i, c->stream);
-        }
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(sums.data(), c->seg_out, 48 * (size_t)ns, cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        for (int i = 0; i < ns && e == cudaSuccess; ++i) hmean[i] = sums[6 * i] > 0 ? sums[6 * i + 1] / sums[6 * i] : 0.0;
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(dmean, hmean.data(), 8 * (size_t)ns, cudaMemcpyHostToDevice, c->stream);
+            e = launch_warm_means(ns, c->max_blocks, c->seg_dev, c->rho, c->area, c->mask, c->scratch, dmean,
+                                  c->stream);
     }
     if (e == cudaSuccess)
         e = launch_warm_fill(n, c->perm, c->S.node_sample, c->meta, c->eqv, Y, no, dscale_u, c->rho, dmean, flag, c->io,
@@ -1869,7 +1875,7 @@ static mlbm_status part_set(mlbm_part* P, const double* v, int width, bool field
 
 static mlbm_status part_get(mlbm_part* P, double* v, int width, bool fields) {
     for (mlbm_ctx* c : P->ctx) {
-        if (fields) MLBM_TRY(fields_to_work(c, P->io));
+        if (fields) MLBM_TRY(fields_to(c, P->io, 0));
         else MLBM_CUDA(launch_get_bgk((int)c->n, c->perm, c->f8[c->cur], c->f0[c->cur], P->io, P->stream));
     }
     MLBM_CUDA(cudaMemcpyAsync(v, P->io, (size_t)P->n * width * 8, cudaMemcpyDeviceToHost, P->stream));
@@ -1904,11 +1910,8 @@ mlbm_status mlbm_part_permeability(mlbm_part* P, double* k, double* us, double* 
     // all-reduce of a run whose partitions live on separate devices)
     double tot[6] = {0, 0, 0, 0, 0, 0};
     for (mlbm_ctx* c : P->ctx) {
-        MLBM_TRY(fields_to_work(c, nullptr));
-        MLBM_CUDA(launch_reduce_fields(c->rho, c->ux, c->uy, c->area, c->mask, c->n, c->scratch, c->small, c->stream));
         double h[6];
-        MLBM_CUDA(cudaMemcpyAsync(h, c->small, 48, cudaMemcpyDeviceToHost, c->stream));
-        MLBM_TRY(sync(c));
+        MLBM_TRY(sums_of_all(c, h));
         for (int i = 0; i < 6; ++i) tot[i] += h[i];
     }
     const mlbm_params& pp = P->ctx[0]->params;

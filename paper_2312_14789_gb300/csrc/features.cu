@@ -198,6 +198,50 @@ __global__ void warm_drho(int n, const int* __restrict__ perm, const uint16_t* _
     drho[p] = (meta[p] & 3) == 2 ? 0.f : (float)(scale_rho[smp] * (double)Y[no * (int64_t)perm[p] + 2]);
 }
 
+// area-weighted mean of drho over every sample's masked nodes (0 without any):
+// partial sums of A and drho A per block, then one block per sample
+__global__ void __launch_bounds__(256) warm_means_partial(const int64_t* __restrict__ seg, int max_nb,
+                                                          const float* __restrict__ drho,
+                                                          const float* __restrict__ area,
+                                                          const uint8_t* __restrict__ mask,
+                                                          double* __restrict__ partial) {
+    const int64_t first = seg[blockIdx.y], end = seg[blockIdx.y + 1];
+    double a = 0.0, d = 0.0;
+    for (int64_t i = first + blockIdx.x * 256LL + threadIdx.x; i < end; i += (int64_t)max_nb * 256)
+        if (mask[i]) {
+            a += area[i];
+            d += (double)drho[i] * area[i];
+        }
+    __shared__ double sa[256], sd[256];
+    sa[threadIdx.x] = a;
+    sd[threadIdx.x] = d;
+    __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+        if ((int)threadIdx.x < h) {
+            sa[threadIdx.x] += sa[threadIdx.x + h];
+            sd[threadIdx.x] += sd[threadIdx.x + h];
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        partial[2 * ((size_t)blockIdx.y * max_nb + blockIdx.x)] = sa[0];
+        partial[2 * ((size_t)blockIdx.y * max_nb + blockIdx.x) + 1] = sd[0];
+    }
+}
+__global__ void __launch_bounds__(32) warm_means_final(int max_nb, const double* __restrict__ partial,
+                                                       double* __restrict__ mean) {
+    double a = 0.0, d = 0.0;
+    for (int b = threadIdx.x; b < max_nb; b += 32) {
+        a += partial[2 * ((size_t)blockIdx.x * max_nb + b)];
+        d += partial[2 * ((size_t)blockIdx.x * max_nb + b) + 1];
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        d += __shfl_xor_sync(0xffffffffu, d, o);
+    }
+    if (threadIdx.x == 0) mean[blockIdx.x] = a > 0.0 ? d / a : 0.0;
+}
+
 // rho_u[n][3] (caller order, FP64) of the warm start: rho = 1 + (predicted
 // deviation - its area-weighted sample mean, so the sample's mass stays that
 // of the rest state) and u = predicted velocity; samples flagged cold start
@@ -241,6 +285,13 @@ cudaError_t launch_warm_drho(int n, const int* perm, const uint16_t* node_sample
                              const float* Y, int no, const double* scale_rho, float* drho, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     dev::warm_drho<<<(n + 255) / 256, 256, 0, st>>>(n, perm, node_sample, meta, Y, no, scale_rho, drho);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_warm_means(int ns, int max_nb, const int64_t* seg, const float* drho, const float* area,
+                              const uint8_t* mask, double* partial, double* mean, cudaStream_t st) {
+    dev::warm_means_partial<<<dim3(max_nb, ns), 256, 0, st>>>(seg, max_nb, drho, area, mask, partial);
+    dev::warm_means_final<<<ns, 32, 0, st>>>(max_nb, partial, mean);
     return cudaGetLastError();
 }
 

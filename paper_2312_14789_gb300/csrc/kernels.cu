@@ -7,6 +7,7 @@
 #include <cstdio>
 
 #include "device_common.cuh"
+#include "float_sums.cuh"
 #include "kernels.h"
 #include "launch_util.cuh"
 
@@ -83,50 +84,47 @@ __global__ void get_tau1_to_f64(int n, const int* __restrict__ perm, const float
     v[2] = a.z;
 }
 
-// rho, u of the state into FP32 sorted-order arrays (and optionally FP64
-// caller-order rho_u[n][3]).  BGK: rho = sum f, rho u = sum f e - rho a / 2.
+// (rho - 1, ux, uy) of a BGK state: rho = sum f, rho u = sum f e - rho a / 2
+__device__ __forceinline__ void bgk_moments(const float4& a, const float4& b, float g0, float ax, float ay, float& dr,
+                                            float& ux, float& uy) {
+    dr = g0 + (a.x + a.y + a.z + a.w) + (b.x + b.y + b.z + b.w);
+    const float jx = (a.x - a.z) + (b.x - b.y) + (b.w - b.z);
+    const float jy = (a.y - a.w) + (b.x + b.y) - (b.z + b.w);
+    const float rho = 1.0f + dr;
+    ux = jx / rho - 0.5f * ax;
+    uy = jy / rho - 0.5f * ay;
+}
+
+// (rho, ux, uy) of caller's node i of n into FP64 caller-order arrays: rows
+// [n][3], or (split) rho[n] followed by u[n][2]
+__device__ __forceinline__ void put_fields(double* out, int split, int n, int i, double rho, float ux, float uy) {
+    double* r = split ? out + i : out + 3 * (size_t)i;
+    double* u = split ? out + (size_t)n + 2 * (size_t)i : r + 1;
+    r[0] = rho;
+    u[0] = ux;
+    u[1] = uy;
+}
+
+// rho, u of the state into FP64 caller-order arrays
 __global__ void macroscopics_bgk(int n, const int* __restrict__ perm, const float4* __restrict__ f8,
                                  const float* __restrict__ f0, float ax0, float ay0,
-                                 const uint16_t* __restrict__ node_sample, const Collide* __restrict__ coll,
-                                 float* __restrict__ rho_o, float* __restrict__ ux_o, float* __restrict__ uy_o,
-                                 double* __restrict__ ru) {
+                                 const uint16_t* __restrict__ node_sample, const Collide* __restrict__ coll, int split,
+                                 double* __restrict__ out) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const float ax = node_sample ? coll[node_sample[p]].ax : ax0;
     const float ay = node_sample ? coll[node_sample[p]].ay : ay0;
-    const float4 a = f8[2 * (size_t)p], b = f8[2 * (size_t)p + 1];
-    const float g0 = f0[p];
-    const float dr = g0 + (a.x + a.y + a.z + a.w) + (b.x + b.y + b.z + b.w);
-    const float jx = (a.x - a.z) + (b.x - b.y) + (b.w - b.z);
-    const float jy = (a.y - a.w) + (b.x + b.y) - (b.z + b.w);
-    const float rho = 1.0f + dr;
-    const float ux = jx / rho - 0.5f * ax, uy = jy / rho - 0.5f * ay;
-    rho_o[p] = rho;
-    ux_o[p] = ux;
-    uy_o[p] = uy;
-    if (ru) {
-        double* v = ru + 3 * (size_t)perm[p];
-        v[0] = 1.0 + (double)dr;
-        v[1] = ux;
-        v[2] = uy;
-    }
+    float dr, ux, uy;
+    bgk_moments(f8[2 * (size_t)p], f8[2 * (size_t)p + 1], f0[p], ax, ay, dr, ux, uy);
+    put_fields(out, split, n, perm[p], 1.0 + (double)dr, ux, uy);
 }
 
-__global__ void macroscopics_tau1(int n, const int* __restrict__ perm, const float4* __restrict__ s,
-                                  float* __restrict__ rho_o, float* __restrict__ ux_o, float* __restrict__ uy_o,
-                                  double* __restrict__ ru) {
+__global__ void macroscopics_tau1(int n, const int* __restrict__ perm, const float4* __restrict__ s, int split,
+                                  double* __restrict__ out) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const float4 a = s[p];
-    rho_o[p] = 1.0f + a.x;
-    ux_o[p] = a.y;
-    uy_o[p] = a.z;
-    if (ru) {
-        double* v = ru + 3 * (size_t)perm[p];
-        v[0] = 1.0 + (double)a.x;
-        v[1] = a.y;
-        v[2] = a.z;
-    }
+    put_fields(out, split, n, perm[p], 1.0 + (double)a.x, a.y, a.z);
 }
 
 // --------------------------------------------------------- wall force
@@ -264,123 +262,159 @@ __global__ void __launch_bounds__(128) force_kernel(Stencil S, int model, int n_
     }
 }
 
-__global__ void sum_pairs(int nb, const double* __restrict__ partial, double* __restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double a = 0, b = 0;
-        for (int i = 0; i < nb; ++i) { a += partial[2 * i]; b += partial[2 * i + 1]; }
-        out[0] = a;
-        out[1] = b;
+// fixed-order sums of nb partial W-tuples (one block of 256)
+template <int W>
+__device__ __forceinline__ void sum_tuples(int nb, const double* __restrict__ partial, double* __restrict__ out) {
+    double s[W];
+#pragma unroll
+    for (int q = 0; q < W; ++q) s[q] = 0.0;
+    for (int b = threadIdx.x; b < nb; b += 256)
+#pragma unroll
+        for (int q = 0; q < W; ++q) s[q] += partial[W * (size_t)b + q];
+    __shared__ double sh[W][256];
+#pragma unroll
+    for (int q = 0; q < W; ++q) sh[q][threadIdx.x] = s[q];
+    __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+        if ((int)threadIdx.x < h)
+#pragma unroll
+            for (int q = 0; q < W; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + h];
+        __syncthreads();
     }
+    if (threadIdx.x < W) out[threadIdx.x] = sh[threadIdx.x][0];
+}
+
+__global__ void __launch_bounds__(256) sum_pairs(int nb, const double* __restrict__ partial,
+                                                 double* __restrict__ out) {
+    sum_tuples<2>(nb, partial, out);
 }
 
 // ------------------------------------------------------------ reductions
 // Six area-weighted FP64 sums: A, rho A, ux A, uy A, |u| A, |u|^2 A.
 constexpr int kRedThreads = 256;
 
-__global__ void __launch_bounds__(kRedThreads) reduce_fields_partial(int64_t n, const float* __restrict__ rho,
+// the block's sums of s[W] into out[W], in a fixed order
+template <int W>
+__device__ __forceinline__ void block_tuple(const double* s, double* __restrict__ out) {
+    __shared__ double sh[W][kRedThreads];
+#pragma unroll
+    for (int q = 0; q < W; ++q) sh[q][threadIdx.x] = s[q];
+    __syncthreads();
+    for (int h = kRedThreads / 2; h > 0; h >>= 1) {
+        if ((int)threadIdx.x < h)
+#pragma unroll
+            for (int q = 0; q < W; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + h];
+        __syncthreads();
+    }
+    if (threadIdx.x < W) out[threadIdx.x] = sh[threadIdx.x][0];
+}
+
+__global__ void __launch_bounds__(kRedThreads, 4) reduce_fields_partial(int64_t n, const float* __restrict__ rho,
                                                                       const float* __restrict__ ux,
                                                                       const float* __restrict__ uy,
                                                                       const float* __restrict__ area,
                                                                       const uint8_t* __restrict__ mask,
                                                                       double* __restrict__ partial) {
-    double s[6] = {0, 0, 0, 0, 0, 0};
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        if (mask && !mask[i]) continue;
-        const double a = area[i], u = ux[i], v = uy[i];
-        const double m2 = u * u + v * v;
-        s[0] += a;
-        s[1] += (double)rho[i] * a;
-        s[2] += u * a;
-        s[3] += v * a;
-        s[4] += sqrt(m2) * a;
-        s[5] += m2 * a;
-    }
-    __shared__ double sh[6][kRedThreads];
+    FieldSums t;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    // four nodes' loads in flight; the sums go on in node order
+    for (; i + 3 * stride < n; i += 4 * stride) {
+        float r[4], u[4], v[4], a[4];
+        uint8_t m[4];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) sh[q][threadIdx.x] = s[q];
-    __syncthreads();
-    for (int h = kRedThreads / 2; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h)
+        for (int j = 0; j < 4; ++j) {
+            const int64_t k = i + j * stride;
+            m[j] = mask ? mask[k] : 1;
+            r[j] = rho[k];
+            u[j] = ux[k];
+            v[j] = uy[k];
+            a[j] = area[k];
+        }
 #pragma unroll
-            for (int q = 0; q < 6; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + h];
-        __syncthreads();
+        for (int j = 0; j < 4; ++j)
+            if (m[j]) t.add(r[j], u[j], v[j], a[j]);
     }
-    if (threadIdx.x < 6) partial[6 * (size_t)blockIdx.x + threadIdx.x] = sh[threadIdx.x][0];
+    for (; i < n; i += stride)
+        if (!mask || mask[i]) t.add(rho[i], ux[i], uy[i], area[i]);
+    t.flush();
+    block_tuple<6>(t.s, partial + 6 * (size_t)blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kRedThreads) reduce_fields_final(int nb, const double* __restrict__ partial,
                                                                     double* __restrict__ out) {
-    double s[6] = {0, 0, 0, 0, 0, 0};
-    for (int b = threadIdx.x; b < nb; b += blockDim.x)
-#pragma unroll
-        for (int q = 0; q < 6; ++q) s[q] += partial[6 * (size_t)b + q];
-    __shared__ double sh[6][kRedThreads];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) sh[q][threadIdx.x] = s[q];
-    __syncthreads();
-    for (int h = kRedThreads / 2; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h)
-#pragma unroll
-            for (int q = 0; q < 6; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + h];
-        __syncthreads();
-    }
-    if (threadIdx.x < 6) out[threadIdx.x] = sh[threadIdx.x][0];
+    sum_tuples<6>(nb, partial, out);
 }
 
-// over masked nodes: sum |u - u_prev|^2, sum |u|^2, and the number of nodes
-// whose density is not positive or whose fields are not finite; then copy u
-// into u_prev
-__global__ void __launch_bounds__(kRedThreads) change_partial(int64_t n, const float* __restrict__ rho,
-                                                               const float* __restrict__ ux,
-                                                               const float* __restrict__ uy,
-                                                               float* __restrict__ px, float* __restrict__ py,
-                                                               const uint8_t* __restrict__ mask,
-                                                               double* __restrict__ partial) {
-    double d = 0, m = 0, bad = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float u = ux[i], v = uy[i];
-        if (!mask || mask[i]) {
-            const float r = rho[i];
-            if (!(r > 0.f) || !isfinite(r) || !isfinite(u) || !isfinite(v)) bad += 1.0;
-            const double du = (double)u - px[i], dv = (double)v - py[i];
-            d += du * du + dv * dv;
-            m += (double)u * u + (double)v * v;
+// Observables of every sample of a context in one launch, straight from the
+// state (blockIdx.y is the sample; each has the block count it would have on
+// its own, so its sums do not depend on the batch).
+//   CHANGE: over masked nodes sum |u - u_prev|^2, sum |u|^2 and the number of
+//   nodes whose density is not positive or whose fields are not finite, then
+//   u into u_prev;  FIELDS: the six sums above.
+// Partials [sample][max_nb][W], W = 3 or 6 (CHANGE first when both, W = 9).
+__device__ __forceinline__ int blocks_of(int64_t m) {
+    const int64_t b = (m + 4 * kRedThreads - 1) / (4 * kRedThreads);
+    return (int)(b < 1 ? 1 : (b > kReduceMaxBlocks ? kReduceMaxBlocks : b));
+}
+template <int MODEL, bool CHANGE, bool FIELDS>
+__global__ void __launch_bounds__(kRedThreads) observe_partial(const int64_t* __restrict__ seg, int max_nb,
+                                                                const float4* __restrict__ st,
+                                                                const float* __restrict__ f0, float ax0, float ay0,
+                                                                const Collide* __restrict__ coll,
+                                                                const float* __restrict__ area,
+                                                                const uint8_t* __restrict__ mask,
+                                                                float* __restrict__ px, float* __restrict__ py,
+                                                                double* __restrict__ partial) {
+    constexpr int W = (CHANGE ? 3 : 0) + (FIELDS ? 6 : 0);
+    const int smp = blockIdx.y;
+    const int64_t first = seg[smp], end = seg[smp + 1];
+    const int nb = blocks_of(end - first);
+    if ((int)blockIdx.x >= nb) return;
+    const float ax = coll ? coll[smp].ax : ax0, ay = coll ? coll[smp].ay : ay0;
+    double s[W];
+#pragma unroll
+    for (int q = 0; q < W; ++q) s[q] = 0.0;
+    FieldSums t;
+    for (int64_t i = first + blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < end; i += (int64_t)nb * kRedThreads) {
+        float rho, u, v;
+        if (MODEL == 0) {
+            float dr;
+            bgk_moments(st[2 * i], st[2 * i + 1], f0[i], ax, ay, dr, u, v);
+            rho = 1.0f + dr;
+        } else {
+            const float4 a = st[i];
+            rho = 1.0f + a.x;
+            u = a.y;
+            v = a.z;
         }
-        px[i] = u;
-        py[i] = v;
-    }
-    __shared__ double sd[kRedThreads], sm[kRedThreads], sb[kRedThreads];
-    sd[threadIdx.x] = d;
-    sm[threadIdx.x] = m;
-    sb[threadIdx.x] = bad;
-    __syncthreads();
-    for (int h = kRedThreads / 2; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h) {
-            sd[threadIdx.x] += sd[threadIdx.x + h];
-            sm[threadIdx.x] += sm[threadIdx.x + h];
-            sb[threadIdx.x] += sb[threadIdx.x + h];
+        if (mask[i]) {
+            if (CHANGE) {
+                if (!(rho > 0.f) || !isfinite(rho) || !isfinite(u) || !isfinite(v)) s[2] += 1.0;
+                const double du = (double)u - px[i], dv = (double)v - py[i];
+                s[0] += du * du + dv * dv;
+                s[1] += (double)u * u + (double)v * v;
+            }
+            if (FIELDS) t.add(rho, u, v, area[i]);
         }
-        __syncthreads();
+        if (CHANGE) {
+            px[i] = u;
+            py[i] = v;
+        }
     }
-    if (threadIdx.x == 0) {
-        partial[3 * (size_t)blockIdx.x] = sd[0];
-        partial[3 * (size_t)blockIdx.x + 1] = sm[0];
-        partial[3 * (size_t)blockIdx.x + 2] = sb[0];
+    if (FIELDS) {
+        t.flush();
+#pragma unroll
+        for (int q = 0; q < 6; ++q) s[(CHANGE ? 3 : 0) + q] = t.s[q];
     }
+    block_tuple<W>(s, partial + W * ((size_t)smp * max_nb + blockIdx.x));
 }
 
-__global__ void sum_triples(int nb, const double* __restrict__ partial, double* __restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double a = 0, b = 0, c = 0;
-        for (int i = 0; i < nb; ++i) {
-            a += partial[3 * i];
-            b += partial[3 * i + 1];
-            c += partial[3 * i + 2];
-        }
-        out[0] = a;
-        out[1] = b;
-        out[2] = c;
-    }
+template <int W>
+__global__ void __launch_bounds__(256) observe_final(const int64_t* __restrict__ seg, int max_nb,
+                                                     const double* __restrict__ partial, double* __restrict__ out) {
+    const int smp = blockIdx.x;
+    sum_tuples<W>(blocks_of(seg[smp + 1] - seg[smp]), partial + W * ((size_t)smp * max_nb), out + W * (size_t)smp);
 }
 
 }  // namespace dev
@@ -413,14 +447,13 @@ cudaError_t launch_get_tau1(int n, const int* perm, const float4* s, double* ru,
 }
 cudaError_t launch_macroscopics(int model, int n, const int* perm, const float4* f8, const float* f0,
                                 const float4* ruv, float ax, float ay, const uint16_t* node_sample,
-                                const dev::Collide* coll, float* rho, float* ux, float* uy, double* ru,
-                                cudaStream_t st) {
+                                const dev::Collide* coll, int split, double* out, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     if (model == 0)
-        dev::macroscopics_bgk<<<blocks_for(n, 256), 256, 0, st>>>(n, perm, f8, f0, ax, ay, node_sample, coll, rho, ux,
-                                                                   uy, ru);
+        dev::macroscopics_bgk<<<blocks_for(n, 256), 256, 0, st>>>(n, perm, f8, f0, ax, ay, node_sample, coll, split,
+                                                                   out);
     else
-        dev::macroscopics_tau1<<<blocks_for(n, 256), 256, 0, st>>>(n, perm, ruv, rho, ux, uy, ru);
+        dev::macroscopics_tau1<<<blocks_for(n, 256), 256, 0, st>>>(n, perm, ruv, split, out);
     return cudaGetLastError();
 }
 
@@ -435,7 +468,7 @@ cudaError_t launch_force(const dev::Stencil& S, int model, int n_link_nodes, con
     } else {
         MLBM_DISPATCH_KQ(S.Kq, (dev::force_kernel<KQC><<<nb, 128, 0, st>>>(S, model, n_link_nodes, link_nodes, area_over_s2, f8, ruv, C, partial)));
     }
-    dev::sum_pairs<<<1, 32, 0, st>>>(nb, partial, out);
+    dev::sum_pairs<<<1, 256, 0, st>>>(nb, partial, out);
     return cudaGetLastError();
 }
 
@@ -446,19 +479,34 @@ int reduce_blocks(int64_t n) {
 
 cudaError_t launch_reduce_fields(const float* rho, const float* ux, const float* uy, const float* area,
                                  const uint8_t* mask, int64_t n, double* partial, double* out, cudaStream_t st) {
-    const int nb = reduce_blocks(n);
+    // no more blocks than are resident at once: a second, partial round of them
+    // would cost as much as the first
+    const int nb = std::min(reduce_blocks(n), 4 * 152);
     dev::reduce_fields_partial<<<nb, dev::kRedThreads, 0, st>>>(n, rho, ux, uy, area, mask, partial);
     dev::reduce_fields_final<<<1, dev::kRedThreads, 0, st>>>(nb, partial, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_change(const float* rho, const float* ux, const float* uy, float* px, float* py,
-                          const uint8_t* mask, int64_t n, double* partial, double* out, cudaStream_t st) {
-    const int nb = reduce_blocks(n);
-    dev::change_partial<<<nb, dev::kRedThreads, 0, st>>>(n, rho, ux, uy, px, py, mask, partial);
-    dev::sum_triples<<<1, 32, 0, st>>>(nb, partial, out);
+cudaError_t launch_observe(int model, int what, int ns, int max_nb, const int64_t* seg, const float4* f8,
+                           const float* f0, const float4* ruv, const dev::Collide& C, const dev::Collide* coll,
+                           const float* area, const uint8_t* mask, float* px, float* py, double* partial, double* out,
+                           cudaStream_t st) {
+    const dim3 grid(max_nb, ns);
+    auto run = [&](auto first, auto last) {
+        first<<<grid, dev::kRedThreads, 0, st>>>(seg, max_nb, model == 0 ? f8 : ruv, f0, C.ax, C.ay, coll, area, mask,
+                                                 px, py, partial);
+        last<<<ns, 256, 0, st>>>(seg, max_nb, partial, out);
+    };
+    if (what == kObserveChange)
+        model == 0 ? run(dev::observe_partial<0, true, false>, dev::observe_final<3>)
+                   : run(dev::observe_partial<1, true, false>, dev::observe_final<3>);
+    else if (what == kObserveFields)
+        model == 0 ? run(dev::observe_partial<0, false, true>, dev::observe_final<6>)
+                   : run(dev::observe_partial<1, false, true>, dev::observe_final<6>);
+    else
+        model == 0 ? run(dev::observe_partial<0, true, true>, dev::observe_final<9>)
+                   : run(dev::observe_partial<1, true, true>, dev::observe_final<9>);
     return cudaGetLastError();
 }
-
 
 }  // namespace mlbm

@@ -63,8 +63,7 @@ cudaError_t launch_step_warp(int variant, int model, const dev::Stencil& S, cons
 cudaError_t launch_get_tau1(int n, const int* perm, const float4* s, double* ru, cudaStream_t st);
 cudaError_t launch_macroscopics(int model, int n, const int* perm, const float4* f8, const float* f0,
                                 const float4* ruv, float ax, float ay, const uint16_t* node_sample,
-                                const dev::Collide* coll, float* rho, float* ux, float* uy, double* ru,
-                                cudaStream_t st);
+                                const dev::Collide* coll, int split, double* out, cudaStream_t st);
 // persistent bulk-copy pipelined step (kernels_tma.cu), variants 4..7
 bool tma_supported(int Kq);
 cudaError_t launch_step_tma(int variant, int model, const dev::Stencil& S, const float4* f8in, const float* f0in,
@@ -79,10 +78,17 @@ constexpr int kReduceMaxBlocks = 1024;
 int reduce_blocks(int64_t n);
 cudaError_t launch_reduce_fields(const float* rho, const float* ux, const float* uy, const float* area,
                                  const uint8_t* mask, int64_t n, double* partial, double* out, cudaStream_t st);
-// per sample: sum |u - u_prev|^2, sum |u|^2 and the count of nodes with a
-// non-positive density or non-finite field (3 doubles into out); u -> u_prev
-cudaError_t launch_change(const float* rho, const float* ux, const float* uy, float* px, float* py,
-                          const uint8_t* mask, int64_t n, double* partial, double* out, cudaStream_t st);
+// observables of all samples of a context from its state, `out` [sample][W]:
+// kObserveChange (W = 3) sum |u - u_prev|^2, sum |u|^2 and the count of nodes
+// with a non-positive density or non-finite field, then u -> u_prev (px, py);
+// kObserveFields (W = 6) the sums of launch_reduce_fields; kObserveBoth (W =
+// 9).  seg (device): first position of each sample and the end; max_nb:
+// reduce_blocks of the largest sample; partial: ns * max_nb * W doubles
+enum { kObserveChange = 3, kObserveFields = 6, kObserveBoth = 9 };
+cudaError_t launch_observe(int model, int what, int ns, int max_nb, const int64_t* seg, const float4* f8,
+                           const float* f0, const float4* ruv, const dev::Collide& C, const dev::Collide* coll,
+                           const float* area, const uint8_t* mask, float* px, float* py, double* partial, double* out,
+                           cudaStream_t st);
 
 // warm start (features.cu)
 cudaError_t launch_warm_check(int n, const int* perm, const uint16_t* node_sample, const uint8_t* meta,
@@ -90,6 +96,10 @@ cudaError_t launch_warm_check(int n, const int* perm, const uint16_t* node_sampl
                               float drho_max, int* flag, cudaStream_t st);
 cudaError_t launch_warm_drho(int n, const int* perm, const uint16_t* node_sample, const uint8_t* meta,
                              const float* Y, int no, const double* scale_rho, float* drho, cudaStream_t st);
+// area-weighted mean of drho per sample (0 where the areas sum to nothing);
+// partial: 2 * ns * max_nb doubles
+cudaError_t launch_warm_means(int ns, int max_nb, const int64_t* seg, const float* drho, const float* area,
+                              const uint8_t* mask, double* partial, double* mean, cudaStream_t st);
 cudaError_t launch_warm_fill(int n, const int* perm, const uint16_t* node_sample, const uint8_t* meta,
                              const float4* eqv, const float* Y, int no, const double* scale_u, const float* drho,
                              const double* drho_mean, const int* flag, double* ru, cudaStream_t st);
