@@ -30,7 +30,9 @@
 // SM (143 KB of shared memory a block for two weight copies and gradient
 // accumulators), 2-byte transposed staging stores, dW accumulated in shared
 // memory, uncoalesced weight conversion in every block and 304 partials summed
-// one after the other took 133 us a step; this form takes 36 us.
+// one after the other took 133 us a step; this form took 36 us, and 34 us since
+// a round's rows are drawn and read while the round before adds its dW (twelve
+// warps a block, 168 registers, took 37 us).
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -142,10 +144,9 @@ __device__ __forceinline__ int64_t data_row(int64_t r, int64_t n_data, uint64_t 
     return (int64_t)(z % (uint64_t)n_data);
 }
 
-// A fragment of the feature tile (rows g, g + 8 of the warp's 16 rows);
+// this lane's features of the tile (rows g, g + 8 of the warp's 16 rows);
 // src0 / src1: data rows of those two rows, -1 for padding
-__device__ __forceinline__ void load_x(const float* __restrict__ X, int64_t src0, int64_t src1, int t, uint32_t* a) {
-    float v[8];
+__device__ __forceinline__ void read_x(const float* __restrict__ X, int64_t src0, int64_t src1, int t, float* v) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] = 0.f;
     if (src0 >= 0) {
@@ -158,6 +159,10 @@ __device__ __forceinline__ void load_x(const float* __restrict__ X, int64_t src0
         v[2] = x[2 * t]; v[3] = x[2 * t + 1];
         v[6] = x[2 * t + 8]; v[7] = x[2 * t + 9];
     }
+}
+
+// ... and as an A fragment
+__device__ __forceinline__ void pack_x(const float* v, uint32_t* a) {
     a[0] = pack2(v[0], v[1]);
     a[1] = pack2(v[2], v[3]);
     a[2] = pack2(v[4], v[5]);
@@ -235,7 +240,9 @@ __global__ void __launch_bounds__(32 * kFwdWarps) forward_kernel(const Image* __
     for (int64_t tile = (int64_t)blockIdx.x * kFwdWarps + warp; tile < tiles; tile += (int64_t)gridDim.x * kFwdWarps) {
         const int64_t row0 = tile * 16;
         uint32_t a1[1][4], a2[4][4], a3[4][4], a4[4][4];
-        load_x(X, row0 + g < n ? row0 + g : -1, row0 + g + 8 < n ? row0 + g + 8 : -1, t, a1[0]);
+        float xv[8];
+        read_x(X, row0 + g < n ? row0 + g : -1, row0 + g + 8 < n ? row0 + g + 8 : -1, t, xv);
+        pack_x(xv, a1[0]);
         hidden_layer<1>(a1, s.wt1, kS16, s.b1, lane, a2);
         hidden_layer<4>(a2, s.wt2, kS64, s.b2, lane, a3);
         hidden_layer<4>(a3, s.wt3, kS64, s.b3, lane, a4);
@@ -338,32 +345,43 @@ __global__ void __launch_bounds__(32 * kGradWarps, 1)
     GradSmem& s = *reinterpret_cast<GradSmem*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     dev::pdl_trigger();
-    dev::pdl_wait();  // the image is written by the kernel before
-    fetch_image(&s.w, I, &s.bar);
     float m1[4] = {}, m2[4][4] = {}, m3[4][4] = {}, m4[4] = {};
     float mb0 = 0.f, mb1 = 0.f;
     double my_loss = 0.0;
     // contiguous 16-row tiles per block
     const int64_t tiles = (n + 15) / 16;
     const int64_t tile0 = tiles * blockIdx.x / gridDim.x, tile1 = tiles * (blockIdx.x + 1) / gridDim.x;
+    // the warp's 16 rows of the round at tb: drawn and read a round ahead, so
+    // that the draw and the latency of scattered rows lie behind other work
+    float xv[8], tv[4];
+    bool real[2];
+    auto read_rows = [&](int64_t tb) {
+        const int64_t row0 = (tb + warp) * 16;
+        int64_t mine = -1;
+        if (tb + warp < tile1 && lane < 16 && row0 + lane < n) mine = data_row(row0 + lane, n_data, seed, step);
+        const int64_t src0 = __shfl_sync(0xffffffffu, mine, g), src1 = __shfl_sync(0xffffffffu, mine, g + 8);
+        read_x(X, src0, src1, t, xv);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = 2 * t + (q & 1);
+            const int64_t src = q < 2 ? src0 : src1;
+            tv[q] = c < no && src >= 0 ? T[src * no + c] : 0.f;
+        }
+        real[0] = src0 >= 0;
+        real[1] = src1 >= 0;
+    };
+    // the data are the caller's, complete before the first launch of the call,
+    // which is an ordinary one; the image is written by the kernel before
+    read_rows(tile0);
+    dev::pdl_wait();
+    fetch_image(&s.w, I, &s.bar);
     for (int64_t tb = tile0; tb < tile1; tb += kGradWarps) {
         const int act = (int)(tile1 - tb < kGradWarps ? tile1 - tb : kGradWarps);  // tiles of this round
         const int rb = warp * 16;
         if (warp < act) {
             // ---- forward for the warp's 16 rows, keeping every activation
-            const int64_t row0 = (tb + warp) * 16;
-            int64_t mine = -1;
-            if (lane < 16 && row0 + lane < n) mine = data_row(row0 + lane, n_data, seed, step);
-            const int64_t src0 = __shfl_sync(0xffffffffu, mine, g), src1 = __shfl_sync(0xffffffffu, mine, g + 8);
             uint32_t a1[1][4], a2[4][4], a3[4][4], a4[4][4];
-            load_x(X, src0, src1, t, a1[0]);
-            float tv[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int c = 2 * t + (q & 1);
-                const int64_t src = q < 2 ? src0 : src1;
-                if (c < no && src >= 0) tv[q] = T[src * no + c];
-            }
+            pack_x(xv, a1[0]);
             hidden_layer<1>(a1, s.w.wt1, kS16, s.w.b1, lane, a2);
             hidden_layer<4>(a2, s.w.wt2, kS64, s.w.b2, lane, a3);
             hidden_layer<4>(a3, s.w.wt3, kS64, s.w.b3, lane, a4);
@@ -375,8 +393,7 @@ __global__ void __launch_bounds__(32 * kGradWarps, 1)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int c = 2 * t + (q & 1);
-                const int64_t src = q < 2 ? src0 : src1;
-                if (c < no && src >= 0) {
+                if (c < no && real[q >> 1]) {
                     const float e = y[q] - tv[q];
                     my_loss += (double)e * e;
                     dy[q] = inv_n2 * e;
@@ -401,6 +418,7 @@ __global__ void __launch_bounds__(32 * kGradWarps, 1)
             back_layer<4>(dn, s.w.wt2, a2, lane, dz);
             stage(s.dz[0], dz, rb, lane);
         }
+        if (tb + kGradWarps < tile1) read_rows(tb + kGradWarps);
         __syncthreads();
         // ---- weight gradients: chains of up to 64 rows, added in FP32
         const int mt = warp & 3, c0 = 32 * (warp >> 2);
@@ -688,12 +706,19 @@ namespace {
 // one gradient evaluation over n minibatch rows into m->grad and the device
 // loss sum m->loss, and with lr > 0 the Adam step number m->t on it
 mlbm_status grad_pass(mlbm_mlp* m, const float* X, const float* T, int64_t n, int64_t n_data, uint64_t seed,
-                      uint64_t step, float lr, cudaStream_t st) {
+                      uint64_t step, float lr, bool first, cudaStream_t st) {
     const int nb = grad_blocks(n);
     const size_t smem = sizeof(mlp::GradSmem);
     MLP_CUDA(cudaFuncSetAttribute(mlp::grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    MLP_CUDA(launch_pdl_smem(mlp::grad_kernel, nb, 32 * mlp::kGradWarps, smem, st, m->img, X, T, m->n_out, n, n_data,
-                             seed, step, (float)(2.0 / (double)n), m->partial, m->loss_partial));
+    const float inv_n2 = (float)(2.0 / (double)n);
+    if (first) {  // reads the caller's data at once, so not before what is on the stream has ended
+        mlp::grad_kernel<<<nb, 32 * mlp::kGradWarps, smem, st>>>(m->img, X, T, m->n_out, n, n_data, seed, step, inv_n2,
+                                                                 m->partial, m->loss_partial);
+        MLP_CUDA(cudaGetLastError());
+    } else {
+        MLP_CUDA(launch_pdl_smem(mlp::grad_kernel, nb, 32 * mlp::kGradWarps, smem, st, m->img, X, T, m->n_out, n,
+                                 n_data, seed, step, inv_n2, m->partial, m->loss_partial));
+    }
     const int blocks = (m->kp + mlp::kSumParams - 1) / mlp::kSumParams, threads = mlp::kSumParams * mlp::kSumSlices;
     const double c1 = 1.0 - std::pow(0.9, (double)m->t), c2 = 1.0 - std::pow(0.999, (double)m->t);
     auto fn = lr > 0 ? mlp::sum_partials<true> : mlp::sum_partials<false>;
@@ -717,7 +742,7 @@ mlbm_status mlbm_mlp_gradients_device(mlbm_mlp* m, const float* X, const float* 
                                       double* loss, void* stream) {
     if (!m || !X || !T || n <= 0) return set_error(MLBM_E_INVALID, "mlp_gradients: bad arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    mlbm_status s = grad_pass(m, X, T, n, n, 0, 0, 0.f, st);
+    mlbm_status s = grad_pass(m, X, T, n, n, 0, 0, 0.f, true, st);
     if (s != MLBM_OK) return s;
     if (grads) MLP_CUDA(cudaMemcpyAsync(grads, m->grad, m->kp * 4, cudaMemcpyDeviceToDevice, st));
     if (loss) return read_loss(m, n, loss, st);
@@ -732,7 +757,7 @@ mlbm_status mlbm_mlp_train_device(mlbm_mlp* m, const float* X, const float* T, i
     for (int64_t k = 0; k < steps; ++k) {
         const uint64_t draw = (uint64_t)m->t;
         m->t += 1;
-        mlbm_status s = grad_pass(m, X, T, batch, n, seed, draw, lr, st);
+        mlbm_status s = grad_pass(m, X, T, batch, n, seed, draw, lr, k == 0, st);
         if (s != MLBM_OK) {
             m->t -= 1;
             return s;
