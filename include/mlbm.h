@@ -399,7 +399,7 @@ double mlbm_last_step_ms(const mlbm_ctx* ctx);
  *        10 and 12 to the persistent kernel (uncapped / capped for 2 blocks),
  *        0 to the plain uncapped kernel, 20 and 21 to the plain capped and the
  *        persistent uncapped kernel with the early loads, and the rest to the
- *        plain kernel capped for 2 blocks
+ *        plain kernel capped for 2 blocks ("the plain capped kernel", see 29)
  *   22   least-squares BGK with staged neighbourhoods: persistent blocks of
  *        256 threads copy the union of a 256-node tile's stencil members
  *        (32 bytes each, listed when the context is created) into shared
@@ -424,8 +424,11 @@ double mlbm_last_step_ms(const mlbm_ctx* ctx);
  *        shared-memory slot of its own, one tile ahead, with bulk async
  *        copies; a warp with interpolated bounce-back links evaluates them in
  *        the same pass: 27 = 12 warps per SM (K = 24: 10, K = 32: 8), 28 = 8
- *        (K = 32: 6), 29 = 14 (K = 24: 11, K = 32: 7) (BGK and tau = 1;
- *        RBF-FD stencils run the plain capped kernel)
+ *        (K = 32: 6), 29 = 14 (K = 24: 11, K = 32: 7) (BGK and tau = 1).
+ * RBF-FD stencils: where a number runs "the plain capped kernel", a BGK
+ * context of a large set with stencils per Lagrangian point, or after 28 or
+ * 29 was set, steps from tile records of its non-zero weights instead (same
+ * results).
  * Variants 4 and up are available for K = 12, 16, 24 and 32.
  * The default is 27 when available, else 1.  mlbm_autotune times every
  * available variant for steps_per_variant steps on the context's stream

@@ -219,11 +219,69 @@ mlbm_status launch_one_step(mlbm_ctx* c, int variant) {
             MLBM_CUDA(launch_step_warp(variant, model, c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->ruv[a],
                                        c->ruv[b], c->C, a, c->err, W, c->stream));
     }
+    else if (model == 0 && c->S.rbf_rec && variant != 0 && variant != 10 && variant != 12 && variant != 20 &&
+             variant != 21)  // the numbers that run the plain capped kernel without records
+        MLBM_CUDA(launch_step_rbf_tiles(c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->C, a, c->err,
+                                        dev::Wait{c->wait_ns, 0}, c->stream));
     else if (model == 0)
         MLBM_CUDA(launch_bgk_step(c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->C, variant, c->stream));
     else
         MLBM_CUDA(launch_tau1_step(c->S, c->ruv[a], c->ruv[b], c->C, variant, c->stream));
     c->cur = b;
+    return MLBM_OK;
+}
+
+// A BGK context of RBF-FD stencils steps from tile records of its non-zero weights
+// where the plain rows (36 K bytes a node) take more than 100 MB, so that they
+// come from HBM, and the records at most two thirds of that.  Stencils per
+// Lagrangian point of 25 nodes in 64 slots (us a step, plain / records): 65k nodes
+// (150 MB) 25.4 / 18.8, 46k (107 MB) 20.9 / 13.5, 24k 10.3 / 10.5.  Stencils of the
+// node's own 24 have no zeros to leave out: 147k nodes 23.1 / 26.7, 260k 41.1 /
+// 44.5.  Kernel variants 28 and 29 take the records in any case.
+constexpr size_t kRbfTilesFrom = size_t(100) << 20;
+
+// The records of the RBF-FD step from the uploaded stencils.  Where they do
+// not fit (node numbers of 28 bits, no memory) the context steps without them.
+mlbm_status build_rbf_tiles(mlbm_ctx* c, bool always) {
+    const int tiles = (int)((c->n + 15) / 16);
+    if (tiles == 0 || c->n + c->n_halo >= (int64_t)1 << 28) return MLBM_OK;
+    std::vector<void*> made;
+    auto room = [&](void** p, size_t bytes) {
+        if (cudaMalloc(p, std::max<size_t>(bytes, 128)) != cudaSuccess) {
+            (void)cudaGetLastError();
+            for (void* q : made) cudaFree(q);
+            return false;
+        }
+        made.push_back(*p);
+        return true;
+    };
+    void *dsize = nullptr, *drec = nullptr, *dhead = nullptr, *drange = nullptr;
+    if (!room(&dsize, (size_t)tiles * sizeof(int2))) return MLBM_OK;
+    std::vector<int2> size((size_t)tiles);
+    cudaError_t e = rbf_tile_sizes(c->S, tiles, static_cast<int2*>(dsize), c->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(size.data(), dsize, size.size() * sizeof(int2), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    cudaFree(dsize);
+    made.clear();
+    MLBM_CUDA(e);
+    std::vector<int4> head;
+    std::vector<int> range;
+    const int blocks = std::min(tiles, warp_step_ranges(1 << 30));
+    if (!rbf_tiles_plan(size, blocks, head, range, c->S.rbf_slot, c->S.rbf_bytes)) return MLBM_OK;
+    if (!always && 3 * c->S.rbf_bytes > 2 * (size_t)c->n * 36 * c->K) return MLBM_OK;
+    if (!room(&drec, c->S.rbf_bytes) || !room(&dhead, head.size() * sizeof(int4)) ||
+        !room(&drange, range.size() * sizeof(int)))
+        return MLBM_OK;
+    for (void* q : made) c->allocations.push_back(q);
+    MLBM_TRY(upload(c, dhead, head.data(), head.size() * sizeof(int4)));
+    MLBM_TRY(upload(c, drange, range.data(), range.size() * sizeof(int)));
+    MLBM_CUDA(rbf_tile_fill(c->S, tiles, static_cast<int4*>(dhead), static_cast<uint8_t*>(drec), c->stream));
+    MLBM_CUDA(cudaStreamSynchronize(c->stream));
+    c->S.rbf_rec = static_cast<uint8_t*>(drec);
+    c->S.rbf_head = static_cast<int4*>(dhead);
+    c->S.rbf_range = static_cast<int*>(drange);
+    c->S.rbf_blocks = blocks;
     return MLBM_OK;
 }
 
@@ -522,6 +580,7 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         c->S.stage_max = stage_max;
     }
     MLBM_CUDA(launch_record_kinds(c->S, c->rec, c->need, c->range, c->stream));
+    if (rbf && p->model == MLBM_MODEL_BGK && (size_t)n * 36 * K > kRbfTilesFrom) MLBM_TRY(build_rbf_tiles(c, false));
     set_collide(c);
     // ---- initial state
     std::vector<double> ru((size_t)n * 3);
@@ -1123,6 +1182,8 @@ mlbm_status mlbm_set_kernel_variant(mlbm_ctx* c, int variant) {
         return set_error(MLBM_E_INVALID, "set_kernel_variant: variant not available for this K");
     if (variant == 22 && c->params.model == MLBM_MODEL_BGK && !c->S.Wr && !c->S.lidx)
         return set_error(MLBM_E_INVALID, "set_kernel_variant: no staged neighbourhoods for this context");
+    if ((variant == 28 || variant == 29) && c->S.Wr && c->params.model == MLBM_MODEL_BGK && !c->S.rbf_rec)
+        MLBM_TRY(build_rbf_tiles(c, true));
     c->variant = variant;
     return MLBM_OK;
 }

@@ -64,6 +64,15 @@ struct Stencil {
     // RBF-FD stencils: per-direction weights [8 K/4][n_pad] float4 (row
     // r = direction k - 1), null for the least-squares fit
     const float4* Wr;
+    // RBF-FD stencils of a BGK context: tile records with the non-zero weights
+    // (kernels_rbf_tiles.cu), each tile's (offset in 128 bytes, member groups,
+    // weight rows, 0), the tile ranges of the blocks, the bytes of a record
+    // slot and of all records; null where not built
+    const uint8_t* rbf_rec;
+    const int4* rbf_head;
+    const int* rbf_range;
+    int rbf_blocks, rbf_slot;
+    size_t rbf_bytes;
     // neighbourhood staging (step variant 22, least-squares BGK): for each
     // tile of kStageTile consecutive nodes the sorted union of the stencil
     // members of its least-squares nodes without links (stage_ids, from
@@ -126,6 +135,7 @@ struct PartDev {
     const int2* sends;
 };
 
+constexpr int kRbfMaxWarps = 12;   // warps of a block of the RBF-FD tile step
 constexpr int kStageTile = 256;   // nodes per staged tile (one block)
 constexpr int kStageMax = 1536;   // largest neighbourhood that is staged (48 KiB per buffer)
 

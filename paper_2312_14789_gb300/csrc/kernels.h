@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <vector>
 
 #include "device_common.cuh"
 
@@ -60,6 +61,16 @@ cudaError_t launch_exchange(const dev::PartDev* parts, const int4* list, int64_t
 cudaError_t launch_step_warp(int variant, int model, const dev::Stencil& S, const float4* a8, const float* a0,
                              float4* b8, float* b0, const float4* ra, float4* rb, const dev::Collide& C, int backward,
                              int* err, const dev::Wait& W, cudaStream_t st);
+// RBF-FD tile records (kernels_rbf_tiles.cu; tiles of 16 nodes): their sizes,
+// the layout from the sizes (false where they do not fit), their contents,
+// and the step from them
+cudaError_t rbf_tile_sizes(const dev::Stencil& S, int tiles, int2* size, cudaStream_t st);
+bool rbf_tiles_plan(const std::vector<int2>& size, int blocks, std::vector<int4>& head, std::vector<int>& range,
+                    int& slot, size_t& bytes);
+cudaError_t rbf_tile_fill(const dev::Stencil& S, int tiles, const int4* head, uint8_t* rec, cudaStream_t st);
+cudaError_t launch_step_rbf_tiles(const dev::Stencil& S, const float4* in, const float* f0in, float4* out,
+                                  float* f0out, const dev::Collide& C, int backward, int* err, const dev::Wait& W,
+                                  cudaStream_t st);
 cudaError_t launch_get_tau1(int n, const int* perm, const float4* s, double* ru, cudaStream_t st);
 cudaError_t launch_macroscopics(int model, int n, const int* perm, const float4* f8, const float* f0,
                                 const float4* ruv, float ax, float ay, const uint16_t* node_sample,
