@@ -66,6 +66,7 @@ struct mlbm_ctx {
     int variant = 27;
     std::vector<int> inv_perm;  // caller's node id -> device position
     int* err = nullptr;  // device error word of the bounded waits
+    int cluster = 0;  // blocks of the cluster that takes runs of steps (0: the set does not fit one)
     dev::Stencil S{};
     dev::Collide C{};
     std::vector<void*> allocations;
@@ -228,6 +229,26 @@ mlbm_status launch_one_step(mlbm_ctx* c, int variant) {
     else
         MLBM_CUDA(launch_tau1_step(c->S, c->ruv[a], c->ruv[b], c->C, variant, c->stream));
     c->cur = b;
+    return MLBM_OK;
+}
+
+// Runs of at least this many steps go to the cluster kernel where the set fits
+// it; a shorter one does not repay the fetch of all records.
+constexpr int kClusterMin = 4;
+constexpr int kClusterSteps = 4096;  // most steps of one launch
+
+bool by_cluster(const mlbm_ctx* c, int64_t n_steps, int variant) {
+    return c->cluster > 0 && variant == 27 && c->use_graphs && n_steps >= kClusterMin && !c->withhold_next;
+}
+
+mlbm_status launch_cluster_steps(mlbm_ctx* c, int64_t n_steps) {
+    for (int64_t left = n_steps; left > 0;) {
+        const int m = (int)std::min<int64_t>(left, kClusterSteps), a = c->cur, b = a ^ (m & 1);
+        MLBM_CUDA(launch_step_cluster(c->cluster, c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->C, m, c->err,
+                                      dev::Wait{c->wait_ns, 0}, c->stream));
+        c->cur = b;
+        left -= m;
+    }
     return MLBM_OK;
 }
 
@@ -516,6 +537,7 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
     MLBM_TRY(dalloc(c, &c->seg_dev, ns + 1));
     MLBM_TRY(upload(c, c->seg_dev, c->seg_off.data(), (ns + 1) * sizeof(int64_t)));
     MLBM_CUDA(cudaMemsetAsync(c->err, 0, sizeof(double), c->stream));
+    if (!rbf && c->n_halo == 0 && p->model == MLBM_MODEL_BGK) c->cluster = step_cluster_size(Kq, (int)n);
     if (!tma_supported(Kq)) c->variant = 1;  // variants >= 4 exist for K in {12, 16, 24, 32}
     if (rbf) {
         MLBM_TRY(upload(c, c->idx, hidx.data(), hidx.size() * 4));
@@ -937,8 +959,12 @@ mlbm_status mlbm_step(mlbm_ctx* c, int64_t n_steps) {
     if (n_steps == 0) return MLBM_OK;
     if (c->timing) MLBM_CUDA(cudaEventRecord(c->ev0, c->stream));
     int64_t left = n_steps;
+    if (by_cluster(c, n_steps, c->variant)) {
+        MLBM_TRY(launch_cluster_steps(c, n_steps));
+        left = 0;
+    }
     // a launch that must withhold a tile runs directly, not from a graph
-    if (c->use_graphs && n_steps >= kGraphSteps && !c->withhold_next) {
+    else if (c->use_graphs && n_steps >= kGraphSteps && !c->withhold_next) {
         refresh_graphs(c);
         while (left >= kGraphSteps) {
             MLBM_TRY(ensure_graph(c, c->cur));
@@ -960,7 +986,7 @@ mlbm_status mlbm_step(mlbm_ctx* c, int64_t n_steps) {
 
 mlbm_status mlbm_prepare_graphs(mlbm_ctx* c) {
     if (!c) return set_error(MLBM_E_INVALID, "prepare_graphs: NULL context");
-    if (!c->use_graphs) return MLBM_OK;
+    if (!c->use_graphs || by_cluster(c, kGraphSteps, c->variant)) return MLBM_OK;
     refresh_graphs(c);
     MLBM_TRY(ensure_graph(c, 0));
     MLBM_TRY(ensure_graph(c, 1));
@@ -1278,7 +1304,10 @@ mlbm_status mlbm_autotune_ex(mlbm_ctx* c, int steps_per_variant, int flush_l2, d
             per = tot / steps_per_variant;
         } else {
             if (cudaEventRecord(c->ev0, c->stream) != cudaSuccess) break;
-            for (int i = 0; i < steps_per_variant && st == MLBM_OK; ++i) st = launch_one_step(c, v);
+            if (by_cluster(c, steps_per_variant, v))
+                st = launch_cluster_steps(c, steps_per_variant);
+            else
+                for (int i = 0; i < steps_per_variant && st == MLBM_OK; ++i) st = launch_one_step(c, v);
             if (st != MLBM_OK) break;
             cudaEventRecord(c->ev1, c->stream);
             if (cudaEventSynchronize(c->ev1) != cudaSuccess) {

@@ -61,6 +61,13 @@ cudaError_t launch_exchange(const dev::PartDev* parts, const int4* list, int64_t
 cudaError_t launch_step_warp(int variant, int model, const dev::Stencil& S, const float4* a8, const float* a0,
                              float4* b8, float* b0, const float4* ra, float4* rb, const dev::Collide& C, int backward,
                              int* err, const dev::Wait& W, cudaStream_t st);
+// many BGK steps of a small set by one cluster that keeps everything in shared
+// memory (kernels_cluster.cu): its size for a set (0: does not fit), and
+// `steps` steps from one state into another (the same buffers, or others)
+int step_cluster_size(int Kq, int n);
+cudaError_t launch_step_cluster(int size, const dev::Stencil& S, const float4* in, const float* f0in, float4* out,
+                                float* f0out, const dev::Collide& C, int steps, int* err, const dev::Wait& W,
+                                cudaStream_t st);
 // RBF-FD tile records (kernels_rbf_tiles.cu; tiles of 16 nodes): their sizes,
 // the layout from the sizes (false where they do not fit), their contents,
 // and the step from them

@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kRbfMaxWarps * 32, 1)
                 s[b] = acc[b] + o[b];
                 if ((links >> b) & 1u)
                     s[b] = S.bb_mode == 0 ? o[b ^ 2]
-                                          : lagrange_link(in, block, r, cx, cy, 4 * h + 1 + b,
+                                          : lagrange_link([&](int j, int k) { return pop(in, j, k); }, block, r, cx, cy, 4 * h + 1 + b,
                                                           S.links[S.link_slot[p]].t[4 * h + b], o[b ^ 2]);
             }
         }

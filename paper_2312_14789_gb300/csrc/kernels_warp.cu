@@ -24,7 +24,7 @@
 //   - When the records outgrow L2, steps walk the tiles forwards and backwards
 //     in turn, so that a step starts on what the last one left in L2.
 // Step times before (variant 25, rows loaded by each thread) and after, us,
-// K = 16, graph replay on one GB300: 2k-node channel (K = 12) 5.2 / 2.7; 192k
+// K = 16, graph replay on one GB300: 2k-node channel (K = 12) 5.2 / 2.9; 192k
 // porous tau = 1 15.7 / 14.3; nine flows of it, 1.73M nodes, 142.4 / 120.1
 // (6.7 TB/s of stored bytes); 96k porous TRT with interpolated links 24.5 /
 // 8.1; vortex street 260k 25.3 / 20.4; its hybrid set, 165k, 13.1 / 9.8.
@@ -63,20 +63,6 @@ struct WarpTile {
     static constexpr int kWarps = WARPS;
     static constexpr int kSmem = kWarps * (kBytes + 16);
 };
-
-__device__ __forceinline__ int at4(const int4& v, int c) { return c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w)); }
-__device__ __forceinline__ float at4(const float4& v, int c) { return c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w)); }
-
-// the six rows of stencil group q from the warp's slot (base: row 0, this lane)
-template <int KQ>
-__device__ __forceinline__ void slot_rows(const float4* base, int q, float4* m) {
-    using R = TileRec<KQ>;
-    const float4* b = base + R::m_row(q) * 32;
-#pragma unroll
-    for (int a = 0; a < 5; ++a) m[a] = b[a * 32];
-    if (q == R::kSp) m[5] = make_float4(m[0].w, m[1].w, m[2].w, 0.f);
-    else m[5] = b[5 * 32];
-}
 
 // Increments of the eight streamed populations over the node's own.  The
 // gather of group q + 1 goes out member by member as group q is used up.
@@ -205,7 +191,8 @@ __device__ __forceinline__ void walk_tiles(const Stencil& S, const float4* __res
         if (!ok) {
             if (lane == 0) {
                 atomicExch(err, 2);
-                // do not leave while the matrix rows may still be landing
+                // do not leave while copies may still be landing
+                if (!withhold) mbar_wait(bar, ph, W.budget_ns);
                 if (need == 2 && !withhold) mbar_wait(bar + 1, phm, W.budget_ns);
             }
             return;
@@ -228,12 +215,13 @@ __device__ __forceinline__ void walk_tiles(const Stencil& S, const float4* __res
             // the slot's matrix rows are read: refill them for the warp's next tile
             if (need == 2) {
                 m_ok = __all_sync(0xffffffffu, m_ok && mbar_wait(bar + 1, phm, W.budget_ns));
+                if (!m_ok) return false;
                 phm ^= 1u;
             } else {
                 __syncwarp();
             }
             if (lane == 0 && !last) copy_m(tn);
-            return m_ok;
+            return true;
         };
         const Collide C = S.coll ? S.coll[word >> 8] : C0;
         if (MODEL == 0) {
@@ -264,10 +252,9 @@ __device__ __forceinline__ void walk_tiles(const Stencil& S, const float4* __res
             if (!m_done()) {
                 if (lane == 0) {
                     atomicExch(err, 2);
-                    if (!last) {
-                        mbar_wait(bar, ph, W.budget_ns);
-                        if (need_next == 2) mbar_wait(bar + 1, phm, W.budget_ns);
-                    }
+                    // do not leave while copies may still be landing
+                    if (!last) mbar_wait(bar, ph, W.budget_ns);
+                    mbar_wait(bar + 1, phm, W.budget_ns);
                 }
                 return;
             }
@@ -289,7 +276,8 @@ __device__ __forceinline__ void walk_tiles(const Stencil& S, const float4* __res
                                         id[2].x};
                     const float r = __int_as_float(id[2].y), cx = (float)ex_of(meta >> 4),
                                 cy = (float)ey_of(meta >> 4);
-                    lagrange_increments<1>(in, ids, r, cx, cy, oa, ob, 0, acc);
+                    lagrange_increments<1>([&](int j, float4& a, float4& b) { ldg_pair(in + 2 * (size_t)j, a, b); },
+                                           ids, r, cx, cy, oa, ob, 0, acc);
 #pragma unroll
                     for (int k = 0; k < 8; ++k) g[k + 1] = acc[k] + own[k];
                     if (links)
@@ -298,7 +286,8 @@ __device__ __forceinline__ void walk_tiles(const Stencil& S, const float4* __res
                             if (!((lk.mask >> k) & 1u)) continue;
                             const int kp = opp_of(k);
                             g[k] = S.bb_mode == 0 ? own[kp - 1]
-                                                  : lagrange_link(in, ids, r, cx, cy, k, lk.t[k - 1], own[kp - 1]);
+                                                  : lagrange_link([&](int j, int kk) { return pop(in, j, kk); }, ids, r,
+                                                                  cx, cy, k, lk.t[k - 1], own[kp - 1]);
                         }
                 }
                 g[0] = f0own;
@@ -350,10 +339,9 @@ __device__ __forceinline__ void walk_tiles(const Stencil& S, const float4* __res
             if (!m_done()) {
                 if (lane == 0) {
                     atomicExch(err, 2);
-                    if (!last) {
-                        mbar_wait(bar, ph, W.budget_ns);
-                        if (need_next == 2) mbar_wait(bar + 1, phm, W.budget_ns);
-                    }
+                    // do not leave while copies may still be landing
+                    if (!last) mbar_wait(bar, ph, W.budget_ns);
+                    mbar_wait(bar + 1, phm, W.budget_ns);
                 }
                 return;
             }
@@ -381,7 +369,7 @@ __device__ __forceinline__ void walk_tiles(const Stencil& S, const float4* __res
                     cx = (float)ex_of(meta >> 4);
                     cy = (float)ey_of(meta >> 4);
                 }
-                const float4 o = tau1_finish(S, C, me, kind, c, v9, r, cx, cy, (meta & 4) != 0, p);
+                const float4 o = tau1_finish(S, C, me, kind, c, v9, r, cx, cy, links_of(S, p, (meta & 4) != 0));
                 if (p < S.n) {
                     out[p] = o;
                     if (PART && (meta & 8)) send_state(parts, *own, parity, p, o, nullptr);

@@ -90,17 +90,40 @@ struct SmemRows {
     }
 };
 
+__device__ __forceinline__ int at4(const int4& v, int c) { return c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w)); }
+__device__ __forceinline__ float at4(const float4& v, int c) { return c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w)); }
+
+// the six rows of stencil group q from a record in shared memory (base: row 0, this lane)
+template <int KQ>
+__device__ __forceinline__ void slot_rows(const float4* base, int q, float4* m) {
+    using R = TileRec<KQ>;
+    const float4* b = base + R::m_row(q) * 32;
+#pragma unroll
+    for (int a = 0; a < 5; ++a) m[a] = b[a * 32];
+    if (q == R::kSp) m[5] = make_float4(m[0].w, m[1].w, m[2].w, 0.f);
+    else m[5] = b[5 * 32];
+}
+
 template <class Rows>
 __device__ __forceinline__ Rows rows_of(const Stencil& S, int p, const Rows* given) {
     if constexpr (std::is_constructible<Rows, const Stencil&, int>::value) return Rows(S, p);
     else return *given;
 }
 
+// node p's bounce-back links (none without the link bit)
+__device__ __forceinline__ LinkRec links_of(const Stencil& S, int p, bool any) {
+    LinkRec L;
+    L.mask = 0;
+    if (any) L = S.links[S.link_slot[p]];
+    return L;
+}
+
 // Increments of the eight streamed populations over the node's own (oa, ob)
 // from its 3x3 Lagrange block (LPN = 2: this lane's half of the nine points).
-template <int LPN>
-__device__ __forceinline__ void lagrange_increments(const float4* __restrict__ f8in, const int* ids, float r, float cx,
-                                                    float cy, const float4& oa, const float4& ob, int h, float* acc) {
+// pair(j, a, b) gives the populations of member j.
+template <int LPN, class Pair>
+__device__ __forceinline__ void lagrange_increments(Pair pair, const int* ids, float r, float cx, float cy,
+                                                    const float4& oa, const float4& ob, int h, float* acc) {
     // basis values for e_x, e_y in {+1, 0, -1}: t = -r e - c
     float xp[3], x0[3], xm[3], yp[3], y0[3], ym[3];
     lag3(-r - cx, xp[0], xp[1], xp[2]);
@@ -113,9 +136,8 @@ __device__ __forceinline__ void lagrange_increments(const float4* __restrict__ f
     for (int bp = 0; bp < 9; ++bp) {
         if (LPN == 2 && (bp & 1) != h) continue;
         const int b = bp / 3, a = bp % 3;
-        const int j = ids[bp];
         float4 ra, rb;
-        ldg_pair(f8in + 2 * (size_t)j, ra, rb);
+        pair(ids[bp], ra, rb);
         const float4 fa = make_float4(ra.x - oa.x, ra.y - oa.y, ra.z - oa.z, ra.w - oa.w);
         const float4 fb = make_float4(rb.x - ob.x, rb.y - ob.y, rb.z - ob.z, rb.w - ob.w);
         acc[0] = fmaf(xp[a] * y0[b], fa.x, acc[0]);
@@ -131,14 +153,16 @@ __device__ __forceinline__ void lagrange_increments(const float4* __restrict__ f
 
 // A Lagrange node's interpolated bounce-back link in direction k: population
 // k' (own value o) at the reflected point x + tt s e_k.
-__device__ __forceinline__ float lagrange_link(const float4* __restrict__ f8in, const int* ids, float r, float cx,
-                                               float cy, int k, float tt, float o) {
+// at(j, k) gives population k of member j.
+template <class At>
+__device__ __forceinline__ float lagrange_link(At at, const int* ids, float r, float cx, float cy, int k, float tt,
+                                               float o) {
     float lx[3], ly[3];
     lag3(tt * r * ex_of(k) - cx, lx[0], lx[1], lx[2]);
     lag3(tt * r * ey_of(k) - cy, ly[0], ly[1], ly[2]);
     float v = 0.f;
     for (int b = 0; b < 3; ++b)
-        for (int a = 0; a < 3; ++a) v = fmaf(lx[a] * ly[b], pop(f8in, ids[b * 3 + a], opp_of(k)) - o, v);
+        for (int a = 0; a < 3; ++a) v = fmaf(lx[a] * ly[b], at(ids[b * 3 + a], opp_of(k)) - o, v);
     return o + v;
 }
 
@@ -242,7 +266,8 @@ __device__ __forceinline__ void bgk_node(const Stencil& S, const float4* __restr
         } else {
             int ids[9];
             R.lag(ids);
-            lagrange_increments<LPN>(f8in, ids, r, cx, cy, oa, ob, h, acc);
+            lagrange_increments<LPN>([&](int j, float4& a, float4& b) { ldg_pair(f8in + 2 * (size_t)j, a, b); }, ids, r, cx,
+                                     cy, oa, ob, h, acc);
         }
         if (LPN == 2) {
 #pragma unroll
@@ -269,7 +294,8 @@ __device__ __forceinline__ void bgk_node(const Stencil& S, const float4* __restr
                 } else {
                     int ids[9];
                     lag_block(S, p, ids);
-                    acc[k - 1] = lagrange_link(f8in, ids, r, cx, cy, k, L.t[k - 1], own[kp - 1]);
+                    acc[k - 1] = lagrange_link([&](int j, int kk) { return pop(f8in, j, kk); }, ids, r, cx, cy, k,
+                                               L.t[k - 1], own[kp - 1]);
                 }
             }
         }
@@ -483,10 +509,7 @@ __device__ __forceinline__ void eval_coeffs(const float (*c)[6], const float* pb
 // its block's values (kind 1), one lane per node.
 __device__ __forceinline__ float4 tau1_finish(const Stencil& S, const Collide& C, const float4& me, int kind,
                                               const float (*c)[6], const float4* v9, float r, float cx, float cy,
-                                              bool has_links, int p) {
-    LinkRec L;
-    L.mask = 0;
-    if (has_links) L = S.links[S.link_slot[p]];
+                                              const LinkRec& L) {
     const float rhox = 1.0f + me.x;
     float mx = 0.f, my = 0.f;
     float dm = w_of(0) * rhox * (-1.5f * (me.y * me.y + me.z * me.z)) + 0.5f * src(0, rhox, me.y, me.z, C.ax, C.ay);
