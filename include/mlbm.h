@@ -425,7 +425,7 @@ double mlbm_last_step_ms(const mlbm_ctx* ctx);
  *        copies; a warp with interpolated bounce-back links evaluates them in
  *        the same pass: 27 = 12 warps per SM (K = 24: 10, K = 32: 8), 28 = 8
  *        (K = 32: 6), 29 = 14 (K = 24: 11, K = 32: 7) (BGK and tau = 1).
- *        With 27 and graphs enabled, runs of 4 or more BGK steps of a set of
+ *        With 27 and graphs enabled, runs of 8 or more BGK steps of a set of
  *        up to 64 tiles go to one cluster of blocks that keeps records and
  *        states in shared memory for the whole run (same results bit for bit)
  * RBF-FD stencils: where a number runs "the plain capped kernel", a BGK

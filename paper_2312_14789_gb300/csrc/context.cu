@@ -233,8 +233,11 @@ mlbm_status launch_one_step(mlbm_ctx* c, int variant) {
 }
 
 // Runs of at least this many steps go to the cluster kernel where the set fits
-// it; a shorter one does not repay the fetch of all records.
-constexpr int kClusterMin = 4;
+// it; a shorter one does not repay the fetch of all records and states (us a
+// call and wait, launches / cluster, 2000 nodes: 4 steps 22.6 / 24.7, 6 steps
+// 29.1 / 28.9, 8 steps 35.2 / 32.9, 12 steps 47.1 / 42.0; 500 nodes: 22.9 / 21.9,
+// 29.2 / 25.8, 34.7 / 29.3, 47.0 / 35.9).
+constexpr int kClusterMin = 8;
 constexpr int kClusterSteps = 4096;  // most steps of one launch
 
 bool by_cluster(const mlbm_ctx* c, int64_t n_steps, int variant) {
