@@ -17,7 +17,8 @@
 // slot order of the plain kernel: the same state bit for bit.
 // One warp owns one shared-memory slot, which a bulk copy refills while the
 // warp collides and stores; what bounds it now is the chain of a tile, a dozen
-// rounds of gathers and weight reads, on the 11 warps whose slots an SM holds.
+// rounds of gathers and weight reads, on the ten warps whose slots an SM holds
+// (34% of issue slots, stalls on gathers and records).
 // us a step, plain rows / records: 65k nodes 25.4 / 18.8, 46k 20.9 / 13.5.  (A
 // branch for each weight 24.3, three groups of gathers ahead with spills 22.0.)
 #include <algorithm>
