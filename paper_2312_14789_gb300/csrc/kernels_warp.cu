@@ -217,9 +217,9 @@ __device__ __forceinline__ void walk_tiles(const Stencil& S, const float4* __res
                 m_ok = __all_sync(0xffffffffu, m_ok && mbar_wait(bar + 1, phm, W.budget_ns));
                 if (!m_ok) return false;
                 phm ^= 1u;
-            } else {
-                __syncwarp();
             }
+            // the vote above orders no memory: every lane's reads come before the copy over them by this
+            __syncwarp();
             if (lane == 0 && !last) copy_m(tn);
             return true;
         };
