@@ -6,10 +6,14 @@
 // Here every sum is three FP32 numbers of falling magnitude, fed by error-free
 // transforms (Knuth's TwoSum, the FMA product error; the square root by two
 // correction steps on its exact residual), so what is lost per node lies
-// ~2^-70 below it, and the three are added into FP64 every kFlush nodes:
-// fewer FP64 roundings than one per node.  Nodes with a value that is neither
-// zero nor within [2^-45, 2^45] (where an error term could leave the FP32
-// range), infinities and NaN take the FP64 path.  13.25M nodes: 523 -> 148 us.
+// 2^-68 below it, and the three are added into FP64 every kFlush nodes:
+// fewer FP64 roundings than one per node.  For that every product and error
+// term has to lie in the FP32 range: a node takes the FP64 path when a value is
+// neither zero nor within [2^-45, 2^45] (u^2 and rho A then reach 2^90, and
+// their last bits 2^-136), when |u|^2 A, the one product of three values, is
+// neither zero nor within [2^-77, 2^110] (at the lower end the third of its
+// parts rounds at 2^-149, 2^-72 of it; kFlush terms at the upper end add up to
+// 2^118), and for infinities and NaN.  13.25M nodes: 523 -> 148 us.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -66,6 +70,7 @@ struct Float3Sum {
 // sums of A, rho A, ux A, uy A, |u| A, |u|^2 A
 struct FieldSums {
     static constexpr int kFlush = 256;
+    static constexpr float kLeast = 6.617444900424222e-24f, kMost = 1.298074214633707e33f;  // 2^-77, 2^110
     Float3Sum f[6];
     double s[6] = {0, 0, 0, 0, 0, 0};
     int held = 0;
@@ -75,7 +80,13 @@ struct FieldSums {
         return x == 0.f || (a >= 2.84217094304040074e-14f && a <= 3.5184372088832e13f);
     }
     __device__ __forceinline__ void add(float rho, float u, float v, float a) {
-        if (!(plain(rho) && plain(u) && plain(v) && plain(a))) {
+        // |u|^2 = p + e + q + g, and x0 its leading part
+        float p, e, q, g, x0, x1, x2, t, w;
+        exact_prod(u, u, p, e);
+        exact_prod(v, v, q, g);
+        exact_sum(p, q, x0, t);
+        const float m2a = fabsf(__fmul_rn(x0, a));
+        if (!(plain(rho) && plain(u) && plain(v) && plain(a) && (m2a == 0.f || (m2a >= kLeast && m2a <= kMost)))) {
             const double da = a, du = u, dv = v, m2 = du * du + dv * dv;
             s[0] += da;
             s[1] += (double)rho * da;
@@ -90,10 +101,6 @@ struct FieldSums {
         f[2].add_prod(u, a);
         f[3].add_prod(v, a);
         // |u|^2 = x0 + x1 + x2
-        float p, e, q, g, x0, x1, x2, t, w;
-        exact_prod(u, u, p, e);
-        exact_prod(v, v, q, g);
-        exact_sum(p, q, x0, t);
         exact_sum(e, g, x1, x2);
         exact_sum(t, x1, x1, w);
         x2 += w;
