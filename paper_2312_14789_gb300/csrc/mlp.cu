@@ -5,8 +5,8 @@
 // Parameters are kept in FP32 ("master") in the packed order W1[16][64], b1,
 // W2[64][64], b2, W3[64][64], b3, W4[64][n_out], b4 (y = x W + b per layer).
 // Whoever writes a parameter also writes its BF16 copy in the network's weight
-// image ([out][in] rows, padded), so a block fetches all its weights with one
-// bulk copy; the transposed operands of the backward pass come from the same
+// image ([out][in] rows, padded), so a block copies all its weights as they
+// lie; the transposed operands of the backward pass come from the same
 // rows through transposing fragment loads.  Rounding points: the features and
 // every hidden activation (after bias and ReLU) are rounded to BF16 where they
 // become an MMA operand; the output error and every hidden error likewise.
@@ -97,7 +97,7 @@ struct __align__(16) Image {
     __nv_bfloat16 wt4[8 * kS64];
     float b1[kH], b2[kH], b3[kH], b4[8];
 };
-static_assert(sizeof(Image) % 16 == 0, "copied in bulk");
+static_assert(sizeof(Image) % 16 == 0, "copied 16 bytes at a time");
 
 // parameter i (packed order) into the image
 __device__ __forceinline__ void image_put(Image* I, int no, int i, float v) {
@@ -117,20 +117,16 @@ __global__ void refresh_image(int kp, int no, const float* __restrict__ P, Image
     if (i < kp) image_put(I, no, i, P[i]);
 }
 
-// the image into the block's shared memory: started by one thread, awaited by
-// all.  The wait polls a copy this block issued itself; it gives up after two
-// seconds, as a lost copy would otherwise hold the GPU (the results are then
-// of whatever the memory held).
-__device__ __forceinline__ void fetch_image(Image* s, const Image* I, uint64_t* bar) {
-    if (threadIdx.x == 0) {
-        dev::mbar_init(bar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async;" ::: "memory");  // the image was written by ordinary stores
-        dev::mbar_expect_tx(bar, sizeof(Image));
-        dev::bulk_g2s(s, I, sizeof(Image), bar);
-    }
+// The image into the block's shared memory, 16 bytes a thread at a time past the
+// registers.  Unlike a bulk copy on a barrier it needs no wait that could run
+// out.
+__device__ __forceinline__ void fetch_image(Image* s, const Image* I) {
+    const uint32_t to = dev::saddr(s);
+    for (uint32_t o = threadIdx.x * 16; o < sizeof(Image); o += blockDim.x * 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + o),
+                     "l"(reinterpret_cast<const uint8_t*>(I) + o) : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    dev::mbar_wait(bar, 0, 2000000000ULL);
 }
 
 // Row of the data set that minibatch row r reads: r itself (seed 0), else a
@@ -232,9 +228,8 @@ __global__ void __launch_bounds__(32 * kFwdWarps) forward_kernel(const Image* __
                                                                  const float* __restrict__ X, int64_t n, int no,
                                                                  float* __restrict__ Y) {
     __shared__ Image s;
-    __shared__ uint64_t bar;
     dev::pdl_wait();
-    fetch_image(&s, I, &bar);
+    fetch_image(&s, I);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int64_t tiles = (n + 15) / 16;
     for (int64_t tile = (int64_t)blockIdx.x * kFwdWarps + warp; tile < tiles; tile += (int64_t)gridDim.x * kFwdWarps) {
@@ -274,7 +269,6 @@ struct GradSmem {
     __nv_bfloat16 dy[kRound * 8];
     double loss[kGradWarps];
     float bias[kGradWarps * 32];
-    uint64_t bar;
 };
 
 // store a warp's [16 rows x 64] A fragments row-major
@@ -374,7 +368,7 @@ __global__ void __launch_bounds__(32 * kGradWarps, 1)
     // which is an ordinary one; the image is written by the kernel before
     read_rows(tile0);
     dev::pdl_wait();
-    fetch_image(&s.w, I, &s.bar);
+    fetch_image(&s.w, I);
     for (int64_t tb = tile0; tb < tile1; tb += kGradWarps) {
         const int act = (int)(tile1 - tb < kGradWarps ? tile1 - tb : kGradWarps);  // tiles of this round
         const int rb = warp * 16;
