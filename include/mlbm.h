@@ -724,8 +724,8 @@ mlbm_status mlbm_mlp_train_device(mlbm_mlp* m, const float* X, const float* T, i
  *   14  porosity of the box, 1 - sum(pi r^2) / box area
  *   15  4 (y - y0) (y1 - y) / (y1 - y0)^2 (position across the box)
  * With no solid object d1 = d2 = 4 L.  Computed on the device with the
- * positions as pairs of floats and the geometry in FP32 (the features
- * feed a BF16 network): within about 1e-5 of an FP64 evaluation, except that
+ * positions, from the box's corner, as pairs of floats and the geometry in
+ * FP32 (the features feed a BF16 network): within about 1e-5 of an FP64 evaluation, except that
  * the nearest of two nearly equidistant objects, or a ray grazing a disk, may
  * be decided the other way.
  * Inputs are host arrays (copied to the device inside); synchronous.

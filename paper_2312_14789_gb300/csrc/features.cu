@@ -94,9 +94,10 @@ __device__ __forceinline__ void diff2(float a, float b, float& s, float& e) {
     e = __fadd_rn(__fsub_rn(a, __fadd_rn(s, bb)), __fsub_rn(bb, b));
 }
 
-// A double as two floats (48 bits): positions, disk centres and box lengths.
-// Differences of them are formed with their rounding errors, which gives the
-// FP32 displacement to its last bit or so; in FP64 the subtraction, the
+// A double as two floats (48 bits): positions and disk centres from the box's
+// corner (taken off in FP64, so that a box far from the origin keeps its bits),
+// and box lengths.  Differences of them are formed with their rounding errors,
+// which gives the FP32 displacement to its last bit or so; in FP64 the subtraction, the
 // division by the box length and the conversions of every disk were most of
 // the kernel on this GPU (two FP64 instructions per clock and SM).
 struct Two {
@@ -128,20 +129,21 @@ __device__ __forceinline__ float image_diff(const Two& x, const Two& c, const Tw
 struct Disk {
     Two x, y;
     float r;
-    float bx, by;  // centre moved into the box along periodic axes
+    float bx, by;  // centre from the box's corner, moved into the box along periodic axes
 };
 
 // Disks that can come within `reach` of a point of each grid cell (any of
 // their periodic images), in disk order: one block per cell, list[cell * cap
-// ..], count[cell].  margin covers FP32 rounding.
+// ..], count[cell], cells and centres counted from the box's corner.  margin
+// covers FP32 rounding.
 __global__ void __launch_bounds__(128) bin_disks(FeatGeo G, const Disk* __restrict__ disks, int ncx, int ncy,
                                                  float cw, float ch, float reach, int* __restrict__ list,
                                                  int* __restrict__ count) {
     __shared__ int warp_n[4], base;
     const int cx = blockIdx.x % ncx, cy = blockIdx.x / ncx;
-    const float x0 = (float)G.x0 + cx * cw, y0 = (float)G.y0 + cy * ch, x1 = x0 + cw, y1 = y0 + ch;
+    const float x0 = cx * cw, y0 = cy * ch, x1 = x0 + cw, y1 = y0 + ch;
     const float lx = (float)G.lx, ly = (float)G.ly;
-    const float margin = 1e-4f * (reach + fabsf(x0) + fabsf(y0) + lx + ly);
+    const float margin = 1e-4f * (reach + lx + ly);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int* out = list + (size_t)blockIdx.x * G.n_disks;
     if (threadIdx.x == 0) base = 0;
@@ -151,7 +153,7 @@ __global__ void __launch_bounds__(128) bin_disks(FeatGeo G, const Disk* __restri
         bool near = false;
         if (k < G.n_disks) {
             const Disk d = disks[k];
-            const float lim = reach + d.r + margin;
+            const float lim = reach + d.r + margin + 1e-6f * (fabsf(d.bx) + fabsf(d.by) + fabsf(d.r));
             for (int ix = -2 * G.perx; ix <= 2 * G.perx; ++ix)
                 for (int iy = -2 * G.pery; iy <= 2 * G.pery; ++iy) {
                     const float X = d.bx + ix * lx, Y = d.by + iy * ly;
@@ -187,7 +189,7 @@ __global__ void __launch_bounds__(128) features_kernel(int64_t n, const double* 
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double x = xy[2 * i], y = xy[2 * i + 1];
-    const Two x2 = two_of(x), y2 = two_of(y), lx2 = two_of(G.lx), ly2 = two_of(G.ly);
+    const Two x2 = two_of(x - G.x0), y2 = two_of(y - G.y0), lx2 = two_of(G.lx), ly2 = two_of(G.ly);
     float d1 = INFINITY, d2 = INFINITY, nx = 0.f, ny = 0.f;
     float fp[4] = {G.ell, G.ell, G.ell, G.ell};  // +x, -x, +y, -y
     float S[kRadii] = {0.f, 0.f, 0.f, 0.f};
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(128) features_kernel(int64_t n, const double* 
     const float reach = fmaxf(G.rho[kRadii - 1], G.ell);  // beyond it a disk cuts no circle and no ray
     const float lxf = (float)G.lx, lyf = (float)G.ly;
     // the node's cell (a node outside the box takes all disks)
-    const float px = (float)(x - G.x0), py = (float)(y - G.y0);
+    const float px = x2.h, py = y2.h;
     const bool inside = ncx > 0 && px >= 0.f && py >= 0.f && px <= lxf && py <= lyf;
     const int cell = inside ? min(ncy - 1, (int)(py / ch)) * ncx + min(ncx - 1, (int)(px / cw)) : 0;
     const int* ids = inside ? list + (size_t)cell * G.n_disks : nullptr;
@@ -463,10 +465,10 @@ extern "C" mlbm_status mlbm_features_device(const mlbm_nodes* nodes, const mlbm_
         return dev::Two{h, (float)(v - (double)h)};
     };
     for (int k = 0; k < nd; ++k) {
-        const double cx = geo->disks[3 * k], cy = geo->disks[3 * k + 1];
+        const double cx = geo->disks[3 * k] - G.x0, cy = geo->disks[3 * k + 1] - G.y0;  // from the box's corner
         hd[k] = {two(cx), two(cy), (float)geo->disks[3 * k + 2],
-                 (float)(G.perx ? cx - lx * std::floor((cx - G.x0) / lx) : cx),
-                 (float)(G.pery ? cy - ly * std::floor((cy - G.y0) / ly) : cy)};
+                 (float)(G.perx ? cx - lx * std::floor(cx / lx) : cx),
+                 (float)(G.pery ? cy - ly * std::floor(cy / ly) : cy)};
     }
     // one buffer: positions, disks, lists, counts
     const size_t bytes_xy = (size_t)n * 2 * sizeof(double), bytes_d = ((size_t)nd * sizeof(dev::Disk) + 15) / 16 * 16;
