@@ -353,7 +353,8 @@ mlbm_status mlbm_set_wait_limit(mlbm_ctx* ctx, double seconds);
 mlbm_status mlbm_test_withhold_copy(mlbm_ctx* ctx);
 
 /* Checkpoint the state, step count and parameters to a file / restore them
-   into a context built from the same stencils (node count and K checked). */
+   into a context built from the same stencils (node count and K checked).  A
+   batch of several samples keeps the parameters it was created with. */
 mlbm_status mlbm_save(mlbm_ctx* ctx, const char* path);
 mlbm_status mlbm_load(mlbm_ctx* ctx, const char* path);
 

@@ -1191,8 +1191,18 @@ mlbm_status mlbm_load(mlbm_ctx* c, const char* path) {
     ok = std::fread(buf.data(), 8, buf.size(), f) == buf.size();
     std::fclose(f);
     if (!ok) return set_error(MLBM_E_IO, "load: truncated file");
+    // every copy of a single sample's parameters: the host's, those in captured
+    // steps, and the table of a batch of one (a larger batch keeps its samples'
+    // own, which the file does not hold)
+    MLBM_CUDA(cudaStreamSynchronize(c->stream));
+    drop_graphs(c);
     c->params = p;
     set_collide(c);
+    if (c->seg_params.size() == 1) {
+        c->seg_params[0] = p;
+        if (c->S.coll)
+            MLBM_TRY(upload(c, const_cast<dev::Collide*>(c->S.coll), &c->C, sizeof(dev::Collide)));
+    }
     if (per == 9) {
         MLBM_TRY(upload(c, c->io, buf.data(), buf.size() * 8));
         MLBM_CUDA(launch_set_bgk((int)c->n, c->perm, c->io, c->f8[c->cur], c->f0[c->cur], c->stream));
