@@ -429,10 +429,10 @@ double mlbm_last_step_ms(const mlbm_ctx* ctx);
  *        With 27 and graphs enabled, runs of 8 or more BGK steps of a set of
  *        up to 64 tiles go to one cluster of blocks that keeps records and
  *        states in shared memory for the whole run (same results bit for bit)
- * RBF-FD stencils: where a number runs "the plain capped kernel", a BGK
- * context of a large set with stencils per Lagrangian point, or after 28 or
- * 29 was set, steps from tile records of its non-zero weights instead (same
- * results).
+ * RBF-FD stencils: 28 and 29 step a BGK context from tile records of its
+ * non-zero weights, and so does, where the context is of a large set with
+ * stencils per Lagrangian point, every number that runs "the plain capped
+ * kernel" (same results).
  * Variants 4 and up are available for K = 12, 16, 24 and 32.
  * The default is 27 when available, else 1.  mlbm_autotune times every
  * available variant for steps_per_variant steps on the context's stream

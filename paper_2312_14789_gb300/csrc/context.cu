@@ -66,6 +66,7 @@ struct mlbm_ctx {
     int variant = 27;
     std::vector<int> inv_perm;  // caller's node id -> device position
     int* err = nullptr;  // device error word of the bounded waits
+    bool rbf_tiles_default = false;  // large sets: every plain capped number steps from RBF-FD tile records
     int cluster = 0;  // blocks of the cluster that takes runs of steps (0: the set does not fit one)
     dev::Stencil S{};
     dev::Collide C{};
@@ -207,6 +208,14 @@ mlbm_status read_results(mlbm_ctx* c, double* h, size_t count) {
     return MLBM_OK;
 }
 
+// whether a number steps from RBF-FD tile records, which exist where any does
+bool by_rbf_tiles(const mlbm_ctx* c, int variant) {
+    if (!c->S.rbf_rec) return false;
+    if (variant == 28 || variant == 29) return true;
+    // the numbers that run the plain capped kernel
+    return c->rbf_tiles_default && variant != 0 && variant != 10 && variant != 12 && variant != 20 && variant != 21;
+}
+
 mlbm_status launch_one_step(mlbm_ctx* c, int variant) {
     const int a = c->cur, b = c->cur ^ 1;
     const int model = c->params.model == MLBM_MODEL_BGK ? 0 : 1;
@@ -220,8 +229,7 @@ mlbm_status launch_one_step(mlbm_ctx* c, int variant) {
             MLBM_CUDA(launch_step_warp(variant, model, c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->ruv[a],
                                        c->ruv[b], c->C, a, c->err, W, c->stream));
     }
-    else if (model == 0 && c->S.rbf_rec && variant != 0 && variant != 10 && variant != 12 && variant != 20 &&
-             variant != 21)  // the numbers that run the plain capped kernel without records
+    else if (model == 0 && by_rbf_tiles(c, variant))
         MLBM_CUDA(launch_step_rbf_tiles(c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->C, a, c->err,
                                         dev::Wait{c->wait_ns, 0}, c->stream));
     else if (model == 0)
@@ -261,8 +269,20 @@ mlbm_status launch_cluster_steps(mlbm_ctx* c, int64_t n_steps) {
 // Lagrangian point of 25 nodes in 64 slots (us a step, plain / records): 65k nodes
 // (150 MB) 25.4 / 18.8, 46k (107 MB) 20.9 / 13.5, 24k 10.3 / 10.5.  Stencils of the
 // node's own 24 have no zeros to leave out: 147k nodes 23.1 / 26.7, 260k 41.1 /
-// 44.5.  Kernel variants 28 and 29 take the records in any case.
+// 44.5.  Kernel variants 28 and 29 take the records in any case, and only they
+// where the rule does not make them the default.
 constexpr size_t kRbfTilesFrom = size_t(100) << 20;
+
+// Releases the records (no step that reads them may be in flight).
+void drop_rbf_tiles(mlbm_ctx* c) {
+    for (const void* p : {(const void*)c->S.rbf_rec, (const void*)c->S.rbf_head, (const void*)c->S.rbf_range}) {
+        c->allocations.erase(std::find(c->allocations.begin(), c->allocations.end(), p));
+        cudaFree(const_cast<void*>(p));
+    }
+    c->S.rbf_rec = nullptr;
+    c->S.rbf_head = nullptr;
+    c->S.rbf_range = nullptr;
+}
 
 // The records of the RBF-FD step from the uploaded stencils.  Where they do
 // not fit (node numbers of 28 bits, no memory) the context steps without them.
@@ -605,7 +625,10 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         c->S.stage_max = stage_max;
     }
     MLBM_CUDA(launch_record_kinds(c->S, c->rec, c->need, c->range, c->stream));
-    if (rbf && p->model == MLBM_MODEL_BGK && (size_t)n * 36 * K > kRbfTilesFrom) MLBM_TRY(build_rbf_tiles(c, false));
+    if (rbf && p->model == MLBM_MODEL_BGK && (size_t)n * 36 * K > kRbfTilesFrom) {
+        MLBM_TRY(build_rbf_tiles(c, false));
+        c->rbf_tiles_default = c->S.rbf_rec != nullptr;
+    }
     set_collide(c);
     // ---- initial state
     std::vector<double> ru((size_t)n * 3);
@@ -1282,6 +1305,10 @@ mlbm_status mlbm_autotune_ex(mlbm_ctx* c, int steps_per_variant, int flush_l2, d
     } else {
         st = save_buf(c->ruv[cur0], np * sizeof(float4));
     }
+    // RBF-FD stencils: 28 and 29 step from tile records, as after set_kernel_variant
+    const bool had_rbf_tiles = c->S.rbf_rec != nullptr;
+    if (st == MLBM_OK && c->S.Wr && c->params.model == MLBM_MODEL_BGK && tma_supported(c->K / 4) && !had_rbf_tiles)
+        st = build_rbf_tiles(c, true);
     int best = c->variant;
     double best_t = 1e30;
     c->tune_ms.assign(kMaxVariant + 1, -1.0);
@@ -1353,8 +1380,13 @@ mlbm_status mlbm_autotune_ex(mlbm_ctx* c, int steps_per_variant, int flush_l2, d
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     c->steps = steps0;
+    if (st == MLBM_OK) c->variant = best;
+    // records that the chosen number does not step from are given back
+    if (!had_rbf_tiles && c->S.rbf_rec && !by_rbf_tiles(c, c->variant)) {
+        cudaStreamSynchronize(c->stream);  // and no graph holds them: they were not there before
+        drop_rbf_tiles(c);
+    }
     if (st != MLBM_OK) return st;
-    c->variant = best;
     if (best_ms) *best_ms = best_t;
     return MLBM_OK;
 }
