@@ -264,14 +264,22 @@ mlbm_status launch_cluster_steps(mlbm_ctx* c, int64_t n_steps) {
 }
 
 // A BGK context of RBF-FD stencils steps from tile records of its non-zero weights
-// where the plain rows (36 K bytes a node) take more than 100 MB, so that they
-// come from HBM, and the records at most two thirds of that.  Stencils per
-// Lagrangian point of 25 nodes in 64 slots (us a step, plain / records): 65k nodes
-// (150 MB) 25.4 / 18.8, 46k (107 MB) 20.9 / 13.5, 24k 10.3 / 10.5.  Stencils of the
-// node's own 24 have no zeros to leave out: 147k nodes 23.1 / 26.7, 260k 41.1 /
-// 44.5.  Kernel variants 28 and 29 take the records in any case, and only they
-// where the rule does not make them the default.
-constexpr size_t kRbfTilesFrom = size_t(100) << 20;
+// where the plain rows (36 K bytes a node) take more than 60 MB and the records at
+// most two thirds of that.  From about 55 MB on, the plain step depends on where
+// the rows happen to lie in L2: the same set took up to 40% longer in one process
+// than in another, while the records, of half the size, always took the same.  us a
+// step, plain least .. median .. most of eight processes / records:
+//   K = 64, 25 nodes a point: 38 MB 9.5 .. 9.6 .. 9.6 / 6.6, 55 MB 9.8 .. 11.4 ..
+//   12.5 / 9.6, 66 MB 10.2 .. 14.2 .. 14.7 / 11.9, 79 MB 12.5 .. 16.0 .. 16.4 /
+//   11.9, 87 MB 14.4 .. 17.6 .. 18.0 / 12.6; 150 MB 25.4 / 18.8
+//   K = 48, 15 nodes: 54 MB 8.2 / 9.6, 59 MB 8.7 / 10.0, 73 MB 13.0 .. 14.4 .. 14.9 / 10.3
+//   K = 32, 7 nodes: 39 MB 6.3 / 8.0, 64 MB 9.8 .. 10.9 .. 11.1 / 9.4, 75 MB 10.6 ..
+//   12.3 .. 13.3 / 11.6, 88 MB 12.7 .. 15.2 .. 15.5 / 12.1
+// Below the line the winner changes with K.  Stencils of the node's own 24 have no
+// zeros to leave out: 147k nodes 23.1 / 26.7, 260k 41.1 / 44.5.  Kernel variants 28
+// and 29 take the records in any case, and only they where the rule does not make
+// them the default.
+constexpr size_t kRbfTilesFrom = 60000000;
 
 // Releases the records (no step that reads them may be in flight).
 void drop_rbf_tiles(mlbm_ctx* c) {

@@ -60,10 +60,13 @@ def test_autotune_times_the_records(M):
     assert np.array_equal(M.get_populations(ctx), M.get_populations(ref))
 
 
-def test_large_sets_step_from_records_by_default(M):
-    w = I.poiseuille_channel(300, 157, 0.2, seed=4)  # 47,100 nodes of 2.3 KB
+@pytest.mark.parametrize("nx,ny,large", [(160, 150, False), (190, 145, True), (300, 157, True)])
+def test_large_sets_step_from_records_by_default(M, nx, ny, large):
+    """Plain rows of 55, 63 and 109 MB: records from 60 MB on."""
+    w = I.poiseuille_channel(nx, ny, 0.2, seed=4)
     st = M.build_stencils_for(w, K=64, s=0.5, bb_mode=1, interp=M.INTERP_RBF_POINTS, n_l=25)
-    ctx = M.init(st, M.Params(M.MODEL_BGK, 0.8, 0.0, 1e-5, 0.0))
-    for variant, records in ((1, True), (0, False)):
-        M.set_kernel_variant(ctx, variant)
-        assert (RECORDS in _kernels(lambda: M.step(ctx, 2))) == records, variant
+    ctx, ref = (M.init(st, M.Params(M.MODEL_BGK, 0.8, 0.0, 1e-5, 0.0)) for _ in range(2))
+    assert (RECORDS in _kernels(lambda: M.step(ctx, 2))) == large
+    M.set_kernel_variant(ref, 0)
+    assert RECORDS not in _kernels(lambda: M.step(ref, 2))
+    assert np.array_equal(M.get_populations(ctx), M.get_populations(ref))
