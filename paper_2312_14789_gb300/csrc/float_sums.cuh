@@ -13,7 +13,10 @@
 // their last bits 2^-136), when |u|^2 A, the one product of three values, is
 // neither zero nor within [2^-77, 2^110] (at the lower end the third of its
 // parts rounds at 2^-149, 2^-72 of it; kFlush terms at the upper end add up to
-// 2^118), and for infinities and NaN.  13.25M nodes: 523 -> 148 us.
+// 2^118), and for infinities and NaN.  13.25M nodes: 523 -> 144 us.  Blocks of
+// one or two nodes a thread keep to FP64, whose pipe they do not fill, and skip
+// the flush (us a call, FP64 / FP32 pipe: 64 nodes 8.9 / 10.4, 256 10.0 / 11.4,
+// 512 11.6 / 12.1; FP64 alone at 600 12.5 / 12.3, at 1000 17.0 / 13.7).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -70,6 +73,7 @@ struct Float3Sum {
 // sums of A, rho A, ux A, uy A, |u| A, |u|^2 A
 struct FieldSums {
     static constexpr int kFlush = 256;
+    static constexpr int kFew = 2;  // nodes a thread up to which add64 is the faster one
     static constexpr float kLeast = 6.617444900424222e-24f, kMost = 1.298074214633707e33f;  // 2^-77, 2^110
     Float3Sum f[6];
     double s[6] = {0, 0, 0, 0, 0, 0};
@@ -79,6 +83,15 @@ struct FieldSums {
         const float a = fabsf(x);
         return x == 0.f || (a >= 2.84217094304040074e-14f && a <= 3.5184372088832e13f);
     }
+    __device__ __forceinline__ void add64(float rho, float u, float v, float a) {
+        const double da = a, du = u, dv = v, m2 = du * du + dv * dv;
+        s[0] += da;
+        s[1] += (double)rho * da;
+        s[2] += du * da;
+        s[3] += dv * da;
+        s[4] += sqrt(m2) * da;
+        s[5] += m2 * da;
+    }
     __device__ __forceinline__ void add(float rho, float u, float v, float a) {
         // |u|^2 = p + e + q + g, and x0 its leading part
         float p, e, q, g, x0, x1, x2, t, w;
@@ -87,13 +100,7 @@ struct FieldSums {
         exact_sum(p, q, x0, t);
         const float m2a = fabsf(__fmul_rn(x0, a));
         if (!(plain(rho) && plain(u) && plain(v) && plain(a) && (m2a == 0.f || (m2a >= kLeast && m2a <= kMost)))) {
-            const double da = a, du = u, dv = v, m2 = du * du + dv * dv;
-            s[0] += da;
-            s[1] += (double)rho * da;
-            s[2] += du * da;
-            s[3] += dv * da;
-            s[4] += sqrt(m2) * da;
-            s[5] += m2 * da;
+            add64(rho, u, v, a);
             return;
         }
         f[0].add(a);
@@ -123,6 +130,7 @@ struct FieldSums {
         if (++held == kFlush) flush();
     }
     __device__ __forceinline__ void flush() {
+        if (!held) return;
 #pragma unroll
         for (int q = 0; q < 6; ++q) f[q].flush(s[q]);
         held = 0;

@@ -335,8 +335,12 @@ __global__ void __launch_bounds__(kRedThreads, 4) reduce_fields_partial(int64_t 
         for (int j = 0; j < 4; ++j)
             if (m[j]) t.add(r[j], u[j], v[j], a[j]);
     }
+    const bool few = n <= FieldSums::kFew * stride;
     for (; i < n; i += stride)
-        if (!mask || mask[i]) t.add(rho[i], ux[i], uy[i], area[i]);
+        if (!mask || mask[i]) {
+            if (few) t.add64(rho[i], ux[i], uy[i], area[i]);
+            else t.add(rho[i], ux[i], uy[i], area[i]);
+        }
     t.flush();
     block_tuple<6>(t.s, partial + 6 * (size_t)blockIdx.x);
 }
@@ -376,6 +380,7 @@ __global__ void __launch_bounds__(kRedThreads) observe_partial(const int64_t* __
 #pragma unroll
     for (int q = 0; q < W; ++q) s[q] = 0.0;
     FieldSums t;
+    const bool few = end - first <= FieldSums::kFew * (int64_t)nb * kRedThreads;
     for (int64_t i = first + blockIdx.x * (int64_t)kRedThreads + threadIdx.x; i < end; i += (int64_t)nb * kRedThreads) {
         float rho, u, v;
         if (MODEL == 0) {
@@ -395,7 +400,10 @@ __global__ void __launch_bounds__(kRedThreads) observe_partial(const int64_t* __
                 s[0] += du * du + dv * dv;
                 s[1] += (double)u * u + (double)v * v;
             }
-            if (FIELDS) t.add(rho, u, v, area[i]);
+            if (FIELDS) {
+                if (few) t.add64(rho, u, v, area[i]);
+                else t.add(rho, u, v, area[i]);
+            }
         }
         if (CHANGE) {
             px[i] = u;
