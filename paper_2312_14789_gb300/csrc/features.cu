@@ -449,14 +449,17 @@ extern "C" mlbm_status mlbm_features_device(const mlbm_nodes* nodes, const mlbm_
     for (int k = 0; k < geo->n_disks; ++k) solid += dev::kPi * geo->disks[3 * k + 2] * geo->disks[3 * k + 2];
     G.porosity = (float)(1.0 - solid / (lx * ly));
     // grid of the disk lists: cells of a quarter of the reach, at most 32 MB
-    // of lists, none when the disks are few enough to look at all of them
+    // of lists (fewer, longer cells in a thin box), none when the disks are few
+    // enough to look at all of them
     const int nd = geo->n_disks;
     const double reach = std::fmax((double)G.rho[dev::kRadii - 1], (double)G.ell);
     int ncx = 0, ncy = 0;
     if (nd >= 16) {
-        const double edge = std::fmax(0.25 * reach, std::sqrt(lx * ly * nd / (double(32 << 20) / sizeof(int))));
-        ncx = std::max(1, (int)std::ceil(lx / edge));
-        ncy = std::max(1, (int)std::ceil(ly / edge));
+        const double most = std::fmax(1.0, std::floor(double(32 << 20) / sizeof(int) / nd));  // cells
+        const double edge = std::fmax(0.25 * reach, std::sqrt(lx * ly / most));
+        const double wide = std::ceil(lx / edge), high = std::ceil(ly / edge);
+        ncx = (int)std::fmax(1.0, std::fmin(wide, most / std::fmin(high, most)));
+        ncy = (int)std::fmax(1.0, std::fmin(high, most / ncx));
     }
     const size_t cells = (size_t)ncx * ncy;
     std::vector<dev::Disk> hd(nd);
