@@ -282,6 +282,8 @@ mlbm_status mlbm_lattice_init(mlbm_lattice** out, int nx, int ny, int periodic_x
     // rest state (shifted populations zero), equilibrium cells at their values
     if (e == cudaSuccess) e = cudaMemset(L->f[0], 0, 9 * n * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(L->f[1], 0, 9 * n * sizeof(float));
+    // steps run on a stream that does not wait for the default stream's work
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     for (int from = 0; from < 2 && e == cudaSuccess; ++from) e = capture_lattice(L, from);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();

@@ -24,3 +24,11 @@ def test_no_bounded_wait_is_dropped():
             recorded = code.rfind("atomicExch(err", 0, at)
             assert recorded >= 0 and "}" not in code[recorded:at], (os.path.basename(path), code[at:at + 60])
     assert waits >= 15
+
+
+def test_lattice_is_handed_out_with_its_buffers_set():
+    code = re.sub(r"//[^\n]*|/\*.*?\*/", " ", open(os.path.join(CSRC, "lattice.cu")).read(), flags=re.S)
+    init = code[code.index("mlbm_lattice_init("):code.index("void mlbm_lattice_destroy(")]
+    assert "cudaStreamNonBlocking" in init
+    last = max(m.end() for m in re.finditer(r"cudaMem(?:set|cpy)\(", init))
+    assert "cudaStreamSynchronize(nullptr)" in init[last:init.index("*out = L")]
