@@ -108,11 +108,12 @@ def algorithmic_bytes(info, K, model="bgk", rows=6):
 
 
 def kernel_source_hash():
+    """Of every step kernel's source and every device header."""
+    csrc = os.path.join(ROOT, "paper_2312_14789_gb300", "csrc")
     h = hashlib.sha256()
-    for f in ("kernels.cu", "kernels_bgk.cu", "kernels_bgk_generic.cu", "kernels_bgk_alt.cu", "kernels_tau1.cu",
-              "kernels_rbf.cu", "kernels_warp.cu",
-              "kernels_tma.cu", "step_node.cuh", "ring.cuh", "launch_util.cuh", "device_common.cuh"):
-        h.update(open(os.path.join(ROOT, "paper_2312_14789_gb300", "csrc", f), "rb").read())
+    for f in sorted(os.listdir(csrc)):
+        if f.endswith(".cuh") or (f.startswith("kernels") and f.endswith(".cu")):
+            h.update(open(os.path.join(csrc, f), "rb").read())
     return h.hexdigest()[:16]
 
 
