@@ -335,7 +335,9 @@ mlbm_status mlbm_run_to_steady_mean(mlbm_ctx* ctx, double threshold, int64_t dn,
 
 /*
  * Bounded device waits.  The bulk-copy step variants (4..7, 27..29) wait on
- * shared-memory barriers for their tile copies; each wait gives up after
+ * shared-memory barriers for their tile copies, and so do the cluster runs of
+ * 27 and RBF-FD contexts under every number that steps from tile records (see
+ * mlbm_set_kernel_variant); each wait gives up after
  * `seconds` (default 2; accepted range [1e-4, 60]), records an error word,
  * waits (bounded again) for the copies it issued and returns, and the next
  * call that synchronises the context returns MLBM_E_TIMEOUT with the step's
@@ -345,8 +347,9 @@ mlbm_status mlbm_run_to_steady_mean(mlbm_ctx* ctx, double threshold, int64_t dn,
 mlbm_status mlbm_set_wait_limit(mlbm_ctx* ctx, double seconds);
 /*
  * Test of the bounded waits: the next step launch (which must use a
- * bulk-copy variant, 4..7 or 27..29, else MLBM_E_INVALID) issues no copies for
- * the first tile of its first block, so that block's consumers wait for a
+ * bulk-copy variant, 4..7 or 27..29, of least-squares stencils, else
+ * MLBM_E_INVALID) issues no copies for the first tile of its first block (a
+ * cluster run: for the first block), so that block's consumers wait for a
  * tile that never arrives until the wait limit runs out.  One launch only;
  * it is launched directly, never from a captured graph.  No paper counterpart.
  */

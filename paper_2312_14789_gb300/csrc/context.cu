@@ -88,7 +88,7 @@ struct mlbm_ctx {
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     int graph_variant = -1;
     cudaStream_t graph_stream = nullptr;
-    // bounded waits of the bulk-copy ring variants (4..7): budget of one wait,
+    // bounded waits of the bulk-copy variants (4..7, 27..29): budget of one wait,
     // and the test switch that makes the next launch withhold one tile
     unsigned long long wait_ns = 2000000000ULL;
     int withhold_next = 0;
@@ -249,14 +249,16 @@ constexpr int kClusterMin = 8;
 constexpr int kClusterSteps = 4096;  // most steps of one launch
 
 bool by_cluster(const mlbm_ctx* c, int64_t n_steps, int variant) {
-    return c->cluster > 0 && variant == 27 && c->use_graphs && n_steps >= kClusterMin && !c->withhold_next;
+    return c->cluster > 0 && variant == 27 && c->use_graphs && n_steps >= kClusterMin;
 }
 
 mlbm_status launch_cluster_steps(mlbm_ctx* c, int64_t n_steps) {
     for (int64_t left = n_steps; left > 0;) {
         const int m = (int)std::min<int64_t>(left, kClusterSteps), a = c->cur, b = a ^ (m & 1);
-        MLBM_CUDA(launch_step_cluster(c->cluster, c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->C, m, c->err,
-                                      dev::Wait{c->wait_ns, 0}, c->stream));
+        const dev::Wait W{c->wait_ns, c->withhold_next};
+        c->withhold_next = 0;
+        MLBM_CUDA(launch_step_cluster(c->cluster, c->S, c->f8[a], c->f0[a], c->f8[b], c->f0[b], c->C, m, c->err, W,
+                                      c->stream));
         c->cur = b;
         left -= m;
     }

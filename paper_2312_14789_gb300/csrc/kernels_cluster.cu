@@ -21,7 +21,8 @@
 namespace mlbm {
 namespace dev {
 
-// all blocks of the cluster (one that has given up and left does not hold it)
+// all blocks of the cluster (one whose records never came steps nothing, but
+// takes part in every barrier)
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -200,10 +201,13 @@ __global__ void __launch_bounds__(kClusterWarps * 32, 1)
     // states behind the records: buffer b of tile i at (b * per + i) * 32 nodes
     float4* states = reinterpret_cast<float4*>(smem + (size_t)per * kBytes);
     const uint32_t buffer_bytes = (uint32_t)per * 32 * kState * 16;
-    if (threadIdx.x == 0) {  // what each tile needs of its record (see step_warp), all on one barrier
+    const bool withhold = W.withhold && blockIdx.x == 0;  // test switch: the block's copies are never issued
+    if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (threadIdx.x == 0 && !withhold) {  // what each tile needs of its record (see step_warp), all on one barrier
         uint32_t bytes = 0;
         for (int i = 0; i < nt; ++i) {
             const int need = S.need[t0 + i];
@@ -236,7 +240,7 @@ __global__ void __launch_bounds__(kClusterWarps * 32, 1)
     const bool ok = __syncthreads_and(mbar_wait(&bar, 0, W.budget_ns));
     if (!ok && threadIdx.x == 0) {
         atomicExch(err, 2);
-        mbar_wait(&bar, 0, W.budget_ns);  // do not leave while copies may still be landing
+        if (!withhold) mbar_wait(&bar, 0, W.budget_ns);  // do not leave while copies may still be landing
     }
     const float4* base = reinterpret_cast<const float4*>(smem + (size_t)warp * kBytes) + lane;
     const bool mine = ok && warp < nt;
