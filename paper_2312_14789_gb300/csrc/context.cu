@@ -3,6 +3,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -360,7 +361,12 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
     // ---- host-side device layout
     const bool rbf = H.interp != MLBM_INTERP_WLS;  // per-direction RBF-FD weights
     const int rows = 7 * Kq - 1, sp = dev::special_group(Kq);
-    std::vector<int32_t> hrec(rbf ? 0 : (size_t)(np / 32) * rows * 128, 0);
+    // (tile records: cleared on all cores, 81 MB at 185k nodes of K = 16, which one
+    // core fills in 4.4 ms)
+    const size_t tile_words = (size_t)rows * 128, n_words = rbf ? 0 : (size_t)(np / 32) * tile_words;
+    const std::unique_ptr<int32_t[]> hrec(new int32_t[n_words]);
+#pragma omp parallel for schedule(static, 128)
+    for (int64_t t = 0; t < (rbf ? 0 : np / 32); ++t) std::fill_n(hrec.get() + (size_t)t * tile_words, tile_words, 0);
     std::vector<int32_t> hidx(rbf ? (size_t)Kq * np * 4 : 0, 0);
     std::vector<float> hW(rbf ? (size_t)8 * Kq * np * 4 : 0, 0.f);
     std::vector<uint8_t> hmeta(np, 0), hmask(np, 0);
@@ -390,7 +396,7 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         // sample of a batch's node, and the node's lane in its tile record
         const int sample =
             parts ? (int)(std::upper_bound(H.part_off.begin(), H.part_off.end(), q) - H.part_off.begin()) - 1 : 0;
-        int32_t* lane = rbf ? nullptr : hrec.data() + ((size_t)(q / 32) * rows * 32 + q % 32) * 4;
+        int32_t* lane = rbf ? nullptr : hrec.get() + (size_t)(q / 32) * tile_words + (q % 32) * 4;
         if (!rbf) lane[sp * 128 + 3] = (int32_t)hmeta[q] | (sample << 8);
         if (kind == kKindWls) {
             // stencil slots in increasing node position: lanes of a warp that
@@ -463,7 +469,7 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
     }
     // lanes past the last node read as equilibrium nodes, which gather nothing
     for (int64_t q = n; !rbf && q < np; ++q)
-        hrec[((size_t)(q / 32) * rows * 32 + q % 32) * 4 + (size_t)sp * 128 + 3] = kKindEq;
+        hrec[(size_t)(q / 32) * tile_words + (q % 32) * 4 + (size_t)sp * 128 + 3] = kKindEq;
     c->n_link_nodes = (int)hlinknodes.size();
     c->inv_perm.assign((size_t)n, -1);
     for (int64_t q = 0; q < n; ++q) c->inv_perm[(size_t)hperm[q]] = (int)q;
@@ -477,28 +483,29 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         const int64_t T = dev::kStageTile, nt = (n + T - 1) / T;
         std::vector<std::vector<int>> lists((size_t)nt);
         hlidx.assign((size_t)Kq * np * 4, 0);
-        auto member = [&](int64_t q, int jj) {
-            return hrec.data() + ((size_t)(q / 32) * rows * 32 + q % 32) * 4 + (size_t)(jj / 4) * 128 + jj % 4;
-        };
+        auto lane_of = [&](int64_t q) { return hrec.get() + (size_t)(q / 32) * tile_words + (q % 32) * 4; };
 #pragma omp parallel for schedule(dynamic, 8)
         for (int64_t b = 0; b < nt; ++b) {
             std::vector<int>& L = lists[(size_t)b];
             const int64_t q0 = b * T, q1 = std::min<int64_t>(n, q0 + T);
             for (int64_t q = q0; q < q1; ++q)
                 if ((hmeta[q] & 7) == 0)
-                    for (int jj = 0; jj < K; ++jj)
-                        if (jj != 4 * sp + 3) L.push_back(*member(q, jj));
+                    for (int g = 0; g < Kq; ++g) {
+                        const int32_t* id = lane_of(q) + g * 128;
+                        L.insert(L.end(), id, id + (g == sp ? 3 : 4));
+                    }
             std::sort(L.begin(), L.end());
             L.erase(std::unique(L.begin(), L.end()), L.end());
             if ((int64_t)L.size() > dev::kStageMax) continue;  // too wide: the whole structure is dropped below
             for (int64_t q = q0; q < q1; ++q)
                 if ((hmeta[q] & 7) == 0)
-                    for (int jj = 0; jj < K; ++jj) {
-                        // the freed slot, whose weight is zero, repeats the first member
-                        const int id = *member(q, jj == 4 * sp + 3 ? 0 : jj);
-                        hlidx[(((size_t)(jj / 4)) * np + q) * 4 + (jj % 4)] =
-                            (uint16_t)(std::lower_bound(L.begin(), L.end(), id) - L.begin());
-                    }
+                    for (int g = 0; g < Kq; ++g)
+                        for (int cc = 0; cc < 4; ++cc) {
+                            // the freed slot, whose weight is zero, repeats the first member
+                            const int id = lane_of(q)[g == sp && cc == 3 ? 0 : g * 128 + cc];
+                            hlidx[((size_t)g * np + q) * 4 + cc] =
+                                (uint16_t)(std::lower_bound(L.begin(), L.end(), id) - L.begin());
+                        }
         }
         hsoff.assign((size_t)nt + 1, 0);
         for (int64_t b = 0; b < nt; ++b) {
@@ -522,7 +529,7 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         MLBM_TRY(dalloc(c, &c->idx, (size_t)Kq * np));
         MLBM_TRY(dalloc(c, &dW, (size_t)8 * Kq * np));
     } else {
-        MLBM_TRY(dalloc(c, &c->rec, hrec.size() / 4));
+        MLBM_TRY(dalloc(c, &c->rec, n_words / 4));
         MLBM_TRY(dalloc(c, &c->need, (size_t)np / 32));
         MLBM_TRY(dalloc(c, &c->range, (size_t)c->S.n_ranges + 1));
     }
@@ -576,7 +583,7 @@ mlbm_status do_init(mlbm_ctx* c, const mlbm_stencils* st, const mlbm_params* p, 
         MLBM_TRY(upload(c, c->idx, hidx.data(), hidx.size() * 4));
         MLBM_TRY(upload(c, dW, hW.data(), hW.size() * 4));
     } else {
-        MLBM_TRY(upload(c, c->rec, hrec.data(), hrec.size() * 4));
+        MLBM_TRY(upload(c, c->rec, hrec.get(), n_words * 4));
     }
     MLBM_TRY(upload(c, c->meta, hmeta.data(), np));
     MLBM_TRY(upload(c, c->mask, hmask.data(), np));
