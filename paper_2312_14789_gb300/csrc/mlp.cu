@@ -112,9 +112,14 @@ __device__ __forceinline__ void image_put(Image* I, int no, int i, float v) {
     else I->b4[i - off_b4(no)] = v;
 }
 
-__global__ void refresh_image(int kp, int no, const float* __restrict__ P, Image* __restrict__ I) {
+// the image of new parameters, and Adam's moments back at zero
+__global__ void take_params(int kp, int no, const float* __restrict__ P, Image* __restrict__ I, float* __restrict__ m,
+                            float* __restrict__ v) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < kp) image_put(I, no, i, P[i]);
+    if (i >= kp) return;
+    image_put(I, no, i, P[i]);
+    m[i] = 0.f;
+    v[i] = 0.f;
 }
 
 // The image into the block's shared memory, 16 bytes a thread at a time past the
@@ -667,9 +672,7 @@ void mlbm_mlp_destroy(mlbm_mlp* m) {
 mlbm_status mlbm_mlp_set_params(mlbm_mlp* m, const float* params) {
     if (!m || !params) return set_error(MLBM_E_INVALID, "mlp_set_params: NULL argument");
     MLP_CUDA(cudaMemcpy(m->p, params, m->kp * 4, cudaMemcpyHostToDevice));
-    MLP_CUDA(cudaMemset(m->m, 0, m->kp * 4));
-    MLP_CUDA(cudaMemset(m->v, 0, m->kp * 4));
-    mlp::refresh_image<<<(m->kp + 255) / 256, 256>>>(m->kp, m->n_out, m->p, m->img);
+    mlp::take_params<<<(m->kp + 255) / 256, 256>>>(m->kp, m->n_out, m->p, m->img, m->m, m->v);
     MLP_CUDA(cudaGetLastError());
     MLP_CUDA(cudaStreamSynchronize(nullptr));
     m->t = 0;
