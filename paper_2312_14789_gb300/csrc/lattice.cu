@@ -243,29 +243,36 @@ mlbm_status mlbm_lattice_init(mlbm_lattice** out, int nx, int ny, int periodic_x
             if (cell[i] == 2)
                 he[i] = make_float4((float)(eq_values[3 * i] - 1.0), (float)eq_values[3 * i + 1],
                                     (float)eq_values[3 * i + 2], 0.f);
-    // what each cell does in a step, and the cells with solid links
+    // what each cell does in a step, and the cells with solid links in cell
+    // order; the rows on all cores
     std::vector<uint16_t> info(n, 0);
-    std::vector<int2> wall;
-    for (int y = 0; y < ny; ++y)
+    std::vector<std::vector<int2>> row_wall((size_t)ny);
+#pragma omp parallel for schedule(static, 8)
+    for (int y = 0; y < ny; ++y) {
+        static const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+        // the rows that populations with e_y = -1, 0, 1 come from, and those outside
+        const int sy[3] = {y + 1 < ny ? y + 1 : 0, y, y > 0 ? y - 1 : ny - 1};
+        const bool out_y[3] = {!L->py && y + 1 == ny, false, !L->py && y == 0};
         for (int x = 0; x < nx; ++x) {
             const size_t i = (size_t)y * nx + x;
             if (cell[i] != dev::kCellFluid) {
                 info[i] = cell[i] == dev::kCellSolid ? dev::kInfoSolid : dev::kInfoEq;
                 continue;
             }
-            static const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1}, ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+            const int sx[3] = {x + 1 < nx ? x + 1 : 0, x, x > 0 ? x - 1 : nx - 1};
+            const bool out_x[3] = {!L->px && x + 1 == nx, false, !L->px && x == 0};
             int bounce = 0, solid = 0;
             for (int k = 1; k < 9; ++k) {
-                int sx = x - ex[k], sy = y - ey[k];
-                const bool outside = (!L->px && (sx < 0 || sx >= nx)) || (!L->py && (sy < 0 || sy >= ny));
-                sx = (sx + nx) % nx;
-                sy = (sy + ny) % ny;
-                if (!outside && cell[(size_t)sy * nx + sx] == dev::kCellSolid) solid |= 1 << (k - 1);
-                if (outside) bounce |= 1 << (k - 1);
+                const int a = ex[k] + 1, b = ey[k] + 1;
+                if (out_x[a] || out_y[b]) bounce |= 1 << (k - 1);
+                else if (cell[(size_t)sy[b] * nx + sx[a]] == dev::kCellSolid) solid |= 1 << (k - 1);
             }
             info[i] = (uint16_t)(bounce | solid);
-            if (solid) wall.push_back(make_int2((int)i, solid));
+            if (solid) row_wall[(size_t)y].push_back(make_int2((int)i, solid));
         }
+    }
+    std::vector<int2> wall;
+    for (const auto& r : row_wall) wall.insert(wall.end(), r.begin(), r.end());
     L->n_wall = (int)wall.size();
     cudaError_t e = cudaStreamCreateWithFlags(&L->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaMalloc(&L->info, n * sizeof(uint16_t));
@@ -284,7 +291,7 @@ mlbm_status mlbm_lattice_init(mlbm_lattice** out, int nx, int ny, int periodic_x
     if (e == cudaSuccess) e = cudaMemset(L->f[1], 0, 9 * n * sizeof(float));
     // steps run on a stream that does not wait for the default stream's work
     if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
-    for (int from = 0; from < 2 && e == cudaSuccess; ++from) e = capture_lattice(L, from);
+    if (e == cudaSuccess) e = capture_lattice(L, 0);  // the one from buffer 1 when steps first start there
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         free_lattice(L);
@@ -300,6 +307,7 @@ mlbm_status mlbm_lattice_step(mlbm_lattice* L, int64_t n_steps) {
     if (!L || n_steps < 0) return set_error(MLBM_E_INVALID, "lattice_step: bad arguments");
     int64_t left = n_steps;
     for (; left >= kLatGraph; left -= kLatGraph) {
+        if (!L->graph[L->cur]) LAT_CUDA(capture_lattice(L, L->cur));
         LAT_CUDA(cudaGraphLaunch(L->graph[L->cur], L->stream));
     }
     for (; left > 0; --left) LAT_CUDA(launch_lattice_step(L));
