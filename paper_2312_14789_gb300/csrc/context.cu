@@ -1784,15 +1784,21 @@ void free_part(mlbm_part* P) {
 int state_width(const mlbm_part* P) { return P->model == MLBM_MODEL_BGK ? 2 : 1; }
 
 template <class T>
-mlbm_status part_upload(mlbm_part* P, T** dst, const std::vector<T>& src) {
+mlbm_status part_alloc(mlbm_part* P, T** dst, size_t count) {
     void* d = nullptr;
-    if (cudaMalloc(&d, std::max<size_t>(src.size(), 1) * sizeof(T)) != cudaSuccess) {
+    if (cudaMalloc(&d, std::max<size_t>(count, 1) * sizeof(T)) != cudaSuccess) {
         (void)cudaGetLastError();
         return set_error(MLBM_E_OOM, "part_init: cudaMalloc");
     }
     P->allocations.push_back(d);
     *dst = static_cast<T*>(d);
-    MLBM_CUDA(cudaMemcpyAsync(d, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, P->stream));
+    return MLBM_OK;
+}
+
+template <class T>
+mlbm_status part_upload(mlbm_part* P, T** dst, const std::vector<T>& src) {
+    MLBM_TRY(part_alloc(P, dst, src.size()));
+    MLBM_CUDA(cudaMemcpyAsync(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, P->stream));
     MLBM_CUDA(cudaStreamSynchronize(P->stream));
     return MLBM_OK;
 }
@@ -1917,7 +1923,7 @@ mlbm_status mlbm_part_init(mlbm_part** out, const mlbm_stencils* st, const mlbm_
             }
     P->n_copies = (int64_t)halo.size();
     mlbm_status us = part_upload(P, &P->halo, halo);
-    if (us == MLBM_OK) us = part_upload(P, &P->io, std::vector<double>(9 * (size_t)P->n));
+    if (us == MLBM_OK) us = part_alloc(P, &P->io, 9 * (size_t)P->n);
     if (us == MLBM_OK) us = part_upload(P, &P->err, std::vector<int>(n_parts, 0));
     if (us != MLBM_OK) return fail(us);
     // the step's blocks, shared out by node count
@@ -1965,7 +1971,7 @@ mlbm_status mlbm_part_init(mlbm_part** out, const mlbm_stencils* st, const mlbm_
     mlbm_status s = exchange(P);
     if (s == MLBM_OK) s = part_sync(P);
     P->graph_variant = P->ctx[0]->variant;
-    for (int parity = 0; parity < 2 && s == MLBM_OK; ++parity) s = part_graph(P, parity);
+    if (s == MLBM_OK) s = part_graph(P, 0);  // the one from buffer 1 when steps first start there
     if (s != MLBM_OK) return fail(s);
     *out = P;
     return MLBM_OK;
