@@ -73,17 +73,6 @@ __global__ void set_tau1_from_f64(int n, const int* __restrict__ perm, const dou
     s[p] = make_float4((float)(v[0] - 1.0), (float)v[1], (float)v[2], 0.f);
 }
 
-__global__ void get_tau1_to_f64(int n, const int* __restrict__ perm, const float4* __restrict__ s,
-                                double* __restrict__ ru) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    double* v = ru + 3 * (size_t)perm[p];
-    const float4 a = s[p];
-    v[0] = (double)a.x + 1.0;
-    v[1] = a.y;
-    v[2] = a.z;
-}
-
 // (rho - 1, ux, uy) of a BGK state: rho = sum f, rho u = sum f e - rho a / 2
 __device__ __forceinline__ void bgk_moments(const float4& a, const float4& b, float g0, float ax, float ay, float& dr,
                                             float& ux, float& uy) {
@@ -446,11 +435,6 @@ cudaError_t launch_set_bgk_equilibrium(int n, const int* perm, const double* ru,
 cudaError_t launch_set_tau1(int n, const int* perm, const double* ru, float4* s, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     dev::set_tau1_from_f64<<<blocks_for(n, 256), 256, 0, st>>>(n, perm, ru, s);
-    return cudaGetLastError();
-}
-cudaError_t launch_get_tau1(int n, const int* perm, const float4* s, double* ru, cudaStream_t st) {
-    if (n == 0) return cudaSuccess;
-    dev::get_tau1_to_f64<<<blocks_for(n, 256), 256, 0, st>>>(n, perm, s, ru);
     return cudaGetLastError();
 }
 cudaError_t launch_macroscopics(int model, int n, const int* perm, const float4* f8, const float* f0,

@@ -78,7 +78,6 @@ cudaError_t rbf_tile_fill(const dev::Stencil& S, int tiles, const int4* head, ui
 cudaError_t launch_step_rbf_tiles(const dev::Stencil& S, const float4* in, const float* f0in, float4* out,
                                   float* f0out, const dev::Collide& C, int backward, int* err, const dev::Wait& W,
                                   cudaStream_t st);
-cudaError_t launch_get_tau1(int n, const int* perm, const float4* s, double* ru, cudaStream_t st);
 cudaError_t launch_macroscopics(int model, int n, const int* perm, const float4* f8, const float* f0,
                                 const float4* ruv, float ax, float ay, const uint16_t* node_sample,
                                 const dev::Collide* coll, int split, double* out, cudaStream_t st);

@@ -65,7 +65,6 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);
 }
-__device__ __forceinline__ uint32_t ld32(const __nv_bfloat16* p) { return *reinterpret_cast<const uint32_t*>(p); }
 
 __device__ __forceinline__ void mma(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
     asm volatile(
@@ -273,7 +272,6 @@ struct GradSmem {
     __nv_bfloat16 dz[3][kRound * kS64];
     __nv_bfloat16 dy[kRound * 8];
     double loss[kGradWarps];
-    float bias[kGradWarps * 32];
 };
 
 // store a warp's [16 rows x 64] A fragments row-major
