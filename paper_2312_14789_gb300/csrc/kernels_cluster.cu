@@ -180,11 +180,12 @@ __device__ __forceinline__ void cluster_node(const Stencil& S, const ClusterStat
 }
 
 // Tiles (and warps) of a block.  More of them share the block's and the cluster's
-// shared-memory ports, and at eight launches of dependent grids are as fast: us a
-// step, launches / cluster, K = 12: 500 nodes (one tile a block) 2.97 / 1.85, 2000
-// nodes (four) 2.97 / 1.98, 3774 nodes (eight) 3.10 / 2.90; K = 16: 3.22 / 2.26,
-// 3.27 / 2.71, 3.48 / 3.83; K = 24: 4.14 / 3.54, 4.43 / 3.93, 4.60 / 5.56.  (With
-// the states in L2 and the same barrier: 2.18 at 2000 nodes, K = 12.)
+// shared-memory ports, and at eight launches of dependent grids are as fast, or
+// faster from K = 16 on (K = 12 is still 7% ahead there; one limit serves every
+// K).  us a step, launches / cluster, at 500 nodes (one tile a block), 2000
+// (four) and 3774 (eight): K = 12 2.97 / 1.85, 2.97 / 1.98, 3.10 / 2.90; K = 16
+// 3.22 / 2.26, 3.27 / 2.71, 3.48 / 3.83; K = 24 4.14 / 3.54, 4.43 / 3.93, 4.60 /
+// 5.56.  (With the states in L2 and the same barrier: 2.18 at 2000 nodes, K = 12.)
 constexpr int kClusterWarps = 4;
 
 template <int KQ>

@@ -12,8 +12,9 @@
 // gathers, and no register holds a row.  No warp waits for another one.
 //   - Twelve slots (166 KB) leave 62 KB of L1 to the gathers and 168 registers
 //     a thread: enough for all 15 gathers of a tau = 1 node, or for a BGK
-//     node's group of four with nothing spilled.  16 slots spill and starve
-//     the L1 (BGK vortex street, 260k nodes: 31 us against 23 with 12).
+//     node's group of four with one register spilled (K = 32, eight slots: 16).
+//     16 slots spill and starve the L1 (BGK vortex street, 260k nodes: 31 us
+//     against 23 with 12).
 //   - A block takes one contiguous range of tiles (neighbouring tiles share
 //     gathers in L1); the ranges are cut to equal cost, because tiles of a
 //     regular region fetch index rows only.
