@@ -30,7 +30,7 @@ constexpr uint16_t kInfoSolid = 0x100, kInfoEq = 0x200;
 // nine cells and the wrap-around divisions, all nine populations loaded at
 // once, and the rare bounced ones fetched again from the cell itself.  Rows of
 // 64 cells by 4 fill narrow lattices too.  577,280 cells (42 MB, in L2), us a
-// step: 14.2 with the types of nine cells and a launch per step, 8.0 now.
+// step: 14.3 with the types of nine cells and a launch per step, 9.3 now.
 constexpr int kLatX = 64, kLatY = 4;
 __global__ void __launch_bounds__(kLatX * kLatY) lattice_step(int nx, int ny, const uint16_t* __restrict__ info,
                                                               const float4* __restrict__ eqv,
